@@ -322,11 +322,30 @@ int plan_flags(const Plan &P, bool only_launch) {
 }
 
 constexpr int MIN_PIECE = 8;   // default shortest row range worth a 4-row halo
-constexpr double DEFAULT_ROW_OVERHEAD = 1.0;   // fixed cost of a strip row, in busy warps
+// Fixed cost of a strip row, in quarters of a full strip's width: a row pass takes nearly
+// the same time for every width (its instructions wait on one another), so narrow last
+// strips cost almost as much as full ones.  32 uneven FP16 lattices, split plan: 232 us a
+// step with 1, 194 with 2, 171 with 4, 150 with 8.
+constexpr double DEFAULT_ROW_OVERHEAD = 8.0;
 
+
+// Shortest row range where MIN_PIECE would leave resident blocks idle.  A block's march is a
+// chain of dependent row passes, so shorter pieces on more blocks win although each loads 4
+// rows more: one 2048 x 128 FP32 lattice 23.2 us a step with 8 rows, 13.9 with 2; 1024 x 300
+// 22.5 and 13.7; from 1024 x 1024 on the blocks are full either way.
+constexpr int SHORT_PIECE = 2;
+
+// Strips of a lattice; plan_rows 0 is set by default_pieces.
 void strips_of(std::vector<StripRef> &out, int sim, int nx, int ny, int plan_rows) {
-    const int mp = plan_rows > 0 ? plan_rows : MIN_PIECE;
-    for (int x0 = 0; x0 < nx; x0 += FUSED_W) out.push_back({sim, x0, std::min(FUSED_W, nx - x0), ny, mp});
+    for (int x0 = 0; x0 < nx; x0 += FUSED_W) out.push_back({sim, x0, std::min(FUSED_W, nx - x0), ny, plan_rows});
+}
+
+void default_pieces(std::vector<StripRef> &strips, int max_blocks, bool may_shorten) {
+    long long pieces = 0;
+    for (const auto &s : strips) pieces += std::max(1, s.ny / (s.min_piece > 0 ? s.min_piece : MIN_PIECE));
+    const int rows = may_shorten && pieces < max_blocks ? SHORT_PIECE : MIN_PIECE;
+    for (auto &s : strips)
+        if (s.min_piece <= 0) s.min_piece = rows;
 }
 
 // Balanced persistent plan: the strip rows are cut into nearly equal shares
@@ -496,10 +515,21 @@ int resident_blocks(int storage, int variant) {
                      : storage == ST_F16DEV ? fused_smem<__half>(variant)
                                             : fused_smem<__nv_bfloat16>(variant);
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, FUSED_W, smem) != cudaSuccess || per < 1) per = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, FUSED_THREADS, smem) != cudaSuccess || per < 1) per = 1;
     if (sms < 1) sms = 1;
     cache[storage][variant] = sms * per;
     return cache[storage][variant];
+}
+
+// Thread blocks a plan over `nodes` nodes is made for: all resident ones (6 per SM), which
+// hides the latency of the row passes best, except on FP32 lattices far beyond L2.  Those
+// are held by DRAM, and 5 per SM load fewer halo rows: 4096 x 512 FP32 62.3 -> 57.9 us a
+// step, 8192 x 256 open 71.5 -> 66.8, 2048 x 2048 120.6 -> 113; at 1024 x 1024 (151 MB of
+// state, mostly in L2) 6 per SM are faster (29.2 against 30.1), and FP16 storage is at every
+// size (2048 x 1280: 61.8 with 6 per SM, 69 with 5).
+int plan_blocks(int storage, int variant, long long nodes) {
+    const int all = resident_blocks(storage, variant);
+    return storage == ST_F32 && nodes >= 1500000 ? std::max(1, all * 5 / 6) : all;
 }
 
 int grid_for(long long n, int threads) {
@@ -777,7 +807,9 @@ lbm_status create_common(int nx, int ny, const lbm_params *p, void *buf, size_t 
     {
         std::vector<StripRef> strips;
         strips_of(strips, 0, nx, ny, p->plan_rows);
-        Plan P = make_plan(strips, p->plan, 0, resident_blocks(p->storage, variant_of(p)), DEFAULT_ROW_OVERHEAD);
+        const int blocks = plan_blocks(p->storage, variant_of(p), (long long)nx * ny);
+        default_pieces(strips, blocks, true);
+        Plan P = make_plan(strips, p->plan, 0, blocks, DEFAULT_ROW_OVERHEAD);
         s->n_items = (int)P.items.size();
         s->n_blocks = P.blocks;
         s->launch_flags = plan_flags(P, true);
@@ -1142,6 +1174,7 @@ lbm_status lbm_plan_preview(const int *nx, const int *ny, const int *plan_rows, 
         strips_of(strips, i, nx[i], ny[i], pr);
     }
     const double ovh = opts->row_overhead < 0.0f ? DEFAULT_ROW_OVERHEAD : (double)opts->row_overhead;
+    default_pieces(strips, max_blocks, false);
     const Plan P = make_plan(strips, opts->plan, opts->rows_per_item, max_blocks, ovh);
     *n_items = (int)P.items.size();
     *n_blocks = P.blocks;
@@ -1201,12 +1234,17 @@ lbm_status lbm_batch_create_ex(lbm_sim *const *sims, int n, const lbm_batch_opts
     for (int st = 0; st < 3; st++)
         for (int cv = 0; cv < N_VARIANTS; cv++) {
             std::vector<StripRef> strips;
+            long long nodes = 0;
             for (int i = 0; i < n; i++)
-                if (sims[i]->p.storage == st && sims[i]->h.variant == cv)
+                if (sims[i]->p.storage == st && sims[i]->h.variant == cv) {
+                    nodes += (long long)sims[i]->nx * sims[i]->ny;
                     strips_of(strips, i, sims[i]->nx, sims[i]->ny,
                               opts->member_plan_rows ? opts->member_plan_rows[i] : sims[i]->p.plan_rows);
+                }
             if (strips.empty()) continue;
-            Plan P = make_plan(strips, opts->plan, rows_per_item, resident_blocks(st, cv), row_overhead);
+            const int blocks = plan_blocks(st, cv, nodes);
+            default_pieces(strips, blocks, true);
+            Plan P = make_plan(strips, opts->plan, rows_per_item, blocks, row_overhead);
             lbm_batch::Group g{st, cv, (int)items.size(), (int)offs.size(), P.blocks, plan_flags(P, true)};
             for (int &o : P.off) o += g.item0;
             items.insert(items.end(), P.items.begin(), P.items.end());

@@ -679,120 +679,270 @@ __device__ __forceinline__ float omega_eff(const Phys &p, float psi) {
     return p.omega_b;
 }
 
+// Two FP32 values in one 64-bit register pair: sm_103a adds, multiplies and fuses
+// both with one issued instruction (add / sub / mul / fma .f32x2, each half rounded
+// like the scalar operation).
+struct alignas(8) f2 {
+    float x, y;
+};
+__device__ __forceinline__ unsigned long long f2_bits(f2 a) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+    return r;
+}
+__device__ __forceinline__ f2 f2_of(unsigned long long r) {
+    f2 a;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a.x), "=f"(a.y) : "l"(r));
+    return a;
+}
+__device__ __forceinline__ f2 operator+(f2 a, f2 b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+    return f2_of(r);
+}
+__device__ __forceinline__ f2 operator-(f2 a, f2 b) {
+    unsigned long long r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+    return f2_of(r);
+}
+__device__ __forceinline__ f2 operator*(f2 a, f2 b) {
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+    return f2_of(r);
+}
+__device__ __forceinline__ f2 fmav(f2 a, f2 b, f2 c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)), "l"(f2_bits(c)));
+    return f2_of(r);
+}
+__device__ __forceinline__ float fmav(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+
+// Node code written once for one node (V = float) and for two neighbouring nodes of a
+// row (V = f2): bc<V> broadcasts a constant, each() applies a scalar function.
+template <class V> __device__ __forceinline__ V bc(float v);
+template <> __device__ __forceinline__ float bc<float>(float v) { return v; }
+template <> __device__ __forceinline__ f2 bc<f2>(float v) { return f2{v, v}; }
+template <class F> __device__ __forceinline__ float each(float a, const F &f) { return f(a); }
+template <class F> __device__ __forceinline__ f2 each(f2 a, const F &f) { return f2{f(a.x), f(a.y)}; }
+
+
+// Literal constants: operands of the scalar code, pairs in the constant bank for the paired
+// code (as immediates a pair costs two moves at each use).
+enum : int { LIT_ZERO, LIT_QUARTER, LIT_HALF, LIT_ONE, LIT_3HALVES, LIT_TWO, LIT_FOUR, LIT_SIXTH, LIT_THIRD, LIT_TWELFTH,
+             LIT_DIAG, LIT_MHALF, LIT_M5, LIT_THREE, LIT_2THIRDS, LIT_144TH, LIT_M72TH, LIT_M2, LIT_N };
+__host__ __device__ constexpr float LIT(int i) {
+    return i == LIT_QUARTER    ? 0.25f
+           : i == LIT_HALF     ? 0.5f
+           : i == LIT_ONE      ? 1.0f
+           : i == LIT_3HALVES  ? 1.5f
+           : i == LIT_TWO      ? 2.0f
+           : i == LIT_FOUR     ? 4.0f
+           : i == LIT_SIXTH    ? 1.0f / 6.0f
+           : i == LIT_THIRD    ? 1.0f / 3.0f
+           : i == LIT_TWELFTH  ? 1.0f / 12.0f
+           : i == LIT_DIAG     ? 0.25f * 0.70710678118654752f
+           : i == LIT_MHALF    ? -0.5f
+           : i == LIT_M5       ? -5.0f
+           : i == LIT_THREE    ? 3.0f
+           : i == LIT_2THIRDS  ? 2.0f / 3.0f
+           : i == LIT_144TH    ? 1.0f / 144.0f
+           : i == LIT_M72TH    ? -1.0f / 72.0f
+           : i == LIT_M2       ? -2.0f
+                               : 0.0f;
+}
+#define LBM_LIT2_(i) {LIT(i), LIT(i)}
+static __constant__ f2 c_lit[LIT_N] = {
+    LBM_LIT2_(0),  LBM_LIT2_(1),  LBM_LIT2_(2),  LBM_LIT2_(3),  LBM_LIT2_(4),  LBM_LIT2_(5),
+    LBM_LIT2_(6),  LBM_LIT2_(7),  LBM_LIT2_(8),  LBM_LIT2_(9),  LBM_LIT2_(10), LBM_LIT2_(11),
+    LBM_LIT2_(12), LBM_LIT2_(13), LBM_LIT2_(14), LBM_LIT2_(15), LBM_LIT2_(16),
+    LBM_LIT2_(17)};
+template <class V, int I>
+__device__ __forceinline__ V lit() {
+    if constexpr (sizeof(V) == 8) return c_lit[I];
+    else return LIT(I);
+}
+
+// Per-simulation constants of the node code; the paired code keeps them in shared memory.
+template <class V>
+struct Consts {
+    V phr, phb;              // phi^r_1, phi^b_1 (phi_2 is a quarter of phi_1)
+    V inv_gamma;
+    V gx, gy, hgx, hgy;      // body acceleration, and half of it
+    V a324;                  // -A / (324 omega_eff): perturbation from the gradient times 12
+    V beta, dphi, ndphi;     // +- (phi^b_1 - phi^r_1)
+    V lam;
+    V herm_r, herm_b;        // half of 3 (c_s^k)^2 - 1
+    V c7x, c7y;              // C^k_7 factors over 12
+    V q_r, q_b;
+};
+template <class V>
+__device__ __forceinline__ void fill_consts(Consts<V> &k, const Phys &p) {
+    k.phr = bc<V>(p.phi_r[1]), k.phb = bc<V>(p.phi_b[1]);
+    k.inv_gamma = bc<V>(p.inv_gamma);
+    k.gx = bc<V>(p.gx), k.gy = bc<V>(p.gy), k.hgx = bc<V>(0.5f * p.gx), k.hgy = bc<V>(0.5f * p.gy);
+    k.a324 = bc<V>(p.a_coef * (-1.0f / 324.0f));
+    k.beta = bc<V>(p.beta), k.dphi = bc<V>(p.dphi[1]), k.ndphi = bc<V>(-p.dphi[1]);
+    k.lam = bc<V>(p.mrt_lambda);
+    k.herm_r = bc<V>(0.5f * p.herm_r), k.herm_b = bc<V>(0.5f * p.herm_b);
+    k.c7x = bc<V>(p.c7x * (1.0f / 12.0f)), k.c7y = bc<V>(p.c7y * (1.0f / 12.0f));
+    k.q_r = bc<V>(p.q_r), k.q_b = bc<V>(p.q_b);
+}
+
+template <class V>
+struct PulledOf {
+    V rr, rb;
+    V e1, e2, e3, e4, e5, e6, e7, e8;   // colour-blind non-rest parts of the links
+};
+
+template <class V>
+__device__ __forceinline__ V colour_field_of(const Consts<V> &K, V rr, V rb) {
+    const V a = rr * K.inv_gamma;
+    const V n = a - rb, d = a + rb;
+    if constexpr (sizeof(V) == 8) return V{n.x / d.x, n.y / d.y};   // IEEE division: exactly +-1 in a pure phase
+    else return n / d;
+}
+
+// Momentum sum_i c_i N_i (the rest parts cancel).
+template <class V>
+__device__ __forceinline__ void momentum_of(const PulledOf<V> &P, V &jx, V &jy) {
+    const V d5 = P.e5 - P.e7, d6 = P.e6 - P.e8;
+    jx = (P.e1 - P.e3) + (d5 - d6);
+    jy = (P.e2 - P.e4) + (d5 + d6);
+}
+
+// Post-collision state of a node: stored deviations (or split-form residuals) of both
+// colours and the split form's node scalars.
+template <class V>
+struct Collided {
+    V r[8], b[8];   // directions 1 .. 8
+    V m, gx, gy;
+};
+
 // Collision (BGK or MRT, Guo forcing, Hermite source), perturbation and
-// recolouring of one pulled node.  F is the colour gradient; dQx = d_x(q u_x),
-// dQy = d_y(q u_y) with q = sum_k (1.8 alpha_k - 0.8) rho_k.  Outputs the
-// post-collision deviations dr[1..8], db[1..8] of the stored state (the colour
-// densities are unchanged by the step's collision part).
-template <int CV, bool SPLIT = false>
-__device__ __forceinline__ void collide_node(const Phys &p, const Pulled &P, float psi, float Fx, float Fy,
-                                             float dQx, float dQy, float (&dr)[9], float (&db)[9], float &o_m,
-                                             float &o_gx, float &o_gy) {
+// recolouring of pulled nodes.  Gradients come times 12, as the S2I4 stencil sums them:
+// F the colour gradient, dQx = d_x(q u_x), dQy = d_y(q u_y) with
+// q = sum_k (1.8 alpha_k - 0.8) rho_k.  The colour densities are unchanged by the
+// step's collision part.
+//
+// Everything is formed per pair of opposite directions: the parts even in c_i once,
+// the odd parts with both signs.  On the diagonals (u.c)^2 = u^2 +- 2 u_x u_y, so the
+// even parts of the equilibrium, W rho (4.5 (u.c)^2 - 1.5 u^2), and of the perturbation
+// (Eq. (eq:perturbation)), A |F| (W (F.c)^2 / F^2 - B), are with k = rho / 6 and
+// s = A / (27 |F|)
+//   a = k u_x^2 - s F_y^2,  b = k u_y^2 - s F_x^2,  c = k u_x u_y + s F_x F_y
+//   axis x: 2 a - b    axis y: 2 b - a    diagonals: (a + b) / 2 +- 3 c / 2.
+template <int CV, bool SPLIT, class V>
+__device__ __forceinline__ void collide_of(const Phys &p, const Consts<V> &K, const PulledOf<V> &P, V psi, V Fx, V Fy, V dQx, V dQy,
+                                           Collided<V> &o) {
     constexpr bool MRT = (CV & CV_MRT) != 0, HERMITE = (CV & CV_HERMITE) != 0;
-    const float rr = P.rr, rb = P.rb;
-    const float rho = rr + rb;
-    const float inv_rho = __fdividef(1.0f, rho);
-    float e[9];
-#pragma unroll
-    for (int i = 0; i < 9; i++) e[i] = P.e[i];
-    const float jx = (e[1] - e[3]) + (e[5] - e[7]) + (e[8] - e[6]);
-    const float jy = (e[2] - e[4]) + (e[5] - e[7]) + (e[6] - e[8]);
-    const float ux = jx * inv_rho + 0.5f * p.gx;
-    const float uy = jy * inv_rho + 0.5f * p.gy;
-    const float w = omega_eff(p, psi);
+    const V half = lit<V, LIT_HALF>(), quarter = lit<V, LIT_QUARTER>(), one_half = lit<V, LIT_3HALVES>();
+    const V rr = P.rr, rb = P.rb;
+    const V rho = rr + rb;
+    const V inv_rho = each(rho, [](float v) { return __fdividef(1.0f, v); });
+    const V d1 = P.e1 - P.e3, d2 = P.e2 - P.e4, d5 = P.e5 - P.e7, d6 = P.e6 - P.e8;
+    const V Jx = fmav(rho, K.hgx, d1 + (d5 - d6)), Jy = fmav(rho, K.hgy, d2 + (d5 + d6));   // rho u
+    const V ux = Jx * inv_rho, uy = Jy * inv_rho;
+    const V w = each(psi, [&](float v) { return omega_eff(p, v); });
     const bool force = (p.gx != 0.0f) || (p.gy != 0.0f);
 
-    // velocity part of the colour-blind equilibrium, sum_k N^{k(e)}_i - R_i
-    // (Eq. (eq:equilibrium) / (eq:equilibrium_hermite)), and the Guo source,
-    // formed per opposite pair (i, OPP(i)) from the part even in c_i and the
-    // part odd in c_i (c_OPP(i) = -c_i)
-    const float usq = ux * ux + uy * uy;
-    const float herm = HERMITE ? 0.5f * (rr * p.herm_r + rb * p.herm_b) : 0.0f;
-    const float Gx = rho * p.gx, Gy = rho * p.gy;
-    const float uG = ux * Gx + uy * Gy;
-    float weq[9], src[9];
-    weq[0] = WT(0) * rho * (-1.5f * usq);
-    src[0] = 0.0f;
-#pragma unroll
-    for (int i : {1, 2, 5, 6}) {
-        const int j = OPP(i);
-        const float cu = CX(i) * ux + CY(i) * uy;
-        const float even = WT(i) * rho * (4.5f * cu * cu - 1.5f * usq);
-        float odd = WT(i) * 3.0f * rho * cu;
-        if (HERMITE) odd += WT(i) * 3.0f * cu * (3.0f * C2(i) - 4.0f) * herm;
-        weq[i] = even + odd;
-        weq[j] = even - odd;
-        src[i] = src[j] = 0.0f;
-    }
-    if (force) {
-        src[0] = WT(0) * (-3.0f * uG);
-#pragma unroll
-        for (int i : {1, 2, 5, 6}) {
-            const int j = OPP(i);
-            const float cu = CX(i) * ux + CY(i) * uy;
-            const float cG = CX(i) * Gx + CY(i) * Gy;
-            const float even = WT(i) * (9.0f * cu * cG - 3.0f * uG);
-            const float odd = WT(i) * 3.0f * cG;
-            src[i] = even + odd;
-            src[j] = even - odd;
-        }
-    }
-
+    // one A/2 term per colour; zero where F is zero
+    const V Fx2 = Fx * Fx, Fy2 = Fy * Fy;
+    const V invF = each(Fx2 + Fy2, [](float v) { return v > 0.0f ? rsqrtf(v) : 0.0f; });
+    const V ns = w * invF * K.a324;   // - s for the gradient times 12
+    const V nR = ns * Fx2, nS = ns * Fy2, nC = ns * Fx * Fy;
+    // Odd part of the equilibrium, 3 W rho cu: with q = rho u / 12 (Hermite: + h u / 6) it is
+    // q_x + q_y on a diagonal and rho u_x / 2 - 2 q_x on an axis, which sums to the momentum
+    // rho u without the rounding of q.  (1/3 and 1/12 of it rounded separately drift by 3e-8
+    // of the momentum every step, in the same direction at every node of a uniform flow.)
+    V herm;
+    if (HERMITE) herm = fmav(rr, K.herm_r, rb * K.herm_b) * lit<V, LIT_SIXTH>();
+    V E1, E2, E3, E4, E5, E6, E7, E8;   // post-collision non-rest parts
     if (!MRT) {
-        const float fw = 1.0f - 0.5f * w;
-#pragma unroll
-        for (int i = 1; i < 9; i++) e[i] = e[i] - w * (e[i] - weq[i]) + fw * src[i];
-    } else {
-        float q[9];
-#pragma unroll
-        for (int i = 0; i < 9; i++) q[i] = e[i] - weq[i];
-        // moments of the non-equilibrium part and of the source, rows of M
-        // (appendix "Transformation matrices"); row 0 (mass) is zero for both.
-        const float ax = q[1] + q[2] + q[3] + q[4], dg = q[5] + q[6] + q[7] + q[8];
-        float m[9], ms[9];
-        m[1] = -4.0f * q[0] - ax + 2.0f * dg;
-        m[2] = 4.0f * q[0] - 2.0f * ax + dg;
-        m[3] = q[1] - q[3] + q[5] - q[6] - q[7] + q[8];
-        m[4] = -2.0f * (q[1] - q[3]) + q[5] - q[6] - q[7] + q[8];
-        m[5] = q[2] - q[4] + q[5] + q[6] - q[7] - q[8];
-        m[6] = -2.0f * (q[2] - q[4]) + q[5] + q[6] - q[7] - q[8];
-        m[7] = q[1] - q[2] + q[3] - q[4];
-        m[8] = q[5] - q[6] + q[7] - q[8];
-        const float sx = src[1] + src[2] + src[3] + src[4], sd = src[5] + src[6] + src[7] + src[8];
-        ms[1] = -4.0f * src[0] - sx + 2.0f * sd;
-        ms[2] = 4.0f * src[0] - 2.0f * sx + sd;
-        ms[3] = src[1] - src[3] + src[5] - src[6] - src[7] + src[8];
-        ms[4] = -2.0f * (src[1] - src[3]) + src[5] - src[6] - src[7] + src[8];
-        ms[5] = src[2] - src[4] + src[5] + src[6] - src[7] - src[8];
-        ms[6] = -2.0f * (src[2] - src[4]) + src[5] + src[6] - src[7] - src[8];
-        ms[7] = src[1] - src[2] + src[3] - src[4];
-        ms[8] = src[5] - src[6] + src[7] - src[8];
-        const float s1 = p.mrt_lambda * w;   // s_0 .. s_6
-        float tm[9];
-#pragma unroll
-        for (int a = 1; a < 9; a++) {
-            const float sa = a < 7 ? s1 : w;  // s_7 = s_8 = omega_eff
-            tm[a] = sa * m[a] - (1.0f - 0.5f * sa) * ms[a];
+        // e + w (e_eq - e) + (1 - w/2) source + perturbation
+        const V Wx = w * Jx, Wy = w * Jy;
+        V qx = Wx * lit<V, LIT_TWELFTH>(), qy = Wy * lit<V, LIT_TWELFTH>();
+        const V kx = qx + qx, ky = qy + qy;
+        V a = fmav(kx, ux, nS), b = fmav(ky, uy, nR), c = kx * uy - nC;
+        if (HERMITE) {
+            const V hw = herm * w;
+            qx = fmav(hw, ux, qx);
+            qy = fmav(hw, uy, qy);
         }
+        V o1 = fmav(lit<V, LIT_M2>(), qx, half * Wx), o2 = fmav(lit<V, LIT_M2>(), qy, half * Wy);
+        V o5 = qx + qy, o6 = qy - qx;
+        if (force) {
+            // Guo source with f = (1 - w/2) rho g / 3: even 9 W cu cG - 3 W uG (the same shape
+            // as the equilibrium with u_x f_x, u_y f_y and the mixed product), odd 3 W cG
+            const V f = fmav(lit<V, LIT_MHALF>(), w, lit<V, LIT_ONE>()) * rho * lit<V, LIT_THIRD>();
+            const V gx = f * K.gx, gy = f * K.gy;
+            a = fmav(ux, gx, a);
+            b = fmav(uy, gy, b);
+            c = fmav(half, fmav(ux, gy, uy * gx), c);
+            o1 = o1 + gx;
+            o2 = o2 + gy;
+            o5 = fmav(quarter, gx + gy, o5);
+            o6 = fmav(quarter, gy - gx, o6);
+        }
+        const V g = lit<V, LIT_ONE>() - w;
+        const V vX = (a - b) + a, vY = (b - a) + b, vD = half * (a + b), vC = one_half * c;
+        const V v5 = vD + vC, v6 = vD - vC;
+        E1 = fmav(P.e1, g, vX + o1), E3 = fmav(P.e3, g, vX - o1);
+        E2 = fmav(P.e2, g, vY + o2), E4 = fmav(P.e4, g, vY - o2);
+        E5 = fmav(P.e5, g, v5 + o5), E7 = fmav(P.e7, g, v5 - o5);
+        E6 = fmav(P.e6, g, v6 + o6), E8 = fmav(P.e8, g, v6 - o6);
+    } else {
+        // M^-1 S M of the appendix written per pair.  With q = e - e_eq and the mass
+        // row zero, the energy rows relax the pair sums of q by s_1 (their axis
+        // and diagonal totals), rows 7 and 8 their differences by omega_eff, and
+        // the flux rows every odd part by s_1 (s_1 = .. = s_6 = lambda omega_eff).
+        const V s1 = w * K.lam;
+        const V f1 = fmav(lit<V, LIT_MHALF>(), s1, lit<V, LIT_ONE>()), fw = fmav(lit<V, LIT_MHALF>(), w, lit<V, LIT_ONE>());
+        V qx = Jx * lit<V, LIT_TWELFTH>(), qy = Jy * lit<V, LIT_TWELFTH>();
+        const V kx = qx * lit<V, LIT_FOUR>(), ky = qy * lit<V, LIT_FOUR>();   // twice the even parts of the equilibrium
+        const V a = kx * ux, b = ky * uy, c = one_half * (kx * uy), vD = half * (a + b);
+        const V qX = (P.e1 + P.e3) - ((a - b) + a), qY = (P.e2 + P.e4) - ((b - a) + b);
+        const V q5 = (P.e5 + P.e7) - (vD + c), q6 = (P.e6 + P.e8) - (vD - c);
+        if (HERMITE) {
+            qx = fmav(herm, ux, qx);
+            qy = fmav(herm, uy, qy);
+        }
+        const V hs = s1 * half;
+        V O1 = hs * fmav(lit<V, LIT_FOUR>(), qx, d1 - Jx), O2 = hs * fmav(lit<V, LIT_FOUR>(), qy, d2 - Jy);
+        V O5 = hs * fmav(lit<V, LIT_M2>(), qx + qy, d5), O6 = hs * fmav(lit<V, LIT_M2>(), qy - qx, d6);
+        V ax = s1 * (qX + qY), dg = s1 * (q5 + q6), t7 = w * (qX - qY), t8 = w * (q5 - q6);
+        if (force) {
+            // twice the even parts of the source, W (9 cu cG - 3 uG)
+            const V g3 = rho * lit<V, LIT_2THIRDS>();
+            const V gx = g3 * K.gx, gy = g3 * K.gy;
+            const V bx = ux * gx, by = uy * gy;
+            ax = ax - f1 * (bx + by);
+            t7 = t7 - fw * lit<V, LIT_THREE>() * (bx - by);
+            dg = dg - f1 * (bx + by);
+            t8 = t8 - fw * one_half * fmav(ux, gy, uy * gx);
+            const V h1 = f1 * half, h2 = h1 * quarter;
+            O1 = O1 - h1 * gx;
+            O2 = O2 - h1 * gy;
+            O5 = O5 - h2 * (gx + gy);
+            O6 = O6 - h2 * (gy - gx);
+        }
+        V gA = ax * quarter, gB = dg * quarter;
         if (HERMITE) {
             // + U = M^-1 C, C_1 = 3 (1 - s_1/2)(dQx + dQy), C_7 = (1 - w/2)(dQx - dQy)
             // (C_7's factor and sign from the Chapman-Enskog expansion: the p_xx
             // moment carries d_xQ_x - d_yQ_y of the third-moment error)
-            tm[1] -= 3.0f * (1.0f - 0.5f * s1) * (dQx + dQy);
-            tm[7] -= (1.0f - 0.5f * w) * (p.c7x * dQx + p.c7y * dQy);
+            const V c1 = f1 * (dQx + dQy);
+            gA = fmav(lit<V, LIT_144TH>(), c1, gA);
+            gB = fmav(lit<V, LIT_M72TH>(), c1, gB);
+            t7 = t7 - fw * fmav(dQx, K.c7x, dQy * K.c7y);
         }
-        // e -= M^-1 tm, M^-1 = (1/36) * integer matrix of the appendix (tm[0] = 0)
-        const float k36 = 1.0f / 36.0f;
-        const float b12 = -tm[1] - 2.0f * tm[2];
-        const float d21 = 2.0f * tm[1] + tm[2];
-        e[1] -= k36 * (b12 + 6.0f * tm[3] - 6.0f * tm[4] + 9.0f * tm[7]);
-        e[2] -= k36 * (b12 + 6.0f * tm[5] - 6.0f * tm[6] - 9.0f * tm[7]);
-        e[3] -= k36 * (b12 - 6.0f * tm[3] + 6.0f * tm[4] + 9.0f * tm[7]);
-        e[4] -= k36 * (b12 - 6.0f * tm[5] + 6.0f * tm[6] - 9.0f * tm[7]);
-        e[5] -= k36 * (d21 + 6.0f * tm[3] + 3.0f * tm[4] + 6.0f * tm[5] + 3.0f * tm[6] + 9.0f * tm[8]);
-        e[6] -= k36 * (d21 - 6.0f * tm[3] - 3.0f * tm[4] + 6.0f * tm[5] + 3.0f * tm[6] - 9.0f * tm[8]);
-        e[7] -= k36 * (d21 - 6.0f * tm[3] - 3.0f * tm[4] - 6.0f * tm[5] - 3.0f * tm[6] + 9.0f * tm[8]);
-        e[8] -= k36 * (d21 + 6.0f * tm[3] + 3.0f * tm[4] - 6.0f * tm[5] - 3.0f * tm[6] - 9.0f * tm[8]);
+        const V h7 = t7 * quarter, h8 = t8 * quarter;
+        const V pD = half * (nR + nS), pC = one_half * nC;
+        const V nX = ((nS - nR) + nS) - (gA + h7), nY = ((nR - nS) + nR) - (gA - h7);
+        const V n5 = (pD - pC) - (gB + h8), n6 = (pD + pC) - (gB - h8);
+        E1 = P.e1 + (nX - O1), E3 = P.e3 + (nX + O1);
+        E2 = P.e2 + (nY - O2), E4 = P.e4 + (nY + O2);
+        E5 = P.e5 + (n5 - O5), E7 = P.e7 + (n5 + O5);
+        E6 = P.e6 + (n6 - O6), E8 = P.e8 + (n6 + O6);
     }
 
     // Eq. (eq:recoloringOperator) written for the stored deviations:
@@ -801,72 +951,59 @@ __device__ __forceinline__ void collide_node(const Phys &p, const Pulled &P, flo
     // with E_i the post-collision non-rest part and term_i the recolouring flux.
     // Each colour is formed from its own density, as in the paper, so a colour
     // that is absent stays exactly zero (no rounding-level phantom colour).
-    const float fr = rr * inv_rho, fb = rb * inv_rho;
-    const float mix = rr * rb * inv_rho;
-    const float F2 = Fx * Fx + Fy * Fy;
-    o_m = mix;
-    o_gx = o_gy = 0.0f;
-    // per |c|^2 class: shift of the stored deviations
-    const float sh1 = mix * (p.phi_b[1] - p.phi_r[1]), sh2 = mix * (p.phi_b[2] - p.phi_r[2]);
-    if (F2 > 0.0f) {
-        // Eq. (eq:perturbation), one A/2 term per colour: A |F| [W (F.c)^2/|F|^2 - B]
-        // (even in c_i), and the recolouring flux (odd in c_i)
-        const float invFn = rsqrtf(F2);
-        const float Fn = F2 * invFn;
-        const float A = p.a_coef * w;
-        const float pa = A * invFn, pb = A * Fn;
-        const float kk = p.beta * mix * inv_rho * invFn;   // beta rr rb / rho^2 / |F|
-        if (SPLIT) {
-            // only the residuals (rho_k / rho) E_i are stored; the shift and the
-            // recolouring flux are rebuilt from m and G = kk F (split_shift)
-            o_gx = kk * Fx;
-            o_gy = kk * Fy;
-#pragma unroll
-            for (int i : {1, 2, 5, 6}) {
-                const int j = OPP(i);
-                const float Fc = CX(i) * Fx + CY(i) * Fy;
-                const float pert = pa * WT(i) * Fc * Fc - pb * BP(i);
-                const float Ei = e[i] + pert, Ej = e[j] + pert;
-                dr[i] = fr * Ei;
-                dr[j] = fr * Ej;
-                db[i] = fb * Ei;
-                db[j] = fb * Ej;
-            }
-            dr[0] = db[0] = 0.0f;
-            return;
-        }
-        // cos(phi_i) = c_i.F / (|c_i| |F|); rest_i = rr phi^r_i + rb phi^b_i
-        const float k1 = kk * (rr * p.phi_r[1] + rb * p.phi_b[1]);
-        const float k2 = kk * 0.70710678118654752f * (rr * p.phi_r[2] + rb * p.phi_b[2]);
-#pragma unroll
-        for (int i : {1, 2, 5, 6}) {
-            const int j = OPP(i);
-            const float Fc = CX(i) * Fx + CY(i) * Fy;
-            const float pert = pa * WT(i) * Fc * Fc - pb * BP(i);
-            const float term = (C2(i) == 1 ? k1 : k2) * Fc;
-            const float sh = C2(i) == 1 ? sh1 : sh2;
-            const float Ei = e[i] + pert, Ej = e[j] + pert;
-            dr[i] = sh + fr * Ei + term;
-            dr[j] = sh + fr * Ej - term;
-            db[i] = -sh + fb * Ei - term;
-            db[j] = -sh + fb * Ej + term;
-        }
-    } else if (SPLIT) {
-#pragma unroll
-        for (int i = 1; i < 9; i++) {
-            dr[i] = fr * e[i];
-            db[i] = fb * e[i];
-        }
+    const V fr = rr * inv_rho, fb = rb * inv_rho;
+    const V mix = rr * fb;
+    const V kk = mix * inv_rho * invF * K.beta;   // beta rr rb / rho^2 / |F|
+    const V Gx = kk * Fx, Gy = kk * Fy;
+    o.m = mix;
+    o.gx = Gx;
+    o.gy = Gy;
+    if (SPLIT) {
+        // only the residuals (rho_k / rho) E_i are stored; the shift and the
+        // recolouring flux are rebuilt from m and G (split_shift)
+        o.r[0] = fr * E1, o.r[1] = fr * E2, o.r[2] = fr * E3, o.r[3] = fr * E4;
+        o.r[4] = fr * E5, o.r[5] = fr * E6, o.r[6] = fr * E7, o.r[7] = fr * E8;
+        o.b[0] = fb * E1, o.b[1] = fb * E2, o.b[2] = fb * E3, o.b[3] = fb * E4;
+        o.b[4] = fb * E5, o.b[5] = fb * E6, o.b[6] = fb * E7, o.b[7] = fb * E8;
     } else {
-#pragma unroll
-        for (int i = 1; i < 9; i++) {
-            const float sh = C2(i) == 1 ? sh1 : sh2;
-            dr[i] = sh + fr * e[i];
-            db[i] = -sh + fb * e[i];
-        }
+        // shift of the deviations by |c|^2, and the flux (odd in c_i):
+        // cos(phi_i) = c_i.F / (|c_i| |F|), rest_i = rr phi^r_i + rb phi^b_i; phi_2 = phi_1 / 4
+        const V sA = mix * K.dphi, nA = mix * K.ndphi;
+        const V sB = sA * quarter, nB = nA * quarter;
+        const V rest = fmav(rr, K.phr, rb * K.phb);
+        const V tx = Gx * rest, ty = Gy * rest;
+        const V D = lit<V, LIT_DIAG>();
+        const V t5 = D * (tx + ty), t6 = D * (ty - tx);
+        o.r[0] = fmav(fr, E1, sA + tx), o.b[0] = fmav(fb, E1, nA - tx);
+        o.r[1] = fmav(fr, E2, sA + ty), o.b[1] = fmav(fb, E2, nA - ty);
+        o.r[2] = fmav(fr, E3, sA - tx), o.b[2] = fmav(fb, E3, nA + tx);
+        o.r[3] = fmav(fr, E4, sA - ty), o.b[3] = fmav(fb, E4, nA + ty);
+        o.r[4] = fmav(fr, E5, sB + t5), o.b[4] = fmav(fb, E5, nB - t5);
+        o.r[5] = fmav(fr, E6, sB + t6), o.b[5] = fmav(fb, E6, nB - t6);
+        o.r[6] = fmav(fr, E7, sB - t5), o.b[6] = fmav(fb, E7, nB + t5);
+        o.r[7] = fmav(fr, E8, sB - t6), o.b[7] = fmav(fb, E8, nB + t6);
     }
-    dr[0] = 0.0f;
-    db[0] = 0.0f;
+}
+
+// One node, in the form the node-parallel kernels use.
+template <int CV, bool SPLIT = false>
+__device__ __forceinline__ void collide_node(const Phys &p, const Pulled &P, float psi, float Fx, float Fy,
+                                             float dQx, float dQy, float (&dr)[9], float (&db)[9], float &o_m,
+                                             float &o_gx, float &o_gy) {
+    const PulledOf<float> q{P.rr, P.rb, P.e[1], P.e[2], P.e[3], P.e[4], P.e[5], P.e[6], P.e[7], P.e[8]};
+    Collided<float> o;
+    Consts<float> K;
+    fill_consts(K, p);
+    collide_of<CV, SPLIT, float>(p, K, q, psi, 12.0f * Fx, 12.0f * Fy, 12.0f * dQx, 12.0f * dQy, o);
+    dr[0] = db[0] = 0.0f;
+#pragma unroll
+    for (int i = 1; i < 9; i++) {
+        dr[i] = o.r[i - 1];
+        db[i] = o.b[i - 1];
+    }
+    o_m = o.m;
+    o_gx = o.gx;
+    o_gy = o.gy;
 }
 
 // --------------------------------------------------------------- PTX helpers
@@ -933,15 +1070,6 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *tm, ui
         "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
         " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(dst)),
         "l"(tm), "r"(c0), "r"(c1), "r"(smem_u32(bar))
-        : "memory");
-}
-
-// 3D tiled TMA load of one box into shared memory, completion on `bar`.
-__device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *tm, uint64_t *bar, int c0, int c1, int c2) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
-        "l"(tm), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar))
         : "memory");
 }
 

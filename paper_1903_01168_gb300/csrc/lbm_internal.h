@@ -17,12 +17,16 @@ void host_fill_desc(SimDesc &h, int nx, int ny, const lbm_params *p, void *state
 // Message returned by lbm_last_error(NULL) on this thread.
 void host_set_global_error(const char *msg);
 
-// Launch shape of the fused kernel: columns per strip (= threads per block)
-// and shared-memory row slots per block.
+// Launch shape of the fused kernel: columns per strip (two per thread) and
+// shared-memory row slots per block.  Each row is read in one pass, so two slots already
+// load the next row during a pass; a third one measured no faster (FP32 sweep 80.3 us a
+// step with 2, 82.5 with 3) and takes open lattices from 6 blocks per SM to 5 (8192 x 256:
+// 81.8 and 90.7).
 #ifndef LBM_FUSED_NSLOT
-#define LBM_FUSED_NSLOT 4
+#define LBM_FUSED_NSLOT 2
 #endif
 constexpr int FUSED_W = 128;
+constexpr int FUSED_THREADS = FUSED_W / 2;
 constexpr int FUSED_NSLOT = LBM_FUSED_NSLOT;
 
 // Launchers of the step kernels.  Each (storage type T, variant CV) pair of the

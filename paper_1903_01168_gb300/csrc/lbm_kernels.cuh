@@ -31,42 +31,40 @@ constexpr long long WAIT_LIMIT_CYCLES = 4000000000LL;   // ~2 s at 2 GHz
 #ifndef LBM_FUSED_PDL
 #define LBM_FUSED_PDL 1
 #endif
-// March direction of the fused steps: 0 every step up, 1 consecutive steps in
-// opposite directions, 2 every step down.
-#ifndef LBM_FUSED_ALTERNATE
-#define LBM_FUSED_ALTERNATE 0
-#endif
-
 // ------------------------------------------------------------------ loaders
 
-// Stored values from global memory; ys is wrapped periodically.
+// Stored values from global memory around one row: pulls of nodes of row y read rows y - 1,
+// y and y + 1 (wrapped periodically when the loader is made).  Three row pointers and 32-bit
+// plane offsets: one address instruction per load.
 template <typename T>
-struct GlobalLoader {
-    const float *rho0;   // &rho[b][0][0][0] (interior column 0)
-    const T *dev0;       // &dev[b][0][0][0]
-    long long rho_plane, dev_plane, rho_row, dev_row;
-    int ny;
+struct RowLoader {
+    const float *rho_m, *rho_c, *rho_p;   // plane 0, interior column 0, of rows y - 1, y, y + 1
+    const T *dev_m, *dev_c, *dev_p;
+    int rho_plane, dev_plane, y;
     int slip;   // free-slip walls
     SplitC q;
-    __device__ __forceinline__ GlobalLoader(const SimDesc &d, int b) {
-        rho0 = d.rho + b * d.rho_buf + d.ghost;
-        dev0 = reinterpret_cast<const T *>(d.dev) + b * d.dev_buf + d.ghost;
-        rho_plane = d.rho_plane;
-        dev_plane = d.dev_plane;
-        rho_row = d.rho_row;
-        dev_row = d.dev_row;
-        ny = d.ph.ny;
+    __device__ __forceinline__ RowLoader(const SimDesc &d, int b, int row) {
+        const int ny = d.ph.ny;
+        auto wrap = [&](int ys) { return ys < 0 ? ys + ny : (ys >= ny ? ys - ny : ys); };
+        const float *r = d.rho + b * d.rho_buf + d.ghost;
+        const T *v = reinterpret_cast<const T *>(d.dev) + b * d.dev_buf + d.ghost;
+        rho_m = r + wrap(row - 1) * d.rho_row, rho_c = r + wrap(row) * d.rho_row, rho_p = r + wrap(row + 1) * d.rho_row;
+        dev_m = v + wrap(row - 1) * d.dev_row, dev_c = v + wrap(row) * d.dev_row, dev_p = v + wrap(row + 1) * d.dev_row;
+        rho_plane = (int)d.rho_plane;
+        dev_plane = (int)d.dev_plane;
+        y = row;
         slip = d.wet.slip;
         q = split_consts(d.ph);
     }
-    __device__ __forceinline__ int wrap(int ys) const { return ys < 0 ? ys + ny : (ys >= ny ? ys - ny : ys); }
     __device__ __forceinline__ float rho(int k, int xs, int ys) const {
-        return rho0[k * rho_plane + (long long)wrap(ys) * rho_row + xs];
+        const int dy = ys - y;
+        return (dy < 0 ? rho_m : (dy == 0 ? rho_c : rho_p))[k * rho_plane + xs];
     }
     static constexpr bool SPLIT = SplitStore<T>::value;
     // stored value r^k_i of node (xs, ys): the deviation itself, or the split-form residual
     __device__ __forceinline__ float res(int k, int i, int xs, int ys) const {
-        return Codec<T>::dec(dev0[(k * 8 + i - 1) * dev_plane + (long long)wrap(ys) * dev_row + xs]);
+        const int dy = ys - y;
+        return Codec<T>::dec((dy < 0 ? dev_m : (dy == 0 ? dev_c : dev_p))[(k * 8 + i - 1) * dev_plane + xs]);
     }
     // split-form shift h_i of node (xs, ys) (0 without the split form)
     __device__ __forceinline__ float shift(int i, int xs, int ys) const {
@@ -83,45 +81,6 @@ struct GlobalLoader {
         const float sh = shift(i, xs, ys);
         return k == 0 ? __fadd_rn(r, sh) : __fsub_rn(r, sh);
     }
-};
-
-// Stored values from the shared-memory row ring (rows y-1, y, y+1 of a strip
-// starting at column x0).  A slot holds [NS][BOXW] floats (padded to RHO_BYTES)
-// then [16][BOXW] T.
-template <typename T, int BOXW, int G, int RHO_BYTES>
-struct SmemLoader {
-    const unsigned char *r0, *r1, *r2;
-    int y, x0;
-    SplitC q;
-    int slip;   // free-slip walls (read only by the wetting variants' links)
-    __device__ __forceinline__ const unsigned char *row(int ys) const {
-        const int dy = ys - y;
-        return dy < 0 ? r0 : (dy == 0 ? r1 : r2);
-    }
-    __device__ __forceinline__ float rho(int k, int xs, int ys) const {
-        return reinterpret_cast<const float *>(row(ys))[k * BOXW + (xs - x0 + G)];
-    }
-    static constexpr bool SPLIT = SplitStore<T>::value;
-    __device__ __forceinline__ float res(int k, int i, int xs, int ys) const {
-        const T *p = reinterpret_cast<const T *>(row(ys) + RHO_BYTES);
-        return Codec<T>::dec(p[(k * 8 + i - 1) * BOXW + (xs - x0 + G)]);
-    }
-    __device__ __forceinline__ float shift(int i, int xs, int ys) const {
-        if (!SPLIT) return 0.0f;
-        return split_shift(q, i, rho(0, xs, ys), rho(1, xs, ys), rho(2, xs, ys), rho(3, xs, ys), rho(4, xs, ys));
-    }
-    __device__ __forceinline__ float own_shift_sum(int xs, int ys) const {
-        return SPLIT ? 4.0f * rho(2, xs, ys) * (q.dph1 + q.dph2) : 0.0f;
-    }
-    __device__ __forceinline__ float dev(int k, int i, int xs, int ys) const {
-        const float r = res(k, i, xs, ys);
-        if (!SPLIT) return r;
-        const float sh = shift(i, xs, ys);
-        return k == 0 ? __fadd_rn(r, sh) : __fsub_rn(r, sh);
-    }
-    // same, for direction indices known only at run time
-    __device__ __forceinline__ float rho_rt(int k, int xs, int ys) const { return rho(k, xs, ys); }
-    __device__ __forceinline__ float dev_rt(int k, int i, int xs, int ys) const { return dev(k, i, xs, ys); }
 };
 
 // psi on a solid wall row: W-weighted mean of the in-domain fluid nodes next
@@ -153,41 +112,12 @@ __device__ __forceinline__ void s2i4(const V &v, float &gx, float &gy) {
     gy = (1.0f / 3.0f) * (n - s) + (1.0f / 12.0f) * (a - b);
 }
 
-// Colour densities of one pulled node computed by 16 lanes of a warp: lane
-// j = 8 k + (i - 1) adds colour k's direction-i term of
-//   rho_k' = rho_k(x) + sum_{i>=1} [phi^k_i (s^k_i - rho_k(x)) + delta^k_i - d^k_i(x)]
-// and the two colour sums are reduced with shuffles inside the 16-lane group.
-// No wall link may touch the node (callers use the serial pull next to walls).
-template <class Loader>
-__device__ __forceinline__ void pull_rho_coop16(const Phys &p, const Loader &ld, int x, int y, int j, float &rr,
-                                                float &rb) {
-    const int k = j >> 3, i = (j & 7) + 1;
-    const int cx = (i == 1 || i == 5 || i == 8) ? 1 : ((i == 3 || i == 6 || i == 7) ? -1 : 0);
-    const int cy = (i == 2 || i == 5 || i == 6) ? 1 : ((i == 4 || i == 7 || i == 8) ? -1 : 0);
-    const int c2 = cx * cx + cy * cy;
-    const float ph = k == 0 ? (c2 == 1 ? p.phi_r[1] : p.phi_r[2]) : (c2 == 1 ? p.phi_b[1] : p.phi_b[2]);
-    const float own = ld.rho_rt(k, x, y);
-    float v;
-    if (Loader::SPLIT) {
-        // split form: residual difference plus the source's shift; the node's own
-        // shifts sum to 4 m (dphi_1 + dphi_2), taken off once after the reduction
-        const float sg = k == 0 ? 1.0f : -1.0f;
-        v = ph * (ld.rho_rt(k, x - cx, y - cy) - own) + (ld.res(k, i, x - cx, y - cy) - ld.res(k, i, x, y)) +
-            sg * ld.shift(i, x - cx, y - cy);
-    } else {
-        v = ph * (ld.rho_rt(k, x - cx, y - cy) - own) + (ld.dev_rt(k, i, x - cx, y - cy) - ld.dev_rt(k, i, x, y));
-    }
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    v += __shfl_xor_sync(0xffffffffu, v, 2);
-    v += __shfl_xor_sync(0xffffffffu, v, 4);
-    if (Loader::SPLIT) v -= (k == 0 ? 1.0f : -1.0f) * ld.own_shift_sum(x, y);
-    const float mine = own + v;                        // colour k's new density
-    const float other = __shfl_xor_sync(0xffffffffu, mine, 8);
-    rr = k == 0 ? mine : other;
-    rb = k == 0 ? other : mine;
-}
-
 // ------------------------------------------------------------ fused kernel
+
+// Rows of open-column values computed at a time, and the values kept of such a node (two
+// densities, eight non-rest parts).
+constexpr int OPEN_ROWS = 32;
+constexpr int OPEN_VALUES = 10;
 
 template <typename T, int CV, int W, int NSLOT>
 struct FusedCfg {
@@ -198,67 +128,215 @@ struct FusedCfg {
     static constexpr int RHO_BYTES = ((NS * BOXW * 4 + 127) / 128) * 128;
     static constexpr int DEV_BYTES = 16 * BOXW * (int)sizeof(T);
     static constexpr int SLOT_BYTES = ((RHO_BYTES + DEV_BYTES + 127) / 128) * 128;
-    static constexpr int RING = W + 2;                       // ring width (columns x0-1 .. x0+W)
+    static constexpr int RING = W + 4;                       // columns x0-2 .. x0+W+1
     static constexpr bool QRING = (CV & CV_MRT) && (CV & CV_HERMITE);
     static constexpr bool WET = (CV & CV_WET) != 0;
-    static constexpr int LINKS = WET ? LINKS_ALL : LINKS_NOSLIP;
-    // shared rings (floats) of what neighbouring threads read: psi and q u over
-    // rows y-1..y+1.  Stage A of row y+1 may run while slower threads still do
-    // stage B of row y-1, so they hold 4 rows.  The node's own rho_r, rho_b and
-    // e_1..8 stay in the registers of the thread that pulled them.
-    static constexpr int PSI_OFF = 0;
-    static constexpr int QX_OFF = PSI_OFF + 4 * RING;
-    static constexpr int QY_OFF = QX_OFF + (QRING ? 4 * RING : 0);
-    static constexpr int RING_FLOATS = QY_OFF + (QRING ? 4 * RING : 0);
+    // shared floats: rings of what neighbouring threads read, psi and q u of the newest
+    // row and the one before (a slower thread may still read that one); psi of the lower
+    // wall; the edge lanes' values of the last four rows (two columns a side next to
+    // walls); the paired constants; open columns of two chunks of rows
+    static constexpr int QX_OFF = 3 * RING;
+    static constexpr int QY_OFF = QX_OFF + (QRING ? 2 * RING : 0);
+    static constexpr int HIST_OFF = ((QY_OFF + (QRING ? 2 * RING : 0)) + 3) / 4 * 4;
+    static constexpr int CONST_OFF = HIST_OFF + 2 * 4 * 32 * 4;
+    static constexpr int OPEN_OFF = CONST_OFF + (int)sizeof(Consts<f2>) / 4;
+    static constexpr int RING_FLOATS = OPEN_OFF + ((CV & CV_OPEN) ? 4 * OPEN_ROWS * OPEN_VALUES : 0);
     static constexpr int DESC_BYTES = ((int)sizeof(SimDesc) + 127) / 128 * 128;
     static constexpr int RING_BYTES = ((RING_FLOATS * 4 + 15) / 16) * 16;
     static constexpr int SMEM = DESC_BYTES + NSLOT * SLOT_BYTES + RING_BYTES + NSLOT * 8 + 16;
     static constexpr uint32_t TX_BYTES = (uint32_t)(NS * BOXW * 4 + DEV_BYTES);
-    // Blocks per SM the registers are sized for: 5 (96 registers) for FP32, 6 (80)
-    // for 16-bit storage, whose smaller rows let 6 blocks share the SM's shared
-    // memory; 4 (128) for MRT + Hermite, whose source term needs them, and for
-    // wetting walls (free-slip links, contact-angle adjustment).  Measured
-    // on the 40-lattice sweep: 4 -> 5 blocks +2.5 % (FP32), 4 -> 6 +7 % (FP16).
-    static constexpr int MINB = LBM_FUSED_MIN_BLOCKS > 0 ? LBM_FUSED_MIN_BLOCKS
-                                : ((QRING || WET) ? 4 : (sizeof(T) == 4 ? 5 : 6));
+    // Blocks per SM the registers are sized for: 6 blocks of 2 warps are 3 warps on each
+    // scheduler, 168 registers a thread, which holds both columns' state without spills in
+    // the loop (spilled variants were 1.5-2x slower: their local memory misses the small L1
+    // that the shared-memory carve-out leaves).  Measured on the 40-lattice sweep with 4 and 6
+    // blocks: BF16 76.9 and 63.8 us a step, FP32 74.3 and 81.4 (the plans of large FP32
+    // lattices use 5, see plan_blocks).
+    static constexpr int MINB = LBM_FUSED_MIN_BLOCKS > 0 ? LBM_FUSED_MIN_BLOCKS : 6;
     static_assert(BOXW <= 256, "TMA box dimension limit");
     static_assert((BOXW * sizeof(T)) % 16 == 0 && (BOXW * 4) % 16 == 0, "TMA inner box bytes");
     static_assert(G <= GMEM && G >= 3, "halo must cover the stencil and fit the memory ghost");
-    static_assert(NSLOT >= 4, "the prologue waits for rows ya-2 .. ya+1 before any slot is refilled");
+    static_assert(NSLOT >= 2, "one row is read while the next ones arrive");
+    static_assert(W / 2 >= 2 * OPEN_ROWS, "one thread per side and row of a chunk");
 };
+
+// Two neighbouring columns' values of one shared-memory row: `at` points at the first.
+template <typename T>
+__device__ __forceinline__ f2 pair_at(const T *at);
+template <>
+__device__ __forceinline__ f2 pair_at<float>(const float *at) {
+    const float2 v = *reinterpret_cast<const float2 *>(at);
+    return f2{v.x, v.y};
+}
+template <>
+__device__ __forceinline__ f2 pair_at<__half>(const __half *at) {
+    const float2 v = __half22float2(*reinterpret_cast<const __half2 *>(at));
+    return f2{v.x, v.y};
+}
+template <>
+__device__ __forceinline__ f2 pair_at<__nv_bfloat16>(const __nv_bfloat16 *at) {
+    const float2 v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(at));
+    return f2{v.x, v.y};
+}
+__device__ __forceinline__ void pair_to(float *at, f2 v) { *reinterpret_cast<float2 *>(at) = make_float2(v.x, v.y); }
+__device__ __forceinline__ void pair_to(__half *at, f2 v) {
+    *reinterpret_cast<__half2 *>(at) = __floats2half2_rn(v.x, v.y);
+}
+__device__ __forceinline__ void pair_to(__nv_bfloat16 *at, f2 v) {
+    *reinterpret_cast<__nv_bfloat162 *>(at) = __floats2bfloat162_rn(v.x, v.y);
+}
+
+// What one stored row r adds, in the two columns of one thread, to the nodes of rows
+// r + 1 (links 2, 5, 6), r (links 1, 3, less the node's own deviations) and r - 1
+// (links 4, 7, 8).  u^k_i = phi^k_i (rho_k(source) - rho_k(x, r)) + d^k_i(source) is
+// taken relative to the column's own density in row r, so that every term is a
+// small difference; moving the reference to the node's own row later costs one
+// density difference per row.  T_i = u^r_i + u^b_i.  h_*: sums of the split-form shifts
+// of the same links (16-bit storage).
+struct RowTerms {
+    f2 own[2];                    // densities of (x, r)
+    f2 up[2], mid[2], dn[2];      // per colour: sums of u over the links into rows r + 1, r, r - 1
+    f2 T1, T2, T3, T4, T5, T6, T7, T8;
+    f2 h_up, h_mid, h_dn;
+};
+
+// `slot`: the row in shared memory; `col`: the first of the thread's columns in it.  Each
+// stored value of a row is read in this one pass only.
+template <typename T, int BOXW, int RHO_BYTES>
+__device__ __forceinline__ RowTerms row_terms(const unsigned char *slot, int col, const Consts<f2> &K) {
+    const float *rp = reinterpret_cast<const float *>(slot) + col;
+    const T *dp = reinterpret_cast<const T *>(slot + RHO_BYTES) + col;
+    const f2 quarter = lit<f2, LIT_QUARTER>();
+    RowTerms R;
+    f2 west[2], east[2];
+    auto half = [&](int k, f2 &T1, f2 &T2, f2 &T3, f2 &T4, f2 &T5, f2 &T6, f2 &T7, f2 &T8) {
+        const f2 own = pair_at(rp + k * BOXW);
+        west[k] = f2{rp[k * BOXW - 1], own.x};
+        east[k] = f2{own.y, rp[k * BOXW + 2]};
+        R.own[k] = own;
+        const f2 phi1 = k == 0 ? K.phr : K.phb;   // phi_2 = phi_1 / 4
+        const f2 pW = phi1 * (west[k] - own), pE = phi1 * (east[k] - own);
+        const T *d = dp + (8 * k - 1) * BOXW;   // direction i at d + i * BOXW
+        auto at = [&](int i, int dx) { return Codec<T>::dec(d[i * BOXW + dx]); };
+        const f2 o1 = pair_at(d + 1 * BOXW), o3 = pair_at(d + 3 * BOXW);
+        T1 = pW + f2{at(1, -1), o1.x};
+        T3 = pE + f2{o3.y, at(3, 2)};
+        f2 out = o1 + o3;
+        R.mid[k] = T1 + T3;
+        const f2 o5 = pair_at(d + 5 * BOXW), o6 = pair_at(d + 6 * BOXW);
+        T5 = fmav(quarter, pW, f2{at(5, -1), o5.x});
+        T6 = fmav(quarter, pE, f2{o6.y, at(6, 2)});
+        out = out + (o5 + o6);
+        T2 = pair_at(d + 2 * BOXW);
+        T4 = pair_at(d + 4 * BOXW);
+        out = out + (T2 + T4);
+        R.up[k] = T2 + (T5 + T6);
+        const f2 o7 = pair_at(d + 7 * BOXW), o8 = pair_at(d + 8 * BOXW);
+        T8 = fmav(quarter, pW, f2{at(8, -1), o8.x});
+        T7 = fmav(quarter, pE, f2{o7.y, at(7, 2)});
+        out = out + (o7 + o8);
+        R.dn[k] = T4 + (T7 + T8);
+        R.mid[k] = R.mid[k] - out;
+    };
+    f2 b1, b2, b3, b4, b5, b6, b7, b8;
+    half(0, R.T1, R.T2, R.T3, R.T4, R.T5, R.T6, R.T7, R.T8);
+    half(1, b1, b2, b3, b4, b5, b6, b7, b8);
+    R.T1 = R.T1 + b1, R.T2 = R.T2 + b2, R.T3 = R.T3 + b3, R.T4 = R.T4 + b4;
+    R.T5 = R.T5 + b5, R.T6 = R.T6 + b6, R.T7 = R.T7 + b7, R.T8 = R.T8 + b8;
+    R.h_up = R.h_mid = R.h_dn = lit<f2, LIT_ZERO>();
+    if (SplitStore<T>::value) {
+        // the shift of direction i is m dphi_c + (c_i . G) / |c_i| rest_c, rest_c = rho_r phi^r_c
+        // + rho_b phi^b_c; phi_2 = phi_1 / 4 for both colours.  The node's own eight shifts sum
+        // to 4 m (dphi_1 + dphi_2) = 5 m dphi_1.
+        const f2 pr = K.phr, pb = K.phb, dph = K.dphi;
+        const f2 rW = fmav(pr, west[0], pb * west[1]), rE = fmav(pr, east[0], pb * east[1]);
+        const f2 rC = fmav(pr, R.own[0], pb * R.own[1]);
+        const float *mp = rp + 2 * BOXW, *xp = rp + 3 * BOXW, *yp = rp + 4 * BOXW;
+        const f2 mC = pair_at(mp), xC = pair_at(xp), yC = pair_at(yp);
+        const f2 a = mC * dph, b = yC * rC;
+        const f2 aWE = (f2{mp[-1], mC.x} + f2{mC.y, mp[2]}) * dph;
+        const f2 xWE = f2{xp[-1], xC.x} * rW - f2{xC.y, xp[2]} * rE;
+        const f2 yWE = fmav(f2{yp[-1], yC.x}, rW, f2{yC.y, yp[2]} * rE);
+        const f2 D = lit<f2, LIT_DIAG>();
+        const f2 even = fmav(D, xWE, fmav(quarter, aWE, a)), odd = fmav(D, yWE, b);
+        R.h_up = even + odd;
+        R.h_dn = even - odd;
+        R.h_mid = fmav(lit<f2, LIT_M5>(), a, aWE + xWE);
+    }
+    return R;
+}
+
+// The nodes (x, r) of a thread between the passes over their own row and over row r + 1:
+// sums over the links from rows r - 1 and r, and the T_i of those links (relative to the
+// nodes' own densities).
+struct HalfPulled {
+    f2 own[2], acc[2];
+    f2 T1, T2, T3, T5, T6, h;
+};
+
+// Close the nodes (x, r): add the links from row r + 1 (dn, T4, T7, T8, h_dn) and form the
+// new densities and the colour-blind non-rest parts.  sr, sb: phi_1 times the density step
+// from (x, r) to (x, r + 1) (zero at a wall): it moves the reference of the links from
+// row r + 1, once on the axis and a quarter on each diagonal, 1.5 in the sum.
+template <bool SPLIT>
+__device__ __forceinline__ void close_node(const Consts<f2> &K, const HalfPulled &H, f2 dn0, f2 dn1, f2 T4, f2 T7, f2 T8,
+                                           f2 h_dn, f2 sr, f2 sb, PulledOf<f2> &P) {
+    const f2 c15 = lit<f2, LIT_3HALVES>(), quarter = lit<f2, LIT_QUARTER>();
+    f2 ar = fmav(c15, sr, H.acc[0] + dn0);
+    f2 ab = fmav(c15, sb, H.acc[1] + dn1);
+    if (SPLIT) {
+        const f2 h = H.h + h_dn;
+        ar = ar + h;
+        ab = ab - h;
+    }
+    P.rr = H.own[0] + ar;
+    P.rb = H.own[1] + ab;
+    // rest part of the density change on the axis links
+    const f2 R1 = fmav(K.phr, P.rr - H.own[0], K.phb * (P.rb - H.own[1]));
+    const f2 up = (sr + sb) - R1, R4 = quarter * R1, up4 = quarter * up;
+    P.e1 = H.T1 - R1;
+    P.e2 = H.T2 - R1;
+    P.e3 = H.T3 - R1;
+    P.e4 = T4 + up;
+    P.e5 = H.T5 - R4;
+    P.e6 = H.T6 - R4;
+    P.e7 = T7 + up4;
+    P.e8 = T8 + up4;
+}
 
 // Persistent fused step.  Block b processes the work items
 // items[item_off[b] .. item_off[b+1]) in order (strip segments, possibly of
 // different simulations), so that every block gets an equal share of rows.
 //
-// Per segment the block marches up rows ya .. yb-1 of a strip of w <= W
-// columns.  Source rows arrive by TMA into a ring of NSLOT shared slots.
-// Iteration y first pulls row y+1 (stage A: new colour densities, colour field
-// and the colour-blind non-rest parts e_i of every node of that row; the colour
-// field also one column each side), then collides row y (stage B) from the
-// densities and e_i that the same thread pulled one iteration earlier (kept in
-// registers) and the colour field of rows y-1..y+1 in a shared ring (S2I4
-// gradient).  Stage B reads no source row, so a row's slot is refilled as soon
-// as stage A of the row above has used it.  One block runs 4 warps; 5 or 6
-// blocks share an SM (FusedCfg::MINB).
+// Per segment the block marches up a strip of w <= W columns, one thread per two
+// neighbouring columns: the arithmetic of both is issued as f32x2 instructions, stored
+// values move as pairs, and loop, address and barrier work is shared.
+// Source rows arrive by TMA into a ring of NSLOT shared slots.  The pass over row r
+//   - reads row r once (the node's own densities and deviations and those entering from
+//     the two sides) and splits it into what it adds to the nodes of rows r + 1, r and
+//     r - 1 (RowTerms), kept in registers;
+//   - closes the nodes of row r - 1 and shares their colour field through a ring;
+//   - collides the nodes of row r - 2, whose gradient now has its three rows, and
+//     stores them.
+// A row's slot is free after its one pass, so NSLOT - 1 rows are in flight.
 //
-// DIR = +1 marches up (rows ya .. yb-1), DIR = -1 down (yb-1 .. ya); every node
-// is computed the same way in both.  Consecutive steps march in opposite
-// directions, so that a step starts on the rows the previous one wrote last,
-// while they are still in L2.
-template <typename T, int CV, int W, int NSLOT, int DIR>
-__global__ void __launch_bounds__(W, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_step_fused(const SimDesc *__restrict__ descs,
-                                                     const WorkItem *__restrict__ items,
-                                                     const int *__restrict__ item_off, int n_blocks,
-                                                     int step_offset, int flags, int *__restrict__ err) {
-    static_assert(DIR == 1 || DIR == -1, "march direction");
+// Bound by the latency of its own instructions: a warp issues once in about six cycles
+// (fixed-latency and shared-memory dependencies), so the time goes with instructions per
+// node and with warps in flight, and FP32 also with DRAM (5.5 TB/s of halo, state and ghost
+// traffic).  Instructions issued per node of the 40-lattice sweep, one column a thread with
+// scalar arithmetic and separate pulls of three rows (before): FP32 681, BF16 973; now FP32
+// 400, BF16 488.  Microseconds a step before and now: sweep BF16 107.6 and 65.6, FP32 78.9
+// and 79.4; eight open channels of mixed storage 293 and 174.
+template <typename T, int CV, int W, int NSLOT>
+__global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_step_fused(
+    const SimDesc *__restrict__ descs, const WorkItem *__restrict__ items, const int *__restrict__ item_off,
+    int n_blocks, int step_offset, int flags, int *__restrict__ err) {
     using Cfg = FusedCfg<T, CV, W, NSLOT>;
-    constexpr int G = Cfg::G, BOXW = Cfg::BOXW, RING = Cfg::RING;
+    constexpr int G = Cfg::G, BOXW = Cfg::BOXW, RING = Cfg::RING, NT = W / 2;
     constexpr bool HERMITE = (CV & CV_HERMITE) != 0;
     constexpr bool HERMITE_SRC = Cfg::QRING;
     constexpr bool WET = Cfg::WET;
     constexpr bool OPEN = (CV & CV_OPEN) != 0;
-    constexpr int LINKS = Cfg::LINKS;
+    constexpr bool SPLIT = SplitStore<T>::value;
     extern __shared__ __align__(128) unsigned char smem[];
 
     // Launched as a programmatic dependent of the previous step: this block
@@ -277,17 +355,14 @@ __global__ void __launch_bounds__(W, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_step_f
     SimDesc &d = *reinterpret_cast<SimDesc *>(smem);
     unsigned char *slots = smem + Cfg::DESC_BYTES;
     float *rings = reinterpret_cast<float *>(slots + NSLOT * Cfg::SLOT_BYTES);
-    float *ring_psi = rings + Cfg::PSI_OFF;
-    float *ring_qx = rings + Cfg::QX_OFF;
-    float *ring_qy = rings + Cfg::QY_OFF;
+    Consts<f2> &K = *reinterpret_cast<Consts<f2> *>(rings + Cfg::CONST_OFF);
+    float *opens = rings + Cfg::OPEN_OFF;
     uint64_t *bars = reinterpret_cast<uint64_t *>(reinterpret_cast<unsigned char *>(rings) + Cfg::RING_BYTES);
-    volatile int &s_bad = *reinterpret_cast<volatile int *>(bars + NSLOT);
 
     if (smem_u32(slots) & 127) {   // TMA destinations must be 128-byte aligned
         if (tid == 0) atomicOr(err, ERR_ALIGN);
         return;
     }
-    if (tid == 0) s_bad = 0;
 
     const int it_end = item_off[blockIdx.x + 1];
     for (int itx = item_off[blockIdx.x]; itx < it_end; ++itx) {
@@ -297,7 +372,7 @@ __global__ void __launch_bounds__(W, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_step_f
         {
             const int4 *src = reinterpret_cast<const int4 *>(gd);
             int4 *dst = reinterpret_cast<int4 *>(smem);
-            for (int j = tid; j < (int)(sizeof(SimDesc) / 16); j += W) dst[j] = src[j];
+            for (int j = tid; j < (int)(sizeof(SimDesc) / 16); j += NT) dst[j] = src[j];
         }
         if (tid == 0) {
             for (int s = 0; s < NSLOT; s++) {
@@ -310,251 +385,419 @@ __global__ void __launch_bounds__(W, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_step_f
             tensormap_acquire(&gd->tmap_dev);
         }
         __syncthreads();
+        if (tid == NT - 1) fill_consts(K, d.ph);
 
-        const Phys p = d.ph;   // per-simulation constants, in registers from here on
-        const SplitC qs = split_consts(p);
+        const Phys &p = d.ph;   // per-simulation constants, in shared memory
         const long long t = d.t0 + step_offset;
         if (t >= d.t_end) continue;   // this simulation has stopped
         const int bsrc = (int)(t & 1), bdst = bsrc ^ 1;
-        const int nx = p.nx, ny = p.ny;
-        const bool wall_y = p.bc_y == BC_WALL;
         const int x0 = it.x0, w = it.w, ya = it.ya, yb = it.yb;
-        if (d.variant != CV || d.ghost != Cfg::GMEM || w <= 0 || w > W || x0 < 0 || x0 + w > nx || (x0 % 8) != 0 ||
-            ya < 0 || yb > ny || ya >= yb) {
+        if (d.variant != CV || d.ghost != Cfg::GMEM || w <= 0 || w > W || x0 < 0 || x0 + w > p.nx || (x0 % 8) != 0 ||
+            ya < 0 || yb > p.ny || ya >= yb) {
             if (tid == 0) atomicOr(err, ERR_BADITEM);
             continue;
         }
-        const int row_first = ya - 2, row_last = yb + 1, n_rows = row_last - row_first + 1;
-        // march index of source row r: the order in which rows are loaded
-        auto mi = [&](int r) { return DIR > 0 ? r - row_first : row_last - r; };
-        auto row_at = [&](int m) { return DIR > 0 ? row_first + m : row_last - m; };
+        const bool wall_y = p.bc_y == BC_WALL;
+        // source rows r0 .. r_load - 1 are loaded (none lies behind a wall)
+        const int r0 = wall_y ? max(ya - 2, 0) : ya - 2;
+        const int r_load = wall_y ? min(yb + 2, p.ny) : yb + 2;
 
-        auto row_valid = [&](int r) { return !wall_y || (r >= 0 && r < ny); };
-        auto slot_of = [&](int r) { return mi(r) % NSLOT; };
-        auto parity_of = [&](int r) { return (uint32_t)((mi(r) / NSLOT) & 1); };
-        auto row_ptr = [&](int r) { return slots + slot_of(r) * Cfg::SLOT_BYTES; };
-        // Load source row r (both colour densities and all 16 deviation planes,
-        // columns x0-G .. x0+W+G-1) into its slot.  A row behind a wall is not
-        // loaded, but its slot barrier still completes one phase (plain arrival)
-        // so that every slot's phase parity stays (use count) & 1.
-        auto issue = [&](int r) {
-            const int s = slot_of(r);
-            if (!row_valid(r)) {
-                mbar_arrive(&bars[s]);
-                return;
-            }
-            const int yr = r < 0 ? r + ny : (r >= ny ? r - ny : r);
+        // Load source row r (densities and all 16 deviation planes, columns
+        // x0-G .. x0+W+G-1) into slot s.
+        auto issue = [&](int r, int s) {
+            const int yr = r < 0 ? r + p.ny : (r >= p.ny ? r - p.ny : r);
             unsigned char *dst = slots + s * Cfg::SLOT_BYTES;
             const int xb = x0 + (Cfg::GMEM - G);   // element index of column x0 - G in the padded row
             mbar_arrive_expect_tx(&bars[s], Cfg::TX_BYTES);
-            const int brow = bsrc * ny + yr;   // row index over both buffers
+            const int brow = bsrc * p.ny + yr;   // row index over both buffers
             tma_load_2d(dst, &gd->tmap_rho, &bars[s], xb, brow * Cfg::NS);
             tma_load_2d(dst + Cfg::RHO_BYTES, &gd->tmap_dev, &bars[s], xb, brow * 16);
         };
-        int next_m = 0;   // march index of the next row to load; meaningful on thread 0 only
         if (tid == 0) {
-            for (; next_m < n_rows && next_m < NSLOT; ++next_m) issue(row_at(next_m));
+            for (int m = 0; m < NSLOT && r0 + m < r_load; ++m) issue(r0 + m, m);
         }
 
-        bool ok = true;
-        auto wait_row = [&](int r) {
-            if (ok && mi(r) < n_rows && row_valid(r)) {
-                if (!mbar_wait_bounded(&bars[slot_of(r)], parity_of(r), WAIT_LIMIT_CYCLES)) {
-                    ok = false;
-                    s_bad = 1;
-                }
+        bool ok = true;   // a thread that gave up waiting does not wait again
+        const int tc = 2 * tid, x = x0 + tc;            // the thread's first column
+        const bool active = tc < w, both = tc + 1 < w;
+        const bool last = tid == (w - 1) / 2;            // has the strip's last column
+        const bool open_l = OPEN && x0 == 0, open_r = OPEN && x0 + w == p.nx;
+        // the outlet column is the first or second one beyond the strip
+        const bool open_next = OPEN && x0 + w == p.nx - 1, open_next2 = OPEN && x0 + w == p.nx - 2;
+        __syncthreads();   // the constants are in place
+
+        // store pointers of the row collided next
+        char *out_rho = reinterpret_cast<char *>(d.rho + bdst * d.rho_buf + (long long)ya * d.rho_row + d.ghost + x);
+        char *out_dev = reinterpret_cast<char *>(reinterpret_cast<T *>(d.dev) + bdst * d.dev_buf +
+                                                 (long long)ya * d.dev_row + d.ghost + x);
+
+        const f2 zero{0.0f, 0.0f};
+        HalfPulled H;        // nodes (x, r - 1) at the start of pass r
+        f2 lo0 = zero, lo1 = zero, lo2 = zero, lo5 = zero, lo6 = zero, lo_h = zero;   // row r - 1's terms for row r
+        PulledOf<f2> Pc, Pn; // pulled state of rows r - 2 and r - 1
+        H.own[0] = H.own[1] = H.acc[0] = H.acc[1] = zero;
+        H.T1 = H.T2 = H.T3 = H.T5 = H.T6 = H.h = zero;
+        Pn.rr = Pn.rb = Pn.e1 = Pn.e2 = Pn.e3 = Pn.e4 = Pn.e5 = Pn.e6 = Pn.e7 = Pn.e8 = zero;
+        // colour field of rows r - 3 (s) and r - 2 (c): the thread's columns, the column west
+        // of them and the one east; q u: the x difference of q u_x, and q u_y
+        f2 sC = zero, cC = zero, sX = zero, cX = zero, qsC = zero, qcC = zero;
+        float sW = 0.0f, sE = 0.0f, cW = 0.0f, cE = 0.0f, qsW = 0.0f, qsE = 0.0f, qcW = 0.0f, qcE = 0.0f;
+
+        // terms of a no-slip wall for the row next to it, from that row's own deviations:
+        // the opposite directions i, j, k of the links out of the wall (an axis, two
+        // diagonals); sgn: the wall's side in y
+        auto wall_terms = [&](const unsigned char *sp, int i, int j, int k, float sgn, f2 &sum_r, f2 &sum_b, f2 &Ti, f2 &Tj,
+                              f2 &Tk, f2 &h) {
+            const float *rp = reinterpret_cast<const float *>(sp) + tc + G;
+            const T *dp = reinterpret_cast<const T *>(sp + Cfg::RHO_BYTES) + tc + G;
+            auto at = [&](int plane) { return pair_at(dp + plane * BOXW); };
+            const f2 ri = at(i - 1), rj = at(j - 1), rk = at(k - 1), bi = at(i + 7), bj = at(j + 7), bk = at(k + 7);
+            sum_r = ri + (rj + rk);
+            sum_b = bi + (bj + bk);
+            Ti = ri + bi;
+            Tj = rj + bj;
+            Tk = rk + bk;
+            if (SPLIT) {
+                const f2 rest = fmav(K.phr, pair_at(rp), K.phb * pair_at(rp + BOXW));
+                h = fmav(bc<f2>(1.5f * p.dphi[1]), pair_at(rp + 2 * BOXW),
+                         bc<f2>(sgn * (1.0f + 0.5f * 0.70710678118654752f)) * (pair_at(rp + 4 * BOXW) * rest));
             }
         };
-        auto loader = [&](int y) {
-            SmemLoader<T, BOXW, G, Cfg::RHO_BYTES> L;
-            L.r0 = row_ptr(y - 1);
-            L.r1 = row_ptr(y);
-            L.r2 = row_ptr(y + 1);
-            L.y = y;
-            L.x0 = x0;
-            L.q = qs;
-            L.slip = WET ? d.wet.slip : 0;
-            return L;
-        };
-
-        auto rs_of = [&](int Y) { return ((Y + 4) & 3) * RING; };   // ring row of lattice row Y
-        // ring column c (0 or w+1) of row Y by one thread's full pull (next to
-        // walls and open columns, or where the node also needs q u)
-        auto edge_full = [&](const auto &L, int Y, int c) {
-            int X = x0 - 1 + c;
-            if (p.bc_x == BC_INOUT) X = X < 0 ? 0 : (X >= nx ? nx - 1 : X);
-            Pulled P;
-            pull_node_rows<HERMITE, LINKS>(p, L, X, Y, t, false, 0.0f, 0.0f, P);
-            ring_psi[rs_of(Y) + c] = colour_field(p, P.rr, P.rb);
-            if (HERMITE_SRC) {
-                const NodeMoments m = node_moments(p, P);
-                const float q = p.q_r * m.rr + p.q_b * m.rb;
-                ring_qx[rs_of(Y) + c] = q * m.ux;
-                ring_qy[rs_of(Y) + c] = q * m.uy;
-            }
-        };
-
-        // stage A: ring row Y, columns x0-1 .. x0+w
-        auto stageA = [&](int Y, Pulled &out) {
-            const int rs = rs_of(Y);
-            if (wall_y && (Y < 0 || Y >= ny)) {
-                const int Yn = Y < 0 ? 0 : ny - 1;
-                const auto L = loader(Yn);
-                for (int c = tid; c < w + 2; c += W) {
-                    const int X = x0 - 1 + c;
-                    const float ps = wall_psi(p, X, [&](int Xp) {
-                        float rr, rb, jx, jy;
-                        pull_moments_rows<HERMITE, false, LINKS>(p, L, Xp, Yn, t, rr, rb, jx, jy);
-                        return colour_field(p, rr, rb);
-                    });
-                    ring_psi[rs + c] = ps;
-                    if (HERMITE_SRC) {
-                        ring_qx[rs + c] = 0.0f;
-                        ring_qy[rs + c] = 0.0f;
-                    }
-                }
-            } else {
-                const auto L = loader(Y);
-                // interior ring columns x0 .. x0+w-1: one node per thread, full pull
-                if (tid < w) {
-                    const int c = tid + 1;
-                    const int X = x0 + tid;
+        int slot = 0;
+        uint32_t phase = 0;
+#pragma unroll 1
+        for (int r = r0; r < yb + 2; ++r) {
+            const int Y = r - 1;                          // row whose nodes this pass closes
+            const bool closes = r >= ya && (Y >= 0 || !wall_y);
+            const bool wall_row = wall_y && Y >= p.ny;    // Y is the wall above
+            const bool by_wall = wall_y && (Y == 0 || Y >= p.ny - 1);
+            if (OPEN && (open_l || open_r || open_next || open_next2) && r >= ya && ((r - ya) & (OPEN_ROWS - 1)) == 0) {
+                // open columns of rows Y .. Y + OPEN_ROWS - 1 by the general pull with the Zou-He
+                // values, one node per thread; row Y's are at slot (Y - ya + 1) mod 2 OPEN_ROWS
+                const int side = tid / OPEN_ROWS, Yo = Y + tid % OPEN_ROWS;
+                if (side < 2 && (side == 0 ? open_l : open_r || open_next || open_next2) && Yo <= yb && !(wall_y && (Yo < 0 || Yo >= p.ny))) {
+                    const RowLoader<T> L(d, bsrc, Yo);
                     Pulled P;
-                    pull_node_rows<HERMITE, LINKS>(p, L, X, Y, t, false, 0.0f, 0.0f, P);
-                    ring_psi[rs + c] = colour_field(p, P.rr, P.rb);
-                    out = P;
-                    if (HERMITE_SRC) {
-                        const NodeMoments m = node_moments(p, P);
-                        const float q = p.q_r * m.rr + p.q_b * m.rb;
-                        ring_qx[rs + c] = q * m.ux;
-                        ring_qy[rs + c] = q * m.uy;
-                    }
-                }
-                // the two edge columns x0-1 and x0+w only need psi (and q u): the
-                // last warp computes them 16 lanes per node, unless a boundary
-                // touches them (wall row) or the node needs q u
-                const int Ye = Y < 0 ? Y + ny : (Y >= ny ? Y - ny : Y);
-                const bool wall_row = wall_y && (Ye == 0 || Ye == ny - 1);
-                if constexpr (!OPEN) {
-                    // bc_x is always periodic here (the variant says so); the
-                    // run-time test stays because without it the compiler lays
-                    // out this loop 0.9 % slower on the periodic sweep (measured)
-                    if (p.bc_x != BC_PERIODIC) {
-                    } else if (!HERMITE_SRC && !wall_row) {
-                        if (tid >= W - 32) {
-                            const int lane = tid & 31, e = lane >> 4;
-                            const int X = e == 0 ? x0 - 1 : x0 + w;
-                            float rr, rb;
-                            pull_rho_coop16(p, L, X, Y, lane & 15, rr, rb);
-                            if ((lane & 15) == 0) ring_psi[rs + (e == 0 ? 0 : w + 1)] = colour_field(p, rr, rb);
-                        }
-                    } else if (tid < 2) {
-                        edge_full(L, Y, tid == 0 ? 0 : w + 1);
-                    }
-                } else {
-                    // open lattice: a side beyond the inlet (x = -1) or the outlet
-                    // (x = nx) takes the values of the open column itself (zero
-                    // gradient, the pull clamps X there), copied by the thread that
-                    // wrote that column; the edge next to an open column (x = 0 or
-                    // nx - 1, whose pull is the Zou-He one) is pulled in full
-                    const bool open_l = x0 == 0, open_r = x0 + w == nx;
-                    const int cc = (open_l && tid == 0) ? 0 : ((open_r && tid == w - 1) ? w + 1 : -1);
-                    if (cc >= 0) {
-                        ring_psi[rs + cc] = ring_psi[rs + tid + 1];
-                        if (HERMITE_SRC) {
-                            ring_qx[rs + cc] = ring_qx[rs + tid + 1];
-                            ring_qy[rs + cc] = ring_qy[rs + tid + 1];
-                        }
-                    }
-                    const bool plain_l = !open_l && x0 - 1 >= 1, plain_r = !open_r && x0 + w <= nx - 2;
-                    if (!HERMITE_SRC && !wall_row && (plain_l || plain_r)) {
-                        if (tid >= W - 32) {
-                            // all 32 lanes take part (full-warp shuffles); a side
-                            // that is not plain pulls column x0 and discards it
-                            const int lane = tid & 31, e = lane >> 4;
-                            const bool plain = e == 0 ? plain_l : plain_r;
-                            const int X = plain ? (e == 0 ? x0 - 1 : x0 + w) : x0;
-                            float rr, rb;
-                            pull_rho_coop16(p, L, X, Y, lane & 15, rr, rb);
-                            if ((lane & 15) == 0 && plain) ring_psi[rs + (e == 0 ? 0 : w + 1)] = colour_field(p, rr, rb);
-                        }
-                    }
-                    const bool full_l = !open_l && (HERMITE_SRC || wall_row || !plain_l);
-                    const bool full_r = !open_r && (HERMITE_SRC || wall_row || !plain_r);
-                    if ((tid == 0 && full_l) || (tid == 1 && full_r)) edge_full(L, Y, tid == 0 ? 0 : w + 1);
-                }
-            }
-        };
-
-        // stage B: collide row y from the rings
-        auto stageB = [&](int y, const Pulled &Pin) {
-            if (tid >= w) return;
-            const int x = x0 + tid;
-            const int rm = ((y + 3) & 3) * RING, r0 = ((y + 4) & 3) * RING, rp = ((y + 5) & 3) * RING;
-            const int c = tid + 1;
-            Pulled P = Pin;
-            float e0 = 0.0f;
+                    pull_node<HERMITE>(p, L, side == 0 ? 0 : p.nx - 1, Yo, t, false, 0.0f, 0.0f, P);
+                    float *o = opens + (side * 2 * OPEN_ROWS + ((Yo - ya + 1) & (2 * OPEN_ROWS - 1))) * OPEN_VALUES;
+                    o[0] = P.rr;
+                    o[1] = P.rb;
 #pragma unroll
-            for (int i = 1; i < 9; i++) e0 += P.e[i];
-            P.e[0] = -e0;
-            auto ring = [&](const float *f) {
-                return [=](int dx, int dy) { return f[(dy < 0 ? rm : (dy == 0 ? r0 : rp)) + c + dx]; };
-            };
-            float Fx, Fy, dQx = 0.0f, dQy = 0.0f;
-            s2i4(ring(ring_psi), Fx, Fy);
-            if (WET) contact_angle_adjust(d.wet, p, y, Fx, Fy);
-            if (HERMITE_SRC) {
-                float gx_, gy_;
-                s2i4(ring(ring_qx), dQx, gy_);
-                s2i4(ring(ring_qy), gx_, dQy);
+                    for (int i = 1; i < 9; i++) o[i + 1] = P.e[i];
+                }
+                __syncthreads();
             }
-            float dr[9], db[9];
-            float sm, sgx, sgy;
-            collide_node<CV, SplitStore<T>::value>(p, P, ring_psi[r0 + c], Fx, Fy, dQx, dQy, dr, db, sm, sgx, sgy);
-            NodeStore<T>(d, p, bdst, x, y).put(P.rr, P.rb, dr, db, sm, sgx, sgy);
-        };
-
-        // prologue: ring rows y0 and y0 - DIR, y0 the first row collided
-        const int y0 = DIR > 0 ? ya : yb - 1;
-        wait_row(y0 - 1);
-        wait_row(y0);
-        wait_row(y0 + 1);
-        Pulled Pc, Pn;   // pulled state of this thread's node in rows y and y + DIR
-        stageA(y0, Pc);
-        wait_row(y0 - 2 * DIR);
-        stageA(y0 - DIR, Pn);
-        __syncthreads();   // rows behind y0 are no longer read: refill their slots
-        if (tid == 0) {
-            for (; next_m < n_rows && next_m <= mi(y0 - DIR) + NSLOT; ++next_m) issue(row_at(next_m));
-        }
-
-        for (int k = 0; k < yb - ya; ++k) {
-            const int y = y0 + DIR * k;
-            wait_row(y + 2 * DIR);
-            stageA(y + DIR, Pn);
-            __syncthreads();
-            if (s_bad) break;
-            if (tid == 0) {
-                // row y and those behind it are no longer read (stage A(y + DIR)
-                // was their last reader)
-                for (; next_m < n_rows && next_m <= mi(y) + NSLOT; ++next_m) issue(row_at(next_m));
-            }
-            stageB(y, Pc);
             Pc = Pn;
+            float *ring_psi = rings + (Y & 1) * RING + 2, *ring_qx = ring_psi + Cfg::QX_OFF, *ring_qy = ring_psi + Cfg::QY_OFF;
+            if (r < r_load) {
+                if (ok && !mbar_wait_bounded(&bars[slot], phase, WAIT_LIMIT_CYCLES)) ok = false;
+                const unsigned char *sp = slots + slot * Cfg::SLOT_BYTES;
+                if (active) {
+                    const RowTerms R = row_terms<T, BOXW, Cfg::RHO_BYTES>(sp, tc + G, K);
+                    f2 sr = K.phr * (R.own[0] - H.own[0]), sb = K.phb * (R.own[1] - H.own[1]);
+                    if (closes) close_node<SPLIT>(K, H, R.dn[0], R.dn[1], R.T4, R.T7, R.T8, R.h_dn, sr, sb, Pn);
+                    if (wall_y && r == 0) {
+                        // links from behind the lower wall: the node's own opposite
+                        // populations (no slip), or those of its row travelling on
+                        // mirrored (free slip)
+                        sr = sb = zero;
+                        if (WET && d.wet.slip) {
+                            lo0 = R.dn[0], lo1 = R.dn[1];
+                            lo2 = R.T4, lo5 = R.T8, lo6 = R.T7, lo_h = R.h_dn;
+                        } else {
+                            wall_terms(sp, 4, 7, 8, -1.0f, lo0, lo1, lo2, lo5, lo6, lo_h);
+                        }
+                    }
+                    const f2 z = sr + sb, z4 = z * lit<f2, LIT_QUARTER>(), c15 = lit<f2, LIT_3HALVES>();
+                    H.own[0] = R.own[0], H.own[1] = R.own[1];
+                    H.acc[0] = (R.mid[0] + lo0) - c15 * sr;
+                    H.acc[1] = (R.mid[1] + lo1) - c15 * sb;
+                    H.T1 = R.T1;
+                    H.T3 = R.T3;
+                    H.T2 = lo2 - z;
+                    H.T5 = lo5 - z4;
+                    H.T6 = lo6 - z4;
+                    if (SPLIT) H.h = lo_h + R.h_mid;
+                    lo0 = R.up[0], lo1 = R.up[1];
+                    lo2 = R.T2, lo5 = R.T5, lo6 = R.T6;
+                    if (SPLIT) lo_h = R.h_up;
+                }
+            } else if (active && !wall_row) {
+                // the row above is the upper wall (r == ny, row ny - 1 still in its slot)
+                f2 dn0 = lo0, dn1 = lo1, T4 = lo2, T7 = lo6, T8 = lo5, h_dn = lo_h;
+                if (!(WET && d.wet.slip))
+                    wall_terms(slots + ((p.ny - 1 - r0) % NSLOT) * Cfg::SLOT_BYTES, 2, 5, 6, 1.0f, dn0, dn1, T4, T7, T8, h_dn);
+                close_node<SPLIT>(K, H, dn0, dn1, T4, T7, T8, h_dn, zero, zero, Pn);
+            }
+            // The columns beside the strip, x0 - 1 and x0 + w, need psi (and q u) only.  The last
+            // warp computes them, 16 lanes per side, lane j = 8 k + (i - 1) for colour k's
+            // direction i: each adds its link's u of the edge node of row Y from the row that the
+            // link's source is in (the values of the rows before are kept in shared memory; a
+            // link from behind a wall stands for the missing row), and the sums are reduced with
+            // shuffles.  Next to a wall the columns one further out are computed as well (outer):
+            // psi of the wall row needs them.
+            if (tid >= NT - 32 && !wall_row) {
+                const int lane = tid & 31, side = lane >> 4, k = (lane >> 3) & 1, i = (lane & 7) + 1;
+                const int cx = (i == 1 || i == 5 || i == 8) ? 1 : ((i == 3 || i == 6 || i == 7) ? -1 : 0);
+                const int cy = (i == 2 || i == 5 || i == 6) ? 1 : ((i == 4 || i == 7 || i == 8) ? -1 : 0);
+                const bool axis = i <= 4;
+                const float phi = (k == 0 ? p.phi_r[1] : p.phi_b[1]) * (axis ? 1.0f : 0.25f);
+                const bool near = wall_y && (r <= 1 || r >= p.ny - 2);
+                for (int outer = 0; outer <= (near ? 1 : 0); outer++) {
+                    const int at = side == 0 ? -1 - outer : w + outer, col = G + at;
+                    // density and decoded deviation of direction (dx, dy), plane j, at slot column q
+                    auto value = [&](const unsigned char *row, int q, int j, int dx, int dy, float &s, float &dv) {
+                        const float *rp = reinterpret_cast<const float *>(row) + q;
+                        s = rp[k * BOXW];
+                        dv = Codec<T>::dec(reinterpret_cast<const T *>(row + Cfg::RHO_BYTES)[(k * 8 + j - 1) * BOXW + q]);
+                        if (SPLIT) {
+                            const float rest = fmav(p.phi_r[1], rp[0], p.phi_b[1] * rp[BOXW]) * (axis ? 1.0f : 0.25f);
+                            const float gc = (float)dx * rp[3 * BOXW] + (float)dy * rp[4 * BOXW];
+                            const float h = (axis ? p.dphi[1] : p.dphi[2]) * rp[2 * BOXW] +
+                                            (axis ? 1.0f : 0.70710678118654752f) * gc * rest;
+                            dv += k == 0 ? h : -h;
+                        }
+                    };
+                    // source across a wall next to `row`: the node itself in the opposite direction, or
+                    // (free slip) the row's neighbour in the mirrored one
+                    auto across = [&](const unsigned char *row, float4 &v) {
+                        const bool slip = WET && d.wet.slip;
+                        const int opp = i <= 4 ? ((i + 1) & 3) + 1 : ((i - 3) & 3) + 5;
+                        const int mir = i == 2 ? 4 : i == 4 ? 2 : i == 5 ? 8 : i == 8 ? 5 : i == 6 ? 7 : i == 7 ? 6 : i;
+                        value(row, slip ? col - cx : col, slip ? mir : opp, slip ? cx : -cx, -cy, v.x, v.y);
+                    };
+                    float4 *hist = reinterpret_cast<float4 *>(rings + Cfg::HIST_OFF) + outer * 128 + lane;
+                    float4 now;   // source density, its deviation, own density, own deviation
+                    if (r < r_load) {
+                        const unsigned char *row = slots + slot * Cfg::SLOT_BYTES;
+                        value(row, col - cx, i, cx, cy, now.x, now.y);
+                        now.z = reinterpret_cast<const float *>(row)[k * BOXW + col];
+                        now.w = Codec<T>::dec(reinterpret_cast<const T *>(row + Cfg::RHO_BYTES)[(k * 8 + i - 1) * BOXW + col]);
+                        // (the node's own shifts sum to 5 m dphi_1: an eighth per lane)
+                        if (SPLIT)
+                            now.w += (k == 0 ? 0.625f : -0.625f) * p.dphi[1] * reinterpret_cast<const float *>(row)[2 * BOXW + col];
+                        if (wall_y && r == 0) across(row, hist[3 * 32]);   // stands for row -1
+                    } else {
+                        across(slots + ((p.ny - 1 - r0) % NSLOT) * Cfg::SLOT_BYTES, now);   // stands for row ny
+                    }
+                    if (closes && (outer == 0 || by_wall)) {
+                        const float4 one = hist[((r - 1) & 3) * 32];
+                        const float4 src = cy < 0 ? now : (cy == 0 ? one : hist[((r - 2) & 3) * 32]);
+                        const float u = fmav(phi, src.x - one.z, src.y);
+                        float v = u - one.w;
+                        v += __shfl_xor_sync(0xffffffffu, v, 1);
+                        v += __shfl_xor_sync(0xffffffffu, v, 2);
+                        v += __shfl_xor_sync(0xffffffffu, v, 4);
+                        const float mine = one.z + v;                        // colour k's new density
+                        const float other = __shfl_xor_sync(0xffffffffu, mine, 8);
+                        const float rr = k == 0 ? mine : other, rb = k == 0 ? other : mine;
+                        float jx = 0.0f, jy = 0.0f;
+                        if (HERMITE_SRC) {   // momentum: the shifts and rest parts cancel
+                            jx = (float)cx * u;
+                            jy = (float)cy * u;
+#pragma unroll
+                            for (int o = 1; o < 16; o <<= 1) {
+                                jx += __shfl_xor_sync(0xffffffffu, jx, o);
+                                jy += __shfl_xor_sync(0xffffffffu, jy, o);
+                            }
+                        }
+                        if ((lane & 15) == 0 &&
+                            !(OPEN && (side == 0 ? open_l : open_r || open_next || (open_next2 && outer)))) {
+                            ring_psi[at] = colour_field(p, rr, rb);
+                            if (HERMITE_SRC && outer == 0) {
+                                const float q = p.q_r * rr + p.q_b * rb, rho = rr + rb;
+                                ring_qx[at] = q * (jx / rho + 0.5f * p.gx);
+                                ring_qy[at] = q * (jy / rho + 0.5f * p.gy);
+                            }
+                        }
+                    }
+                    hist[(r & 3) * 32] = now;
+                }
+            }
+
+            f2 nC = zero, qx = zero, qy = zero;
+            if (closes && !wall_row && active) {
+                if (OPEN && ((open_l && tid == 0) || ((open_r || open_next || open_next2) && last))) {
+                    const float *q = opens + ((Y - ya + 1) & (2 * OPEN_ROWS - 1)) * OPEN_VALUES;
+                    auto put = [&](f2 &v, float s, bool second) { (second ? v.y : v.x) = s; };
+                    auto take = [&](const float *o, bool second) {
+                        put(Pn.rr, o[0], second), put(Pn.rb, o[1], second);
+                        put(Pn.e1, o[2], second), put(Pn.e2, o[3], second), put(Pn.e3, o[4], second);
+                        put(Pn.e4, o[5], second), put(Pn.e5, o[6], second), put(Pn.e6, o[7], second);
+                        put(Pn.e7, o[8], second), put(Pn.e8, o[9], second);
+                    };
+                    // values beyond an open end (x = -1, x = nx) are those of the open column itself
+                    // (zero gradient); a neighbouring outlet column's are its own
+                    auto beside = [&](const float *o, int at) {
+                        ring_psi[at] = colour_field(p, o[0], o[1]);
+                        if (HERMITE_SRC && !open_next2) {
+                            PulledOf<float> P{o[0], o[1], o[2], o[3], o[4], o[5], o[6], o[7], o[8], o[9]};
+                            float jx, jy;
+                            momentum_of(P, jx, jy);
+                            const float rho = o[0] + o[1], u = p.q_r * o[0] + p.q_b * o[1];
+                            ring_qx[at] = u * (jx / rho + 0.5f * p.gx);
+                            ring_qy[at] = u * (jy / rho + 0.5f * p.gy);
+                        }
+                    };
+                    if (open_l && tid == 0) {
+                        take(q, false);
+                        beside(q, -1);
+                    }
+                    if ((open_r || open_next || open_next2) && last) {
+                        if (open_r) take(q + 2 * OPEN_ROWS * OPEN_VALUES, both);
+                        beside(q + 2 * OPEN_ROWS * OPEN_VALUES, open_next2 ? w + 1 : w);
+                    }
+                }
+                nC = colour_field_of(K, Pn.rr, Pn.rb);
+                if (HERMITE_SRC) {
+                    f2 jx, jy;
+                    momentum_of(Pn, jx, jy);
+                    const f2 rho = Pn.rr + Pn.rb;
+                    const f2 q = fmav(K.q_r, Pn.rr, K.q_b * Pn.rb);
+                    qx = q * (f2{jx.x / rho.x, jx.y / rho.y} + K.hgx);
+                    qy = q * (f2{jy.x / rho.x, jy.y / rho.y} + K.hgy);
+                    ring_qx[tc] = qx.x, ring_qy[tc] = qy.x;
+                    if (both) ring_qx[tc + 1] = qx.y, ring_qy[tc + 1] = qy.y;
+                }
+                ring_psi[tc] = nC.x;
+                if (both) ring_psi[tc + 1] = nC.y;
+            }
+            // colour field of the wall row beyond Yn, from that row's own values; q u is zero
+            auto wall_fill = [&](int Yn, float *to) {
+                const float *f = rings + (Yn & 1) * RING + 2;
+                for (int cc = tid - 1; cc <= w; cc += NT)
+                    to[cc] = wall_psi(p, x0 + cc, [&](int Xp) { return f[Xp - x0]; });
+            };
+            if (wall_row) {
+                wall_fill(p.ny - 1, ring_psi);
+                if (HERMITE_SRC)
+                    for (int cc = tid; cc < w + 2; cc += NT) ring_qx[cc - 1] = ring_qy[cc - 1] = 0.0f;
+            }
+            __syncthreads();   // row Y's colour field is in the ring; row r was read
+            if (r < r_load) {
+                if (tid == 0 && r + NSLOT < r_load) issue(r + NSLOT, slot);
+                if (++slot == NSLOT) {
+                    slot = 0;
+                    phase ^= 1u;
+                }
+            }
+            if (!closes) continue;
+            if (wall_y && Y == 0 && ya == 0) {   // the wall below row 0
+                float *wall = rings + 2 * RING + 2;
+                wall_fill(0, wall);
+                __syncthreads();
+                if (active) {
+                    cC = f2{wall[tc], wall[tc + 1]}, cW = wall[tc - 1], cE = wall[tc + 2];
+                    cX = qcC = zero;
+                    qcW = qcE = 0.0f;
+                }
+            }
+            if (!active) continue;
+
+            // (an odd strip's last pair has its second column beyond the strip: that half holds
+            // the edge column, and its results are not stored)
+            const float nW = ring_psi[tc - 1], nE = ring_psi[tc + 2];
+            if (wall_row) nC = f2{ring_psi[tc], ring_psi[tc + 1]};
+            else if (!both) nC.y = ring_psi[tc + 1];
+            f2 nX = zero;
+            float qnE = 0.0f, qnW = 0.0f;
+            if (HERMITE_SRC) {
+                if (!both && !wall_row) qx.y = ring_qx[tc + 1], qy.y = ring_qy[tc + 1];
+                nX = f2{qx.y - ring_qx[tc - 1], ring_qx[tc + 2] - qx.x};
+                qnE = ring_qy[tc + 2];
+                qnW = ring_qy[tc - 1];
+            }
+            if (r - 2 >= ya) {
+                // 12 times the S2I4 gradient (Eq. (eq:colorGradient)), from differences only,
+                // so that a uniform field gives exactly zero
+                const f2 four = lit<f2, LIT_FOUR>();
+                auto row_diff = [](f2 m, float west, float east) { return f2{m.y - west, east - m.x}; };
+                f2 Fx = fmav(four, row_diff(cC, cW, cE), row_diff(nC, nW, nE) + row_diff(sC, sW, sE));
+                const f2 dC = nC - sC;
+                f2 Fy = fmav(four, dC, f2{dC.y + (nW - sW), (nE - sE) + dC.x});
+                f2 dQx = zero, dQy = zero;
+                if (WET) {
+                    contact_angle_adjust(d.wet, p, r - 2, Fx.x, Fy.x);
+                    contact_angle_adjust(d.wet, p, r - 2, Fx.y, Fy.y);
+                }
+                if (HERMITE_SRC) {
+                    dQx = fmav(four, cX, nX + sX);
+                    const f2 dq = qy - qsC;
+                    dQy = fmav(four, dq, f2{dq.y + (qnW - qsW), (qnE - qsE) + dq.x});
+                }
+                Collided<f2> o;
+                collide_of<CV, SPLIT, f2>(p, K, Pc, cC, Fx, Fy, dQx, dQy, o);
+                const uint32_t ps_rho = (uint32_t)d.rho_plane * 4u, ps_dev = (uint32_t)d.dev_plane * (uint32_t)sizeof(T);
+                auto store = [&](char *qr, char *qd) {
+                    auto put = [&](char *q, f2 v) { pair_to(reinterpret_cast<float *>(q), v); };
+                    put(qr, Pc.rr);
+                    put(qr + ps_rho, Pc.rb);
+                    if (SPLIT) {
+                        put(qr + 2ull * ps_rho, o.m);
+                        put(qr + 3ull * ps_rho, o.gx);
+                        put(qr + 4ull * ps_rho, o.gy);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 8; i++) {
+                        pair_to(reinterpret_cast<T *>(qd + (unsigned long long)ps_dev * i), o.r[i]);
+                        pair_to(reinterpret_cast<T *>(qd + (unsigned long long)ps_dev * (i + 8)), o.b[i]);
+                    }
+                };
+                if (both) store(out_rho, out_dev);
+                const bool per_x = !OPEN && p.bc_x == BC_PERIODIC;
+                if (per_x && (p.nx & 1) == 0) {
+                    // the pair's copies in the ghost columns of the other side (both on lattices
+                    // narrower than two ghosts)
+                    const long long nx = p.nx;
+                    if (x < Cfg::GMEM) store(out_rho + nx * 4, out_dev + nx * (long long)sizeof(T));
+                    if (x >= nx - Cfg::GMEM) store(out_rho - nx * 4, out_dev - nx * (long long)sizeof(T));
+                } else if (!both || (per_x && (x < Cfg::GMEM || x + 1 >= p.nx - Cfg::GMEM))) {
+                    // odd widths: single columns, in place (g = 0) or as ghost copies
+                    auto single = [&](int h, auto pick) {
+                        for (int g = both ? 1 : 0; g < 3; g++) {
+                            if (g == 1 && !(per_x && x + h < Cfg::GMEM)) continue;
+                            if (g == 2 && !(per_x && x + h >= p.nx - Cfg::GMEM)) continue;
+                            const long long to = h + (g == 0 ? 0 : (g == 1 ? p.nx : -p.nx));
+                            char *qr = out_rho + to * 4, *qd = out_dev + to * (long long)sizeof(T);
+                            *reinterpret_cast<float *>(qr) = pick(Pc.rr);
+                            *reinterpret_cast<float *>(qr + ps_rho) = pick(Pc.rb);
+                            if (SPLIT) {
+                                *reinterpret_cast<float *>(qr + 2ull * ps_rho) = pick(o.m);
+                                *reinterpret_cast<float *>(qr + 3ull * ps_rho) = pick(o.gx);
+                                *reinterpret_cast<float *>(qr + 4ull * ps_rho) = pick(o.gy);
+                            }
+#pragma unroll
+                            for (int i = 0; i < 8; i++) {
+                                *reinterpret_cast<T *>(qd + (unsigned long long)ps_dev * i) = Codec<T>::enc(pick(o.r[i]));
+                                *reinterpret_cast<T *>(qd + (unsigned long long)ps_dev * (i + 8)) = Codec<T>::enc(pick(o.b[i]));
+                            }
+                        }
+                    };
+                    single(0, [](f2 v) { return v.x; });
+                    if (both) single(1, [](f2 v) { return v.y; });
+                }
+                out_rho += d.rho_row * 4;
+                out_dev += d.dev_row * (long long)sizeof(T);
+            }
+            sC = cC, sW = cW, sE = cE;
+            cC = nC, cW = nW, cE = nE;
+            if (HERMITE_SRC) {
+                sX = cX, cX = nX;
+                qsC = qcC, qsW = qcW, qsE = qcE;
+                qcC = qy, qcW = qnW, qcE = qnE;
+            }
         }
 
-        if (s_bad) {
-            __syncthreads();
+        if (__syncthreads_or(!ok)) {
             if (tid == 0) {
                 atomicOr(err, ERR_TIMEOUT);
                 // wait (bounded) for the copies this block still has in flight, so
                 // that none lands after the block's shared memory is released: the
-                // latest phase issued into each slot covers the earlier ones
+                // latest phase issued into each slot (every row was issued by now)
+                // covers the earlier ones
                 for (int s = 0; s < NSLOT; s++) {
-                    int last = -1;
-                    for (int m = 0; m < next_m; ++m)
-                        if (m % NSLOT == s) last = m;
-                    if (last >= 0) mbar_wait_bounded(&bars[s], (uint32_t)((last / NSLOT) & 1), WAIT_LIMIT_CYCLES / 4);
+                    const int uses = (r_load - r0 - s + NSLOT - 1) / NSLOT;
+                    if (uses > 0) mbar_wait_bounded(&bars[s], (uint32_t)((uses - 1) & 1), WAIT_LIMIT_CYCLES / 4);
                 }
             }
             __syncthreads();
@@ -579,10 +822,10 @@ __global__ void k_tp_moments(const SimDesc *__restrict__ dp, int step_offset, fl
     if (t >= d.t_end) return;   // this simulation has stopped
     const int nx = p.nx, ny = p.ny;
     const long long n = (long long)nx * ny;
-    const GlobalLoader<T> L(d, (int)(t & 1));
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
          k += (long long)gridDim.x * blockDim.x) {
         const int x = (int)(k % nx), y = (int)(k / nx);
+        const RowLoader<T> L(d, (int)(t & 1), y);
         Pulled P;
         pull_node<HERMITE>(p, L, x, y, t, false, 0.0f, 0.0f, P);
         const NodeMoments m = node_moments(p, P);
@@ -630,10 +873,10 @@ __global__ void k_tp_collide(const SimDesc *__restrict__ dp, int step_offset, co
     const int nx = p.nx, ny = p.ny;
     const long long n = (long long)nx * ny;
     const int bsrc = (int)(t & 1);
-    const GlobalLoader<T> L(d, bsrc);
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
          k += (long long)gridDim.x * blockDim.x) {
         const int x = (int)(k % nx), y = (int)(k / nx);
+        const RowLoader<T> L(d, (int)(t & 1), y);
         Pulled P;
         pull_node<HERMITE>(p, L, x, y, t, true, aux[n + k], aux[2 * n + k], P);
         float Fx, Fy, dQx = 0.0f, dQy = 0.0f;
@@ -741,10 +984,10 @@ __global__ void k_fields(const SimDesc *__restrict__ dp, long long t, double *__
     const Phys p = d.ph;
     const int nx = p.nx, ny = p.ny;
     const long long n = (long long)nx * ny;
-    const GlobalLoader<T> L(d, (int)(t & 1));
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
          k += (long long)gridDim.x * blockDim.x) {
         const int x = (int)(k % nx), y = (int)(k / nx);
+        const RowLoader<T> L(d, (int)(t & 1), y);
         Pulled P;
         pull_node<HERMITE>(p, L, x, y, t, false, 0.0f, 0.0f, P);
         const NodeMoments m = node_moments(p, P);
@@ -766,11 +1009,11 @@ __global__ void k_slug_profile(const SimDesc *__restrict__ dp, long long t, doub
     const SimDesc &d = *dp;
     const Phys p = d.ph;
     const int nx = p.nx, ny = p.ny;
-    const GlobalLoader<T> L(d, (int)(t & 1));
     const int ya = (ny - 1) / 2, yb = ny / 2;   // the same row when ny is odd
     for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < nx; x += gridDim.x * blockDim.x) {
         double g = 0.0, pc = 0.0;
         for (int y = 0; y < ny; y++) {
+            const RowLoader<T> L(d, (int)(t & 1), y);
             Pulled P;
             pull_node<HERMITE>(p, L, x, y, t, false, 0.0f, 0.0f, P);
             const double a = (double)P.rr * p.inv_gamma, b = (double)P.rb;
@@ -790,10 +1033,10 @@ __global__ void k_read_pops(const SimDesc *__restrict__ dp, long long t, double 
     const Phys p = d.ph;
     const int nx = p.nx, ny = p.ny;
     const long long n = (long long)nx * ny;
-    const GlobalLoader<T> L(d, (int)(t & 1));
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
          k += (long long)gridDim.x * blockDim.x) {
         const int x = (int)(k % nx), y = (int)(k / nx);
+        const RowLoader<T> L(d, (int)(t & 1), y);
         double nr[9], nb[9];
         pull_populations<HERMITE>(p, L, x, y, t, nr, nb);
 #pragma unroll
@@ -848,13 +1091,13 @@ __global__ void __launch_bounds__(DIAG_THREADS) k_diag(const SimDesc *__restrict
     const Phys p = d.ph;
     const int nx = p.nx, ny = p.ny;
     const long long n = (long long)nx * ny;
-    const GlobalLoader<T> L(d, (int)(t & 1));
     double acc[DIAG_NQ];
 #pragma unroll
     for (int q = 0; q < DIAG_NQ; q++) acc[q] = 0.0;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
          k += (long long)gridDim.x * blockDim.x) {
         const int x = (int)(k % nx), y = (int)(k / nx);
+        const RowLoader<T> L(d, (int)(t & 1), y);
         Pulled P;
         pull_node<HERMITE>(p, L, x, y, t, false, 0.0f, 0.0f, P);
         const NodeMoments m = node_moments(p, P);

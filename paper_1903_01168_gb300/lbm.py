@@ -467,8 +467,8 @@ class Batch:
     def __init__(self, sims, rows_per_item: int = 0, row_overhead: float | None = None,
                  plan: int = LBM_PLAN_AUTO, member_plan_rows=None):
         """rows_per_item > 0: fixed plan; otherwise `plan` (LBM_PLAN_*) with
-        row_overhead, the planner's fixed cost of a strip row in busy warps
-        (None: library default), and optionally one plan_rows per member in
+        row_overhead, the planner's fixed cost of a strip row in quarters of a
+        full strip's width (None: library default), and optionally one plan_rows per member in
         place of the members' own."""
         self.sims = list(sims)
         self.h = lbm_batch_create([s.h for s in self.sims], rows_per_item, row_overhead, plan, member_plan_rows)
