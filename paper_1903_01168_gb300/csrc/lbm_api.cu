@@ -306,19 +306,20 @@ struct Plan {
     int blocks = 0;
 };
 
-// Launch flags for a plan run as the only launch of each step: a plan of one
-// piece per block, all of the same width and within one row of the same
-// height, lets the next step launch early (its blocks then land on whichever
-// SMs free first, which only matters where the pieces differ).
-int plan_flags(const Plan &P, bool only_launch) {
-    if (!only_launch || P.items.empty() || (int)P.items.size() != P.blocks) return 0;
-    int lo = 1 << 30, hi = 0, w0 = P.items[0].w;
+// Launch flags for a plan run as the only launch of each step: a plan of one piece per
+// block, all within an eighth of the same height, lets the next step launch early (its
+// blocks then land on whichever SMs free first, which only matters where the pieces
+// differ): 1000 x 301 MRT, whose last strip is narrower, 19.8 us a step without and 16.5
+// with.  So does a plan that leaves half the resident blocks' slots free.
+int plan_flags(const Plan &P, int resident) {
+    if (P.blocks * 2 <= resident) return FUSED_EARLY_NEXT;
+    if (P.items.empty() || (int)P.items.size() != P.blocks) return 0;
+    int lo = 1 << 30, hi = 0;
     for (const WorkItem &it : P.items) {
-        if (it.w != w0) return 0;
         lo = std::min(lo, it.yb - it.ya);
         hi = std::max(hi, it.yb - it.ya);
     }
-    return hi - lo <= 1 ? FUSED_EARLY_NEXT : 0;
+    return hi - lo <= std::max(1, hi / 8) ? FUSED_EARLY_NEXT : 0;
 }
 
 constexpr int MIN_PIECE = 8;   // default shortest row range worth a 4-row halo
@@ -331,8 +332,10 @@ constexpr double DEFAULT_ROW_OVERHEAD = 8.0;
 
 // Shortest row range where MIN_PIECE would leave resident blocks idle.  A block's march is a
 // chain of dependent row passes, so shorter pieces on more blocks win although each loads 4
-// rows more: one 2048 x 128 FP32 lattice 23.2 us a step with 8 rows, 13.9 with 2; 1024 x 300
-// 22.5 and 13.7; from 1024 x 1024 on the blocks are full either way.
+// rows more: one 2048 x 128 FP32 lattice 23.2 us a step with 8 rows, 13.0 with 2; 1024 x 300
+// 22.5 and 12.7; from 1024 x 1024 on the blocks are full either way.  Single rows are worth
+// it while they share an SM with few others: 128 x 128 8.0 us with 2 rows and 6.4 with 1,
+// 256 x 256 (3.4 blocks per SM with 1) 8.2 and 8.75.
 constexpr int SHORT_PIECE = 2;
 
 // Strips of a lattice; plan_rows 0 is set by default_pieces.
@@ -341,9 +344,12 @@ void strips_of(std::vector<StripRef> &out, int sim, int nx, int ny, int plan_row
 }
 
 void default_pieces(std::vector<StripRef> &strips, int max_blocks, bool may_shorten) {
-    long long pieces = 0;
-    for (const auto &s : strips) pieces += std::max(1, s.ny / (s.min_piece > 0 ? s.min_piece : MIN_PIECE));
-    const int rows = may_shorten && pieces < max_blocks ? SHORT_PIECE : MIN_PIECE;
+    long long pieces = 0, all_rows = 0;
+    for (const auto &s : strips) {
+        pieces += std::max(1, s.ny / (s.min_piece > 0 ? s.min_piece : MIN_PIECE));
+        all_rows += s.ny;
+    }
+    const int rows = !may_shorten || pieces >= max_blocks ? MIN_PIECE : (all_rows * 3 <= max_blocks ? 1 : SHORT_PIECE);
     for (auto &s : strips)
         if (s.min_piece <= 0) s.min_piece = rows;
 }
@@ -812,7 +818,7 @@ lbm_status create_common(int nx, int ny, const lbm_params *p, void *buf, size_t 
         Plan P = make_plan(strips, p->plan, 0, blocks, DEFAULT_ROW_OVERHEAD);
         s->n_items = (int)P.items.size();
         s->n_blocks = P.blocks;
-        s->launch_flags = plan_flags(P, true);
+        s->launch_flags = plan_flags(P, resident_blocks(p->storage, variant_of(p)));
         if (cudaMalloc(&s->d_items, P.items.size() * sizeof(WorkItem)) != cudaSuccess ||
             cudaMalloc(&s->d_off, P.off.size() * sizeof(int)) != cudaSuccess ||
             cudaMemcpy(s->d_items, P.items.data(), P.items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice) !=
@@ -1245,7 +1251,7 @@ lbm_status lbm_batch_create_ex(lbm_sim *const *sims, int n, const lbm_batch_opts
             const int blocks = plan_blocks(st, cv, nodes);
             default_pieces(strips, blocks, true);
             Plan P = make_plan(strips, opts->plan, rows_per_item, blocks, row_overhead);
-            lbm_batch::Group g{st, cv, (int)items.size(), (int)offs.size(), P.blocks, plan_flags(P, true)};
+            lbm_batch::Group g{st, cv, (int)items.size(), (int)offs.size(), P.blocks, plan_flags(P, resident_blocks(st, cv))};
             for (int &o : P.off) o += g.item0;
             items.insert(items.end(), P.items.begin(), P.items.end());
             offs.insert(offs.end(), P.off.begin(), P.off.end());

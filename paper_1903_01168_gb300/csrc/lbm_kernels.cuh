@@ -339,17 +339,6 @@ __global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_st
     constexpr bool SPLIT = SplitStore<T>::value;
     extern __shared__ __align__(128) unsigned char smem[];
 
-    // Launched as a programmatic dependent of the previous step: this block
-    // touches no memory that earlier work writes (descriptors, state, error word)
-    // before every prerequisite grid has completed and its writes are visible.
-    // With FUSED_EARLY_NEXT (plans of equal pieces, one launch per step) the next
-    // step may launch at once, its blocks waiting in the slots this grid frees;
-    // otherwise only once this block's work is done (below): on uneven batches
-    // and concurrent launch groups the early trigger placed waiting blocks on SMs
-    // in the order slots freed and cost 5-16 %.
-    if (flags & FUSED_EARLY_NEXT) asm volatile("griddepcontrol.launch_dependents;");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    if ((int)blockIdx.x >= n_blocks) return;
     const int tid = threadIdx.x;
 
     SimDesc &d = *reinterpret_cast<SimDesc *>(smem);
@@ -364,19 +353,14 @@ __global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_st
         return;
     }
 
-    const int it_end = item_off[blockIdx.x + 1];
-    for (int itx = item_off[blockIdx.x]; itx < it_end; ++itx) {
-        const WorkItem it = items[itx];
-        const SimDesc *gd = descs + it.sim;
-        __syncthreads();   // previous segment fully consumed (all its rows were waited for)
-        {
-            const int4 *src = reinterpret_cast<const int4 *>(gd);
-            int4 *dst = reinterpret_cast<int4 *>(smem);
-            for (int j = tid; j < (int)(sizeof(SimDesc) / 16); j += NT) dst[j] = src[j];
-        }
+    // descriptor of an item into shared memory, its row barriers and constants
+    auto prepare = [&](const SimDesc *gd, bool again) {
+        const int4 *src = reinterpret_cast<const int4 *>(gd);
+        int4 *dst = reinterpret_cast<int4 *>(smem);
+        for (int j = tid; j < (int)(sizeof(SimDesc) / 16); j += NT) dst[j] = __ldcv(src + j);
         if (tid == 0) {
             for (int s = 0; s < NSLOT; s++) {
-                if (itx != item_off[blockIdx.x]) mbar_inval(&bars[s]);
+                if (again) mbar_inval(&bars[s]);
                 mbar_init(&bars[s], 1);
             }
             fence_mbar_init();
@@ -386,10 +370,40 @@ __global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_st
         }
         __syncthreads();
         if (tid == NT - 1) fill_consts(K, d.ph);
+    };
+    // Launched as a programmatic dependent of the previous step: the work table and the
+    // first item's descriptor are read while that step still runs.  Nothing it writes is
+    // touched (state, error word) before every prerequisite grid has completed and its
+    // writes are visible.  The descriptors' times are written between chunks of steps: the
+    // first step of a chunk reads them again after the wait; a later one is launched by
+    // blocks that have all waited for that write themselves.
+    // With FUSED_EARLY_NEXT (plans of equal pieces or with most of the chip idle, one launch
+    // per step) the next step may launch at once, its blocks waiting in free slots;
+    // otherwise only once this block's work is done (below): on uneven batches
+    // and concurrent launch groups the early trigger placed waiting blocks on SMs
+    // in the order slots freed and cost 5-16 %.
+    const bool any = (int)blockIdx.x < n_blocks;
+    const int it_first = any ? item_off[blockIdx.x] : 0, it_end = any ? item_off[blockIdx.x + 1] : 0;
+    if (it_first < it_end) prepare(descs + items[it_first].sim, false);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (flags & FUSED_EARLY_NEXT) asm volatile("griddepcontrol.launch_dependents;");
+
+    for (int itx = it_first; itx < it_end; ++itx) {
+        const WorkItem it = items[itx];
+        const SimDesc *gd = descs + it.sim;
+        if (itx > it_first) {
+            __syncthreads();   // previous segment fully consumed (all its rows were waited for)
+            prepare(gd, true);
+        }
+        long long t0 = d.t0, t_end = d.t_end;
+        if (step_offset == 0 && itx == it_first) {
+            t0 = __ldcv(&gd->t0);
+            t_end = __ldcv(&gd->t_end);
+        }
 
         const Phys &p = d.ph;   // per-simulation constants, in shared memory
-        const long long t = d.t0 + step_offset;
-        if (t >= d.t_end) continue;   // this simulation has stopped
+        const long long t = t0 + step_offset;
+        if (t >= t_end) continue;   // this simulation has stopped
         const int bsrc = (int)(t & 1), bdst = bsrc ^ 1;
         const int x0 = it.x0, w = it.w, ya = it.ya, yb = it.yb;
         if (d.variant != CV || d.ghost != Cfg::GMEM || w <= 0 || w > W || x0 < 0 || x0 + w > p.nx || (x0 % 8) != 0 ||
