@@ -79,8 +79,11 @@ struct lbm_sim {
     int launch_flags = 0;   // fused-kernel flags of the plan (FUSED_EARLY_NEXT)
     int *d_err = nullptr;
     float *d_aux = nullptr;      // two-pass scratch field
-    double *d_part = nullptr;    // diagnostic partials + final
+    double *d_part = nullptr;    // diagnostic partials, the sums of both passes, block ticket
     int diag_blocks = 0;
+    double *d_prof = nullptr;    // slug profile (2 nx), kept from the first call
+    double *h_read = nullptr;    // pinned host buffer of the diagnostics and the profile
+    size_t h_read_bytes = 0;
     cudaGraphExec_t graph = nullptr;
     int graph_steps = 0;
     bool has_center = false;
@@ -588,29 +591,32 @@ void launch_read_pops(lbm_sim *s, int g, double *out) {
 }
 
 template <typename T, bool H>
-void launch_diag_t(lbm_sim *s, int pass, double cx, double cy, double rin, double rout) {
-    k_diag<T, H><<<s->diag_blocks, DIAG_THREADS, 0, s->stream>>>(s->d_desc, s->t, pass, cx, cy, rin, rout, s->d_part);
+void launch_diag_t(lbm_sim *s, double *fin, unsigned *ticket) {
+    k_diag<T, H, 0><<<s->diag_blocks, DIAG_THREADS, 0, s->stream>>>(s->d_desc, s->t, s->has_center, s->cx, s->cy, s->d_part,
+                                                                    fin, ticket);
+    k_diag<T, H, 1><<<s->diag_blocks, DIAG_THREADS, 0, s->stream>>>(s->d_desc, s->t, s->has_center, s->cx, s->cy, s->d_part,
+                                                                    fin, ticket);
 }
 
 template <typename T>
-void launch_diag_s(lbm_sim *s, int pass, double cx, double cy, double rin, double rout) {
-    if (s->h.variant & CV_HERMITE) launch_diag_t<T, true>(s, pass, cx, cy, rin, rout);
-    else launch_diag_t<T, false>(s, pass, cx, cy, rin, rout);
+void launch_diag_s(lbm_sim *s, double *fin, unsigned *ticket) {
+    if (s->h.variant & CV_HERMITE) launch_diag_t<T, true>(s, fin, ticket);
+    else launch_diag_t<T, false>(s, fin, ticket);
 }
 
-void launch_diag(lbm_sim *s, int pass, double cx, double cy, double rin, double rout) {
+void launch_diag(lbm_sim *s, double *fin, unsigned *ticket) {
     switch (s->p.storage) {
-    case ST_F32: launch_diag_s<float>(s, pass, cx, cy, rin, rout); break;
-    case ST_F16DEV: launch_diag_s<__half>(s, pass, cx, cy, rin, rout); break;
-    default: launch_diag_s<__nv_bfloat16>(s, pass, cx, cy, rin, rout); break;
+    case ST_F32: launch_diag_s<float>(s, fin, ticket); break;
+    case ST_F16DEV: launch_diag_s<__half>(s, fin, ticket); break;
+    default: launch_diag_s<__nv_bfloat16>(s, fin, ticket); break;
     }
 }
 
 template <typename T>
 void launch_slug_profile_s(lbm_sim *s, double *out) {
-    const int g = std::max(1, (s->nx + 127) / 128);
-    if (s->h.variant & CV_HERMITE) k_slug_profile<T, true><<<g, 128, 0, s->stream>>>(s->d_desc, s->t, out);
-    else k_slug_profile<T, false><<<g, 128, 0, s->stream>>>(s->d_desc, s->t, out);
+    const int g = std::max(1, std::min((s->nx + 31) / 32, 1 << 16));
+    if (s->h.variant & CV_HERMITE) k_slug_profile<T, true><<<g, 32 * SLUG_WARPS, 0, s->stream>>>(s->d_desc, s->t, out);
+    else k_slug_profile<T, false><<<g, 32 * SLUG_WARPS, 0, s->stream>>>(s->d_desc, s->t, out);
 }
 
 void launch_slug_profile(lbm_sim *s, double *out) {
@@ -701,12 +707,33 @@ lbm_status sync_t0(lbm_sim *s) {
     return LBM_OK;
 }
 
+lbm_status err_word_status(lbm_sim *s, int h) {
+    if (h & ERR_TIMEOUT) { set_err(s->err, "a bounded device wait timed out"); return LBM_ETIMEOUT; }
+    if (h & ERR_BADITEM) { set_err(s->err, "invalid work item"); return LBM_EINVAL; }
+    return LBM_OK;
+}
+
 lbm_status check_err_word(lbm_sim *s, int *d_err) {
     int h = 0;
     CK(cudaMemcpyAsync(&h, d_err, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
-    if (h & ERR_TIMEOUT) { set_err(s->err, "a bounded device wait timed out"); return LBM_ETIMEOUT; }
-    if (h & ERR_BADITEM) { set_err(s->err, "invalid work item"); return LBM_EINVAL; }
+    return err_word_status(s, h);
+}
+
+// The simulation's pinned read-back buffer, at least `bytes` long (kept until lbm_destroy:
+// a pageable copy is staged by the driver and synchronises on its own).
+lbm_status read_buffer(lbm_sim *s, size_t bytes) {
+    if (s->h_read_bytes >= bytes) return LBM_OK;
+    if (s->h_read) cudaFreeHost(s->h_read);
+    s->h_read = nullptr;
+    s->h_read_bytes = 0;
+    if (cudaMallocHost(reinterpret_cast<void **>(&s->h_read), bytes) != cudaSuccess) {
+        cudaGetLastError();
+        s->h_read = nullptr;
+        set_err(s->err, "pinned read-back buffer of %zu bytes failed", bytes);
+        return LBM_ENOMEM;
+    }
+    s->h_read_bytes = bytes;
     return LBM_OK;
 }
 
@@ -834,13 +861,15 @@ lbm_status create_common(int nx, int ny, const lbm_params *p, void *buf, size_t 
         set_err(s->err, "cudaMalloc of scratch field failed");
         return fail(LBM_ENOMEM);
     }
-    s->diag_blocks = grid_for((long long)nn, DIAG_THREADS);
-    if (cudaMalloc(&s->d_part, ((size_t)s->diag_blocks + 1) * DIAG_NQ * sizeof(double)) != cudaSuccess) {
+    s->diag_blocks = std::min(grid_for((long long)nn, DIAG_THREADS), DIAG_BLOCKS);
+    if (cudaMalloc(&s->d_part, ((size_t)s->diag_blocks + 3) * DIAG_NQ * sizeof(double)) != cudaSuccess) {
         set_err(s->err, "cudaMalloc of diagnostic scratch failed");
         return fail(LBM_ENOMEM);
     }
     if (cudaMemcpyAsync(s->d_desc, &s->h, sizeof(SimDesc), cudaMemcpyHostToDevice, s->stream) != cudaSuccess ||
         cudaMemsetAsync(s->d_err, 0, sizeof(int), s->stream) != cudaSuccess ||
+        cudaMemsetAsync(s->d_part + (size_t)(s->diag_blocks + 2) * DIAG_NQ, 0, DIAG_NQ * sizeof(double), s->stream) !=
+            cudaSuccess ||
         cudaMemsetAsync(s->pop, 0, s->pop_bytes, s->stream) != cudaSuccess ||
         cudaStreamSynchronize(s->stream) != cudaSuccess) {
         set_err(s->err, "initial uploads failed: %s", cudaGetErrorString(cudaGetLastError()));
@@ -1051,39 +1080,37 @@ lbm_status lbm_read_populations(lbm_sim *s, double *pops) {
 lbm_status lbm_diagnostics(lbm_sim *s, lbm_diag *out) {
     if (!s || !out) return LBM_EINVAL;
     memset(out, 0, sizeof(*out));
-    double h[DIAG_NQ];
-    double *fin = s->d_part + (size_t)s->diag_blocks * DIAG_NQ;
-    auto run = [&](int pass, double cx, double cy, double rin, double rout) -> lbm_status {
-        launch_diag(s, pass, cx, cy, rin, rout);
-        CK(cudaGetLastError());
-        k_diag_final<<<1, 32, 0, s->stream>>>(s->d_part, s->diag_blocks, fin);
-        CK(cudaGetLastError());
-        CK(cudaMemcpyAsync(h, fin, sizeof(h), cudaMemcpyDeviceToHost, s->stream));
-        CK(cudaStreamSynchronize(s->stream));
-        return LBM_OK;
-    };
-    lbm_status st = run(0, 0, 0, 0, 0);
+    // both passes, one copy, one wait: the second pass takes the first one's sums from
+    // device memory
+    constexpr size_t SUMS = 2 * DIAG_NQ;
+    lbm_status st = read_buffer(s, (SUMS + 1) * sizeof(double));
     if (st != LBM_OK) return st;
+    double *fin = s->d_part + (size_t)s->diag_blocks * DIAG_NQ;
+    launch_diag(s, fin, reinterpret_cast<unsigned *>(fin + SUMS));
+    CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(s->h_read, fin, SUMS * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
+    CK(cudaMemcpyAsync(s->h_read + SUMS, s->d_err, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+    CK(cudaStreamSynchronize(s->stream));
+    const double *h = s->h_read, *h1 = h + DIAG_NQ;
     out->t = s->t;
     out->mass_r = h[0];
     out->mass_b = h[1];
     out->mom_x = h[2];
     out->mom_y = h[3];
     out->area_b = h[4];
-    out->max_u = h[5];
+    out->max_u = std::sqrt(h[5]);
     out->cx_b = h[4] > 0 ? h[6] / h[4] : 0.0;
     out->cy_b = h[4] > 0 ? h[7] / h[4] : 0.0;
     out->ux_b = h[4] > 0 ? h[8] / h[4] : 0.0;
     out->ux_r = h[10] > 0 ? h[9] / h[10] : 0.0;
     out->nonfinite = (long long)h[11];
     out->r_eff = std::sqrt(std::max(h[4], 0.0) / M_PI);
-    const double cx = s->has_center ? s->cx : out->cx_b, cy = s->has_center ? s->cy : out->cy_b;
-    st = run(1, cx, cy, out->r_eff / 2.0, out->r_eff + 8.0);
-    if (st != LBM_OK) return st;
-    out->p_in = h[1] > 0 ? h[0] / h[1] : 0.0;
-    out->p_out = h[3] > 0 ? h[2] / h[3] : 0.0;
+    out->p_in = h1[1] > 0 ? h1[0] / h1[1] : 0.0;
+    out->p_out = h1[3] > 0 ? h1[2] / h1[3] : 0.0;
     out->dp = out->p_in - out->p_out;
-    st = check_err_word(s, s->d_err);
+    int e = 0;
+    memcpy(&e, s->h_read + SUMS, sizeof(int));
+    st = err_word_status(s, e);
     if (st != LBM_OK) return st;
     if (out->nonfinite > 0) {
         set_err(s->err, "%lld non-finite nodes at t = %lld", out->nonfinite, s->t);
@@ -1095,19 +1122,21 @@ lbm_status lbm_diagnostics(lbm_sim *s, lbm_diag *out) {
 lbm_status lbm_slug_geometry(lbm_sim *s, lbm_slug *out, double *gas) {
     if (!s || !out) return LBM_EINVAL;
     memset(out, 0, sizeof(*out));
-    const int nx = s->nx;
-    std::vector<double> h(2 * (size_t)nx);
-    double *d = nullptr;
-    CK(cudaMallocAsync(&d, 2 * (size_t)nx * sizeof(double), s->stream));
-    launch_slug_profile(s, d);
+    const size_t nx = (size_t)s->nx, bytes = 2 * nx * sizeof(double);
+    lbm_status st = read_buffer(s, bytes + sizeof(double));
+    if (st != LBM_OK) return st;
+    if (!s->d_prof) CK(cudaMalloc(&s->d_prof, bytes));
+    launch_slug_profile(s, s->d_prof);
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(h.data(), d, 2 * (size_t)nx * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
-    CK(cudaFreeAsync(d, s->stream));
+    CK(cudaMemcpyAsync(s->h_read, s->d_prof, bytes, cudaMemcpyDeviceToHost, s->stream));
+    CK(cudaMemcpyAsync(s->h_read + 2 * nx, s->d_err, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
     out->t = s->t;
-    slug_from_profile(h.data(), h.data() + nx, nx, s->ny, s->p.bc_x == LBM_BC_PERIODIC, out);
-    if (gas) memcpy(gas, h.data(), (size_t)nx * sizeof(double));
-    return check_err_word(s, s->d_err);
+    slug_from_profile(s->h_read, s->h_read + nx, s->nx, s->ny, s->p.bc_x == LBM_BC_PERIODIC, out);
+    if (gas) memcpy(gas, s->h_read, nx * sizeof(double));
+    int e = 0;
+    memcpy(&e, s->h_read + 2 * nx, sizeof(int));
+    return err_word_status(s, e);
 }
 
 size_t lbm_state_bytes(const lbm_sim *s) { return s ? s->pop_bytes + sizeof(long long) : 0; }
@@ -1150,6 +1179,8 @@ void lbm_destroy(lbm_sim *s) {
     cudaFree(s->d_err);
     cudaFree(s->d_aux);
     cudaFree(s->d_part);
+    cudaFree(s->d_prof);
+    if (s->h_read) cudaFreeHost(s->h_read);
     if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
     delete s;
 }

@@ -13,7 +13,7 @@
 //                  the same step as two plain node-parallel kernels with a
 //                  global scratch field (psi, q u) in between: the reference
 //                  GPU path, bit-identical to the fused one.
-//   k_init, k_fields, k_diag_*, k_advance, k_set_times   support kernels.
+//   k_init, k_fields, k_diag, k_slug_profile, k_advance, k_set_times   support kernels.
 #pragma once
 
 #include "lbm_device.cuh"
@@ -1017,26 +1017,45 @@ __global__ void k_fields(const SimDesc *__restrict__ dp, long long t, double *__
 // FP64: per column x the light-phase thickness g(x) = sum_y (1 - psi)/2, and the
 // colour field psi_c(x) on the channel centreline (the middle row, or the mean
 // of the two middle rows when ny is even).  out[0, nx) = g, out[nx, 2 nx) = psi_c.
-// One thread per column; the threads of a warp read neighbouring columns.
+// A block takes 32 columns, each warp every SLUG_WARPS-th row of them (neighbouring columns
+// in a warp); the warps' sums are added in a fixed order.  Bound by the latency of the
+// pulls, which a thread walking a whole column made one after another: diagnostics and
+// profile of a 2048 x 128 lattice together took 842 us, now 118 (profile 50).
+constexpr int SLUG_WARPS = 16;
 template <typename T, bool HERMITE>
-__global__ void k_slug_profile(const SimDesc *__restrict__ dp, long long t, double *__restrict__ out) {
+__global__ void __launch_bounds__(32 * SLUG_WARPS) k_slug_profile(const SimDesc *__restrict__ dp, long long t,
+                                                                  double *__restrict__ out) {
     const SimDesc &d = *dp;
     const Phys p = d.ph;
     const int nx = p.nx, ny = p.ny;
     const int ya = (ny - 1) / 2, yb = ny / 2;   // the same row when ny is odd
-    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < nx; x += gridDim.x * blockDim.x) {
-        double g = 0.0, pc = 0.0;
-        for (int y = 0; y < ny; y++) {
-            const RowLoader<T> L(d, (int)(t & 1), y);
-            Pulled P;
-            pull_node<HERMITE>(p, L, x, y, t, false, 0.0f, 0.0f, P);
-            const double a = (double)P.rr * p.inv_gamma, b = (double)P.rb;
-            const double psi = (a - b) / (a + b);     // Eq. (eq:color_field)
-            g += 0.5 * (1.0 - psi);
-            if (y == ya || y == yb) pc += psi;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ double sh_g[SLUG_WARPS][32], sh_a[32], sh_b[32];
+    for (int x0 = blockIdx.x * 32; x0 < nx; x0 += gridDim.x * 32) {
+        const int x = x0 + lane;
+        double g = 0.0;
+        if (x < nx) {
+            for (int y = warp; y < ny; y += SLUG_WARPS) {
+                const RowLoader<T> L(d, (int)(t & 1), y);
+                Pulled P;
+                pull_node<HERMITE>(p, L, x, y, t, false, 0.0f, 0.0f, P);
+                const double a = (double)P.rr * p.inv_gamma, b = (double)P.rb;
+                const double psi = (a - b) / (a + b);     // Eq. (eq:color_field)
+                g += 0.5 * (1.0 - psi);
+                if (y == ya) sh_a[lane] = psi;
+                if (y == yb) sh_b[lane] = psi;
+            }
         }
-        out[x] = g;
-        out[nx + x] = ya == yb ? pc : 0.5 * pc;
+        sh_g[warp][lane] = g;
+        __syncthreads();
+        if (warp == 0 && x < nx) {
+            double sum = sh_g[0][lane];
+#pragma unroll
+            for (int k = 1; k < SLUG_WARPS; k++) sum += sh_g[k][lane];
+            out[x] = sum;
+            out[nx + x] = ya == yb ? sh_a[lane] : 0.5 * (sh_a[lane] + sh_b[lane]);
+        }
+        __syncthreads();
     }
 }
 
@@ -1062,101 +1081,139 @@ __global__ void k_read_pops(const SimDesc *__restrict__ dp, long long t, double 
 }
 
 // ---------------------------------------------------------------- diagnostics
-constexpr int DIAG_NQ = 16;
+constexpr int DIAG_NQ = 16;        // slots of a block's partial sums
 constexpr int DIAG_THREADS = 256;
+constexpr int DIAG_BLOCKS = 152 * 2;   // at most: all resident at 128 registers a thread, one reduction each
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-__device__ __forceinline__ double warp_max(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-
-// Block-reduce DIAG_NQ values (slot 5 is a max, the rest sums) into part[block].
-__device__ __forceinline__ void block_reduce_store(double (&acc)[DIAG_NQ], double *part) {
-    __shared__ double sh[DIAG_THREADS / 32][DIAG_NQ];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < DIAG_NQ; q++) {
-        const double v = q == 5 ? warp_max(acc[q]) : warp_sum(acc[q]);
-        if (lane == 0) sh[wid][q] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < DIAG_NQ) {
-        const int q = threadIdx.x;
-        double v = sh[0][q];
-        for (int j = 1; j < DIAG_THREADS / 32; j++) v = q == 5 ? fmax(v, sh[j][q]) : v + sh[j][q];
-        part[(long long)blockIdx.x * DIAG_NQ + q] = v;
-    }
-}
-
-// pass 0: mass_r, mass_b, mom_x, mom_y, area_b, max|u| (slot 5), sum x w_b, sum y w_b,
+// pass 0: mass_r, mass_b, mom_x, mom_y, area_b, max |u|^2 (slot 5), sum x w_b, sum y w_b,
 //         sum ux w_b, sum ux w_r, sum w_r, nonfinite
-// pass 1: sum p (r < r_in), count, sum p (r > r_out), count around (cx, cy)
-template <typename T, bool HERMITE>
-__global__ void __launch_bounds__(DIAG_THREADS) k_diag(const SimDesc *__restrict__ dp, long long t, int pass,
-                                                       double cx, double cy, double r_in, double r_out,
-                                                       double *__restrict__ part) {
+// pass 1: sum p (r < r_eff / 2), count, sum p (r > r_eff + 8), count around the centre, from
+//         pass 0's sums (and the caller's centre, if there is one) in device memory
+// Every block reduces its nodes' values through shared memory into part[block]; the last
+// block to finish adds the blocks in order (deterministic) into fin[pass].  FP64 runs at
+// 2 operations per clock and SM, so a node's FP64 work is kept small (|u| is compared
+// squared, distances are decided in FP32 unless they lie within rounding of a radius), and
+// threads take several nodes before one reduction (a reduction per 256 nodes by shuffles
+// cost more FP64 time than the sums).  lbm_diagnostics of a 2048 x 128 / 8192 x 256 lattice:
+// 68 / 228 us with two resident blocks per SM, 91 / 254 with four.
+template <typename T, bool HERMITE, int PASS>
+__global__ void __launch_bounds__(DIAG_THREADS, 2) k_diag(const SimDesc *__restrict__ dp, long long t, bool has_center,
+                                                       double cx, double cy, double *__restrict__ part,
+                                                       double *__restrict__ fin, unsigned *__restrict__ ticket) {
+    constexpr int NQ = PASS == 0 ? 12 : 4;
     const SimDesc &d = *dp;
     const Phys p = d.ph;
     const int nx = p.nx, ny = p.ny;
     const long long n = (long long)nx * ny;
-    double acc[DIAG_NQ];
+    __shared__ double sh[NQ][DIAG_THREADS];
+    __shared__ bool s_last;
+    double acc[NQ];
 #pragma unroll
-    for (int q = 0; q < DIAG_NQ; q++) acc[q] = 0.0;
+    for (int q = 0; q < NQ; q++) acc[q] = 0.0;
+    double r_in = 0.0, r_out = 0.0;
+    float cxf = 0.0f, cyf = 0.0f, in2 = 0.0f, out2 = 0.0f;
+    if (PASS == 1) {
+        const double area = fin[4];
+        if (!has_center) {
+            cx = area > 0.0 ? fin[6] / area : 0.0;
+            cy = area > 0.0 ? fin[7] / area : 0.0;
+        }
+        const double r_eff = sqrt(fmax(area, 0.0) / 3.14159265358979323846);
+        r_in = r_eff / 2.0;
+        r_out = r_eff + 8.0;
+        cxf = (float)cx, cyf = (float)cy, in2 = (float)(r_in * r_in), out2 = (float)(r_out * r_out);
+    }
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
          k += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(k % nx), y = (int)(k / nx);
+        int x, y;
+        if (n <= 0x7fffffffLL) {
+            y = (int)((unsigned)k / (unsigned)nx);
+            x = (int)((unsigned)k - (unsigned)y * (unsigned)nx);
+        } else {
+            y = (int)(k / nx);
+            x = (int)(k - (long long)y * nx);
+        }
         const RowLoader<T> L(d, (int)(t & 1), y);
         Pulled P;
         pull_node<HERMITE>(p, L, x, y, t, false, 0.0f, 0.0f, P);
-        const NodeMoments m = node_moments(p, P);
-        const double rho = (double)m.rr + m.rb;
-        if (pass == 0) {
+        if (PASS == 0) {
+            const NodeMoments m = node_moments(p, P);
             const bool bad = !(isfinite(m.rr) && isfinite(m.rb) && isfinite(m.ux) && isfinite(m.uy));
-            if (bad) { acc[11] += 1.0; continue; }
+            if (bad) { acc[NQ - 1] += 1.0; continue; }
+            const double rho = (double)m.rr + m.rb, ux = m.ux, uy = m.uy;
             const double wb = 0.5 * (1.0 - m.psi), wr = 1.0 - wb;
             acc[0] += m.rr;
             acc[1] += m.rb;
-            acc[2] += rho * m.ux;
-            acc[3] += rho * m.uy;
-            acc[4] += wb;
-            acc[5] = fmax(acc[5], sqrt((double)m.ux * m.ux + (double)m.uy * m.uy));
-            acc[6] += wb * x;
-            acc[7] += wb * y;
-            acc[8] += wb * m.ux;
-            acc[9] += wr * m.ux;
-            acc[10] += wr;
+            acc[2] += rho * ux;
+            acc[3] += rho * uy;
+            acc[NQ > 4 ? 4 : 0] += wb;
+            acc[NQ > 5 ? 5 : 0] = fmax(acc[NQ > 5 ? 5 : 0], ux * ux + uy * uy);
+            acc[NQ > 6 ? 6 : 0] += wb * x;
+            acc[NQ > 7 ? 7 : 0] += wb * y;
+            acc[NQ > 8 ? 8 : 0] += wb * ux;
+            acc[NQ > 9 ? 9 : 0] += wr * ux;
+            acc[NQ > 10 ? 10 : 0] += wr;
         } else {
-            double dx = fabs(x - cx), dy = fabs(y - cy);
-            if (p.bc_x == BC_PERIODIC) dx = fmin(dx, nx - dx);
-            if (p.bc_y == BC_PERIODIC) dy = fmin(dy, ny - dy);
-            const double r = sqrt(dx * dx + dy * dy);
-            const double pr = (double)m.rr * p.cs2_r + (double)m.rb * p.cs2_b;
-            if (r < r_in) { acc[0] += pr; acc[1] += 1.0; }
-            if (r > r_out) { acc[2] += pr; acc[3] += 1.0; }
+            float fx = fabsf((float)x - cxf), fy = fabsf((float)y - cyf);
+            if (p.bc_x == BC_PERIODIC) fx = fminf(fx, (float)nx - fx);
+            if (p.bc_y == BC_PERIODIC) fy = fminf(fy, (float)ny - fy);
+            const float f2 = fx * fx + fy * fy;
+            bool inside = f2 < in2, outside = f2 > out2;
+            // FP32 rounding of the coordinates and of the squares: 1e-5 of the lattice and of r^2
+            const float slack = 1e-5f * f2 + 4e-6f * (float)(nx + ny) * (fx + fy + 1.0f);
+            if (!(fabsf(f2 - in2) > slack && fabsf(f2 - out2) > slack)) {
+                double dx = fabs(x - cx), dy = fabs(y - cy);
+                if (p.bc_x == BC_PERIODIC) dx = fmin(dx, nx - dx);
+                if (p.bc_y == BC_PERIODIC) dy = fmin(dy, ny - dy);
+                const double r = sqrt(dx * dx + dy * dy);
+                inside = r < r_in;
+                outside = r > r_out;
+            }
+            if (inside || outside) {
+                const double pr = (double)P.rr * p.cs2_r + (double)P.rb * p.cs2_b;
+                if (inside) { acc[0] += pr; acc[1] += 1.0; }
+                if (outside) { acc[2] += pr; acc[3] += 1.0; }
+            }
         }
     }
-    block_reduce_store(acc, part);
+    // 16 threads per quantity add 16 values each, then a shuffle tree over the 16
+    auto is_max = [](int q) { return PASS == 0 && q == 5; };
+    auto tree = [&](int q, double v) {
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+            const double w = __shfl_xor_sync(0xffffffffu, v, o);
+            v = is_max(q) ? fmax(v, w) : v + w;
+        }
+        return v;
+    };
+    const int q = threadIdx.x >> 4, l = threadIdx.x & 15;
+#pragma unroll
+    for (int j = 0; j < NQ; j++) sh[j][threadIdx.x] = acc[j];
+    __syncthreads();
+    double v = 0.0;
+    if (q < NQ) {
+        for (int j = l; j < DIAG_THREADS; j += 16) v = is_max(q) ? fmax(v, sh[q][j]) : v + sh[q][j];
+    }
+    v = tree(q, v);
+    if (q < NQ && l == 0) part[(long long)blockIdx.x * DIAG_NQ + q] = v;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;   // wraps to 0 for the next launch
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    v = 0.0;
+    if (q < NQ) {
+        for (int b = l; b < (int)gridDim.x; b += 16) {
+            const double w = __ldcg(part + (long long)b * DIAG_NQ + q);
+            v = is_max(q) ? fmax(v, w) : v + w;
+        }
+    }
+    v = tree(q, v);
+    if (q < NQ && l == 0) fin[PASS * DIAG_NQ + q] = v;
 }
 
 #ifndef LBM_DEVICE_HELPERS_ONLY   // non-template kernels: defined in one translation unit
-// Sum the per-block partials in block order (deterministic) into out[DIAG_NQ].
-__global__ void k_diag_final(const double *__restrict__ part, int nblocks, double *__restrict__ out) {
-    const int q = threadIdx.x;
-    if (q >= DIAG_NQ) return;
-    double v = q == 5 ? 0.0 : 0.0;
-    for (int b = 0; b < nblocks; b++) {
-        const double x = part[(long long)b * DIAG_NQ + q];
-        v = q == 5 ? fmax(v, x) : v + x;
-    }
-    out[q] = v;
-}
-
 // ------------------------------------------------------------------- time
 __global__ void k_advance(SimDesc *descs, int n, long long k) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) descs[i].t0 += k;
