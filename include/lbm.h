@@ -79,7 +79,9 @@ typedef enum { LBM_KERNEL_AUTO = 0, LBM_KERNEL_FUSED = 1, LBM_KERNEL_TWOPASS = 2
  * gives the same results; only the speed differs. */
 typedef enum {
     LBM_PLAN_AUTO = 0,      /* SPLIT when there are no more 128-column strips than
-                               resident blocks, else BALANCED (the default) */
+                               resident blocks, else BALANCED (the default); a small
+                               lattice periodic in x, with plan_rows 0 too, is stepped
+                               on its own in 64-column tiles instead of strips */
     LBM_PLAN_BALANCED = 1,  /* equal shares of row cost; a block may march over
                                several segments */
     LBM_PLAN_SPLIT = 2      /* one segment per block, the costliest segment as cheap

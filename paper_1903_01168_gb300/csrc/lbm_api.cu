@@ -77,6 +77,7 @@ struct lbm_sim {
     int *d_off = nullptr;        // per-block item ranges of the plan
     int n_items = 0, n_blocks = 0;
     int launch_flags = 0;   // fused-kernel flags of the plan (FUSED_EARLY_NEXT)
+    int tile_rows = 0, tile_warps = 0;   // > 0: lbm_step runs the tile kernel in this shape
     int *d_err = nullptr;
     float *d_aux = nullptr;      // two-pass scratch field
     double *d_part = nullptr;    // diagnostic partials, the sums of both passes, block ticket
@@ -541,6 +542,34 @@ int plan_blocks(int storage, int variant, long long nodes) {
     return storage == ST_F32 && nodes >= 1500000 ? std::max(1, all * 5 / 6) : all;
 }
 
+cudaError_t launch_tile_any(lbm_sim *s, int off) {
+    switch (s->p.storage) {
+    case ST_F32: return tile_launch<float>(s->h.variant, s->d_desc, s->nx, s->ny, s->tile_rows, s->tile_warps, off, s->d_err, s->stream);
+    case ST_F16DEV: return tile_launch<__half>(s->h.variant, s->d_desc, s->nx, s->ny, s->tile_rows, s->tile_warps, off, s->d_err, s->stream);
+    default: return tile_launch<__nv_bfloat16>(s->h.variant, s->d_desc, s->nx, s->ny, s->tile_rows, s->tile_warps, off, s->d_err, s->stream);
+    }
+}
+
+// Shape of the tile kernel for a lattice whose tiles are all resident at once (128 registers a
+// thread: 3 blocks of 5 warps, 2 of 7 or 4 of 4 per SM); strips (tile_rows 0) beyond, with open
+// ends, and where the caller set a plan.  Warps of their own for the nodes around the tile
+// shorten the step while they fit.  Microseconds a step with 2 rows in 5 warps, 4 in 7, 4 in 4
+// and strips: 200 x 200 5.8, 6.9, 6.8, 8.8; 256 x 256 9.7, 6.9, 7.4, 9.5; 512 x 256 14.8, 12.5,
+// 8.9, 11.1; 512 x 512 24.5, 23.3, 16.1, 12.7.
+void tile_shape(lbm_sim *s) {
+    if (s->p.bc_x != LBM_BC_PERIODIC || s->p.plan != LBM_PLAN_AUTO || s->p.plan_rows != 0) return;
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->dev);
+    const struct { int rows, warps, per_sm; } shapes[] = {{2, 5, 3}, {4, 7, 2}, {4, 4, 4}};
+    for (const auto &t : shapes) {
+        const long long tiles = (long long)((s->nx + TILE_W - 1) / TILE_W) * ((s->ny + t.rows - 1) / t.rows);
+        if (tiles > (long long)t.per_sm * sms) continue;
+        s->tile_rows = t.rows;
+        s->tile_warps = t.warps;
+        break;
+    }
+}
+
 int grid_for(long long n, int threads) {
     long long g = (n + threads - 1) / threads;
     return (int)std::max<long long>(1, std::min<long long>(g, 152LL * 16));
@@ -740,7 +769,9 @@ lbm_status read_buffer(lbm_sim *s, size_t bytes) {
 // Launch `n` steps of a single simulation directly (no graph).
 lbm_status step_direct(lbm_sim *s, long n) {
     for (long j = 0; j < n; j++) {
-        if (use_fused(s)) {
+        if (use_fused(s) && s->tile_rows > 0) {
+            CK(launch_tile_any(s, (int)j));
+        } else if (use_fused(s)) {
             CK(launch_fused_any(s->p.storage, s->h.variant, s->d_desc, s->d_items, s->d_off, s->n_blocks, (int)j,
                                 s->launch_flags, s->d_err, s->stream));
         } else {
@@ -855,6 +886,7 @@ lbm_status create_common(int nx, int ny, const lbm_params *p, void *buf, size_t 
             return fail(LBM_ENOMEM);
         }
     }
+    tile_shape(s);
     const size_t nn = (size_t)nx * ny;
     if (p->kernel == LBM_KERNEL_TWOPASS &&
         cudaMalloc(&s->d_aux, AUX_FIELDS * nn * sizeof(float)) != cudaSuccess) {

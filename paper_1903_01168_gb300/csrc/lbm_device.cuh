@@ -729,7 +729,7 @@ template <class F> __device__ __forceinline__ f2 each(f2 a, const F &f) { return
 // Literal constants: operands of the scalar code, pairs in the constant bank for the paired
 // code (as immediates a pair costs two moves at each use).
 enum : int { LIT_ZERO, LIT_QUARTER, LIT_HALF, LIT_ONE, LIT_3HALVES, LIT_TWO, LIT_FOUR, LIT_SIXTH, LIT_THIRD, LIT_TWELFTH,
-             LIT_DIAG, LIT_MHALF, LIT_M5, LIT_THREE, LIT_2THIRDS, LIT_144TH, LIT_M72TH, LIT_M2, LIT_N };
+             LIT_DIAG, LIT_MHALF, LIT_M5, LIT_THREE, LIT_2THIRDS, LIT_144TH, LIT_M72TH, LIT_M2, LIT_MQUARTER, LIT_M3HALVES, LIT_N };
 __host__ __device__ constexpr float LIT(int i) {
     return i == LIT_QUARTER    ? 0.25f
            : i == LIT_HALF     ? 0.5f
@@ -748,6 +748,8 @@ __host__ __device__ constexpr float LIT(int i) {
            : i == LIT_144TH    ? 1.0f / 144.0f
            : i == LIT_M72TH    ? -1.0f / 72.0f
            : i == LIT_M2       ? -2.0f
+           : i == LIT_MQUARTER ? -0.25f
+           : i == LIT_M3HALVES ? -1.5f
                                : 0.0f;
 }
 #define LBM_LIT2_(i) {LIT(i), LIT(i)}
@@ -755,7 +757,7 @@ static __constant__ f2 c_lit[LIT_N] = {
     LBM_LIT2_(0),  LBM_LIT2_(1),  LBM_LIT2_(2),  LBM_LIT2_(3),  LBM_LIT2_(4),  LBM_LIT2_(5),
     LBM_LIT2_(6),  LBM_LIT2_(7),  LBM_LIT2_(8),  LBM_LIT2_(9),  LBM_LIT2_(10), LBM_LIT2_(11),
     LBM_LIT2_(12), LBM_LIT2_(13), LBM_LIT2_(14), LBM_LIT2_(15), LBM_LIT2_(16),
-    LBM_LIT2_(17)};
+    LBM_LIT2_(17), LBM_LIT2_(18), LBM_LIT2_(19)};
 template <class V, int I>
 __device__ __forceinline__ V lit() {
     if constexpr (sizeof(V) == 8) return c_lit[I];
@@ -765,7 +767,7 @@ __device__ __forceinline__ V lit() {
 // Per-simulation constants of the node code; the paired code keeps them in shared memory.
 template <class V>
 struct Consts {
-    V phr, phb;              // phi^r_1, phi^b_1 (phi_2 is a quarter of phi_1)
+    V phr, phb, phr2, phb2;  // phi^r_1, phi^b_1 and a quarter of them, phi^r_2, phi^b_2
     V inv_gamma;
     V gx, gy, hgx, hgy;      // body acceleration, and half of it
     V a324;                  // -A / (324 omega_eff): perturbation from the gradient times 12
@@ -778,6 +780,7 @@ struct Consts {
 template <class V>
 __device__ __forceinline__ void fill_consts(Consts<V> &k, const Phys &p) {
     k.phr = bc<V>(p.phi_r[1]), k.phb = bc<V>(p.phi_b[1]);
+    k.phr2 = bc<V>(0.25f * p.phi_r[1]), k.phb2 = bc<V>(0.25f * p.phi_b[1]);
     k.inv_gamma = bc<V>(p.inv_gamma);
     k.gx = bc<V>(p.gx), k.gy = bc<V>(p.gy), k.hgx = bc<V>(0.5f * p.gx), k.hgy = bc<V>(0.5f * p.gy);
     k.a324 = bc<V>(p.a_coef * (-1.0f / 324.0f));
@@ -796,8 +799,11 @@ struct PulledOf {
 
 template <class V>
 __device__ __forceinline__ V colour_field_of(const Consts<V> &K, V rr, V rb) {
-    const V a = rr * K.inv_gamma;
-    const V n = a - rb, d = a + rb;
+    // (the difference per half: a packed operand has no sign, and the product must be fused)
+    const V d = fmav(rr, K.inv_gamma, rb);
+    V n;
+    if constexpr (sizeof(V) == 8) n = V{fmav(rr.x, K.inv_gamma.x, -rb.x), fmav(rr.y, K.inv_gamma.x, -rb.y)};
+    else n = fmav(rr, K.inv_gamma, -rb);
     if constexpr (sizeof(V) == 8) return V{n.x / d.x, n.y / d.y};   // IEEE division: exactly +-1 in a pure phase
     else return n / d;
 }

@@ -4,4 +4,6 @@
 #include "lbm_inst.cuh"
 
 LBM_INSTANTIATE_FUSED(__nv_bfloat16, 0)
+LBM_INSTANTIATE_TILE(__nv_bfloat16, 0)
 LBM_INSTANTIATE_FUSED(__nv_bfloat16, 1)
+LBM_INSTANTIATE_TILE(__nv_bfloat16, 1)

@@ -3,4 +3,6 @@
 #include "lbm_inst.cuh"
 
 LBM_INSTANTIATE_FUSED(__nv_bfloat16, 2)
+LBM_INSTANTIATE_TILE(__nv_bfloat16, 2)
 LBM_INSTANTIATE_FUSED(__nv_bfloat16, 3)
+LBM_INSTANTIATE_TILE(__nv_bfloat16, 3)

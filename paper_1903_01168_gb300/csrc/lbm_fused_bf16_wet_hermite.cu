@@ -3,4 +3,6 @@
 #include "lbm_inst.cuh"
 
 LBM_INSTANTIATE_FUSED(__nv_bfloat16, 6)
+LBM_INSTANTIATE_TILE(__nv_bfloat16, 6)
 LBM_INSTANTIATE_FUSED(__nv_bfloat16, 7)
+LBM_INSTANTIATE_TILE(__nv_bfloat16, 7)

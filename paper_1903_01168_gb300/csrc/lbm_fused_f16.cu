@@ -4,4 +4,6 @@
 #include "lbm_inst.cuh"
 
 LBM_INSTANTIATE_FUSED(__half, 0)
+LBM_INSTANTIATE_TILE(__half, 0)
 LBM_INSTANTIATE_FUSED(__half, 1)
+LBM_INSTANTIATE_TILE(__half, 1)

@@ -3,4 +3,6 @@
 #include "lbm_inst.cuh"
 
 LBM_INSTANTIATE_FUSED(__half, 2)
+LBM_INSTANTIATE_TILE(__half, 2)
 LBM_INSTANTIATE_FUSED(__half, 3)
+LBM_INSTANTIATE_TILE(__half, 3)

@@ -3,4 +3,6 @@
 #include "lbm_inst.cuh"
 
 LBM_INSTANTIATE_FUSED(__half, 4)
+LBM_INSTANTIATE_TILE(__half, 4)
 LBM_INSTANTIATE_FUSED(__half, 5)
+LBM_INSTANTIATE_TILE(__half, 5)

@@ -3,4 +3,6 @@
 #include "lbm_inst.cuh"
 
 LBM_INSTANTIATE_FUSED(__half, 6)
+LBM_INSTANTIATE_TILE(__half, 6)
 LBM_INSTANTIATE_FUSED(__half, 7)
+LBM_INSTANTIATE_TILE(__half, 7)

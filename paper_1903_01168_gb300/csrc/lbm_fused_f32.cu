@@ -4,4 +4,6 @@
 #include "lbm_inst.cuh"
 
 LBM_INSTANTIATE_FUSED(float, 0)
+LBM_INSTANTIATE_TILE(float, 0)
 LBM_INSTANTIATE_FUSED(float, 1)
+LBM_INSTANTIATE_TILE(float, 1)

@@ -3,4 +3,6 @@
 #include "lbm_inst.cuh"
 
 LBM_INSTANTIATE_FUSED(float, 2)
+LBM_INSTANTIATE_TILE(float, 2)
 LBM_INSTANTIATE_FUSED(float, 3)
+LBM_INSTANTIATE_TILE(float, 3)

@@ -3,4 +3,6 @@
 #include "lbm_inst.cuh"
 
 LBM_INSTANTIATE_FUSED(float, 4)
+LBM_INSTANTIATE_TILE(float, 4)
 LBM_INSTANTIATE_FUSED(float, 5)
+LBM_INSTANTIATE_TILE(float, 5)

@@ -3,4 +3,6 @@
 #include "lbm_inst.cuh"
 
 LBM_INSTANTIATE_FUSED(float, 6)
+LBM_INSTANTIATE_TILE(float, 6)
 LBM_INSTANTIATE_FUSED(float, 7)
+LBM_INSTANTIATE_TILE(float, 7)

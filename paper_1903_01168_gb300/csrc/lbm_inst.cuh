@@ -51,6 +51,20 @@ cudaError_t fused_launch_cv(const SimDesc *descs, const WorkItem *items, const i
 }
 
 template <typename T, int CV>
+cudaError_t tile_launch_cv(const SimDesc *desc, int nx, int ny, int rows, int warps, int off, int *err, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((nx + TILE_W - 1) / TILE_W), (unsigned)((ny + rows - 1) / rows));
+    cfg.blockDim = dim3((unsigned)(32 * warps));
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];   // programmatic dependent launch, as above
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = LBM_FUSED_PDL;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_step_tile<T, CV>, desc, off, rows, err);
+}
+
+template <typename T, int CV>
 cudaError_t twopass_launch_cv(const SimDesc *desc, int off, float *aux, long long nodes, cudaStream_t st) {
     const int g = (int)std::max<long long>(1, std::min<long long>((nodes + 255) / 256, 152LL * 16));
     k_tp_moments<T, CV><<<g, 256, 0, st>>>(desc, off, aux);
@@ -75,6 +89,9 @@ cudaError_t twopass_launch(int variant, const SimDesc *desc, int off, float *aux
                                                      int, int, int, int *, cudaStream_t);                      \
     template const void *lbm::fused_kernel_cv<T, CV>();                                                        \
     template int lbm::fused_smem_cv<T, CV>();
+
+#define LBM_INSTANTIATE_TILE(T, CV)                                                                                  \
+    template cudaError_t lbm::tile_launch_cv<T, CV>(const lbm::SimDesc *, int, int, int, int, int, int *, cudaStream_t);
 
 #define LBM_INSTANTIATE_TWOPASS(T) \
     template cudaError_t lbm::twopass_launch<T>(int, const lbm::SimDesc *, int, float *, long long, cudaStream_t);

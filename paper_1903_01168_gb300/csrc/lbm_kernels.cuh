@@ -199,40 +199,47 @@ struct RowTerms {
     f2 h_up, h_mid, h_dn;
 };
 
-// `slot`: the row in shared memory; `col`: the first of the thread's columns in it.  Each
-// stored value of a row is read in this one pass only.
-template <typename T, int BOXW, int RHO_BYTES>
-__device__ __forceinline__ RowTerms row_terms(const unsigned char *slot, int col, const Consts<f2> &K) {
-    const float *rp = reinterpret_cast<const float *>(slot) + col;
-    const T *dp = reinterpret_cast<const T *>(slot + RHO_BYTES) + col;
-    const f2 quarter = lit<f2, LIT_QUARTER>();
+// `rp`, `dp`: the thread's first column in planes 0 of the row's densities and deviations,
+// `rs`, `ds`: the distances of their planes.  In shared memory each stored value of a row is
+// read in this one pass only.
+template <typename T>
+__device__ __forceinline__ RowTerms row_terms(const float *rp, int rs, const T *dp, int ds, const Consts<f2> &K) {
     RowTerms R;
     f2 west[2], east[2];
     auto half = [&](int k, f2 &T1, f2 &T2, f2 &T3, f2 &T4, f2 &T5, f2 &T6, f2 &T7, f2 &T8) {
-        const f2 own = pair_at(rp + k * BOXW);
-        west[k] = f2{rp[k * BOXW - 1], own.x};
-        east[k] = f2{own.y, rp[k * BOXW + 2]};
+        const f2 own = pair_at(rp + k * rs);
+        west[k] = f2{rp[k * rs - 1], own.x};
+        east[k] = f2{own.y, rp[k * rs + 2]};
         R.own[k] = own;
-        const f2 phi1 = k == 0 ? K.phr : K.phb;   // phi_2 = phi_1 / 4
-        const f2 pW = phi1 * (west[k] - own), pE = phi1 * (east[k] - own);
-        const T *d = dp + (8 * k - 1) * BOXW;   // direction i at d + i * BOXW
-        auto at = [&](int i, int dx) { return Codec<T>::dec(d[i * BOXW + dx]); };
-        const f2 o1 = pair_at(d + 1 * BOXW), o3 = pair_at(d + 3 * BOXW);
-        T1 = pW + f2{at(1, -1), o1.x};
-        T3 = pE + f2{o3.y, at(3, 2)};
+        const f2 phi1 = k == 0 ? K.phr : K.phb;
+        const f2 dW = west[k] - own, dE = east[k] - own;
+        // phi_2 times a density step, added to a deviation.  16-bit storage holds phi_2 as a
+        // constant (2048 x 128 FP16 14.3 us a step, 14.9 with the quarter of phi_1's product
+        // that FP32 storage takes, where the constant costs 12.78 against 12.67).
+        f2 pW, pE;
+        if (!SplitStore<T>::value) pW = phi1 * dW, pE = phi1 * dE;
+        auto diag = [&](f2 step, f2 product, f2 dev) {
+            if (SplitStore<T>::value) return fmav(k == 0 ? K.phr2 : K.phb2, step, dev);
+            return fmav(lit<f2, LIT_QUARTER>(), product, dev);
+        };
+        const T *d = dp + (8 * k - 1) * ds;   // direction i at d + i * ds
+        auto at = [&](int i, int dx) { return Codec<T>::dec(d[i * ds + dx]); };
+        const f2 o1 = pair_at(d + 1 * ds), o3 = pair_at(d + 3 * ds);
+        T1 = fmav(phi1, dW, f2{at(1, -1), o1.x});
+        T3 = fmav(phi1, dE, f2{o3.y, at(3, 2)});
         f2 out = o1 + o3;
         R.mid[k] = T1 + T3;
-        const f2 o5 = pair_at(d + 5 * BOXW), o6 = pair_at(d + 6 * BOXW);
-        T5 = fmav(quarter, pW, f2{at(5, -1), o5.x});
-        T6 = fmav(quarter, pE, f2{o6.y, at(6, 2)});
+        const f2 o5 = pair_at(d + 5 * ds), o6 = pair_at(d + 6 * ds);
+        T5 = diag(dW, pW, f2{at(5, -1), o5.x});
+        T6 = diag(dE, pE, f2{o6.y, at(6, 2)});
         out = out + (o5 + o6);
-        T2 = pair_at(d + 2 * BOXW);
-        T4 = pair_at(d + 4 * BOXW);
+        T2 = pair_at(d + 2 * ds);
+        T4 = pair_at(d + 4 * ds);
         out = out + (T2 + T4);
         R.up[k] = T2 + (T5 + T6);
-        const f2 o7 = pair_at(d + 7 * BOXW), o8 = pair_at(d + 8 * BOXW);
-        T8 = fmav(quarter, pW, f2{at(8, -1), o8.x});
-        T7 = fmav(quarter, pE, f2{o7.y, at(7, 2)});
+        const f2 o7 = pair_at(d + 7 * ds), o8 = pair_at(d + 8 * ds);
+        T8 = diag(dW, pW, f2{at(8, -1), o8.x});
+        T7 = diag(dE, pE, f2{o7.y, at(7, 2)});
         out = out + (o7 + o8);
         R.dn[k] = T4 + (T7 + T8);
         R.mid[k] = R.mid[k] - out;
@@ -247,22 +254,47 @@ __device__ __forceinline__ RowTerms row_terms(const unsigned char *slot, int col
         // the shift of direction i is m dphi_c + (c_i . G) / |c_i| rest_c, rest_c = rho_r phi^r_c
         // + rho_b phi^b_c; phi_2 = phi_1 / 4 for both colours.  The node's own eight shifts sum
         // to 4 m (dphi_1 + dphi_2) = 5 m dphi_1.
-        const f2 pr = K.phr, pb = K.phb, dph = K.dphi;
+        const f2 pr = K.phr, pb = K.phb, dph = K.dphi, quarter = lit<f2, LIT_QUARTER>();
         const f2 rW = fmav(pr, west[0], pb * west[1]), rE = fmav(pr, east[0], pb * east[1]);
         const f2 rC = fmav(pr, R.own[0], pb * R.own[1]);
-        const float *mp = rp + 2 * BOXW, *xp = rp + 3 * BOXW, *yp = rp + 4 * BOXW;
+        const float *mp = rp + 2 * rs, *xp = rp + 3 * rs, *yp = rp + 4 * rs;
         const f2 mC = pair_at(mp), xC = pair_at(xp), yC = pair_at(yp);
-        const f2 a = mC * dph, b = yC * rC;
-        const f2 aWE = (f2{mp[-1], mC.x} + f2{mC.y, mp[2]}) * dph;
-        const f2 xWE = f2{xp[-1], xC.x} * rW - f2{xC.y, xp[2]} * rE;
+        const f2 b = yC * rC, mWE = f2{mp[-1], mC.x} + f2{mC.y, mp[2]};
+        const f2 xWE = fmav(f2{xp[-1], xC.x}, rW, f2{-xC.y, -xp[2]} * rE);
         const f2 yWE = fmav(f2{yp[-1], yC.x}, rW, f2{yC.y, yp[2]} * rE);
         const f2 D = lit<f2, LIT_DIAG>();
-        const f2 even = fmav(D, xWE, fmav(quarter, aWE, a)), odd = fmav(D, yWE, b);
+        const f2 even = fmav(D, xWE, dph * fmav(quarter, mWE, mC)), odd = fmav(D, yWE, b);
         R.h_up = even + odd;
         R.h_dn = even - odd;
-        R.h_mid = fmav(lit<f2, LIT_M5>(), a, aWE + xWE);
+        R.h_mid = fmav(dph, fmav(lit<f2, LIT_M5>(), mC, mWE), xWE);
     }
     return R;
+}
+
+// Terms of a no-slip wall for the row next to it, from that row's own deviations: the
+// opposite directions i, j, k of the links out of the wall (an axis, two diagonals); sgn: the
+// wall's side in y.
+struct WallTerms {
+    f2 sum[2], Ti, Tj, Tk, h;
+};
+template <typename T>
+__device__ __forceinline__ WallTerms wall_row_terms(const float *rp, int rs, const T *dp, int ds, const Consts<f2> &K, float dphi,
+                                                    int i, int j, int k, float sgn) {
+    auto at = [&](int plane) { return pair_at(dp + plane * ds); };
+    const f2 ri = at(i - 1), rj = at(j - 1), rk = at(k - 1), bi = at(i + 7), bj = at(j + 7), bk = at(k + 7);
+    WallTerms L;
+    L.sum[0] = ri + (rj + rk);
+    L.sum[1] = bi + (bj + bk);
+    L.Ti = ri + bi;
+    L.Tj = rj + bj;
+    L.Tk = rk + bk;
+    L.h = lit<f2, LIT_ZERO>();
+    if (SplitStore<T>::value) {
+        const f2 rest = fmav(K.phr, pair_at(rp), K.phb * pair_at(rp + rs));
+        L.h = fmav(bc<f2>(1.5f * dphi), pair_at(rp + 2 * rs),
+                   bc<f2>(sgn * (1.0f + 0.5f * 0.70710678118654752f)) * (pair_at(rp + 4 * rs) * rest));
+    }
+    return L;
 }
 
 // The nodes (x, r) of a thread between the passes over their own row and over row r + 1:
@@ -274,15 +306,34 @@ struct HalfPulled {
 };
 
 // Close the nodes (x, r): add the links from row r + 1 (dn, T4, T7, T8, h_dn) and form the
-// new densities and the colour-blind non-rest parts.  sr, sb: phi_1 times the density step
-// from (x, r) to (x, r + 1) (zero at a wall): it moves the reference of the links from
-// row r + 1, once on the axis and a quarter on each diagonal, 1.5 in the sum.
+// new densities and the colour-blind non-rest parts.  S: phi_1 times the density step from
+// (x, r) to (x, r + 1) (zero at a wall): it moves the reference of the links from row r + 1,
+// once on the axis and a quarter on each diagonal, 1.5 in the sum.
+//
+// Every product that is added to something is an explicit fused operation, here and in
+// row_terms: the compiler fuses a packed product into an addition where it has no other use,
+// which made the same sums round differently in different kernels.
+struct Step {
+    f2 r, b, sum;   // per colour, and of both
+};
+__device__ __forceinline__ Step step_of(const Consts<f2> &K, const f2 (&from)[2], const f2 (&to)[2]) {
+    Step S;
+    const f2 dr = to[0] - from[0];
+    S.r = K.phr * dr;
+    S.b = K.phb * (to[1] - from[1]);
+    S.sum = fmav(K.phr, dr, S.b);
+    return S;
+}
+__device__ __forceinline__ Step no_step() {
+    const f2 zero = lit<f2, LIT_ZERO>();
+    return Step{zero, zero, zero};
+}
 template <bool SPLIT>
 __device__ __forceinline__ void close_node(const Consts<f2> &K, const HalfPulled &H, f2 dn0, f2 dn1, f2 T4, f2 T7, f2 T8,
-                                           f2 h_dn, f2 sr, f2 sb, PulledOf<f2> &P) {
-    const f2 c15 = lit<f2, LIT_3HALVES>(), quarter = lit<f2, LIT_QUARTER>();
-    f2 ar = fmav(c15, sr, H.acc[0] + dn0);
-    f2 ab = fmav(c15, sb, H.acc[1] + dn1);
+                                           f2 h_dn, const Step &S, PulledOf<f2> &P) {
+    const f2 c15 = lit<f2, LIT_3HALVES>(), quarter = lit<f2, LIT_QUARTER>(), mquarter = lit<f2, LIT_MQUARTER>();
+    f2 ar = fmav(c15, S.r, H.acc[0] + dn0);
+    f2 ab = fmav(c15, S.b, H.acc[1] + dn1);
     if (SPLIT) {
         const f2 h = H.h + h_dn;
         ar = ar + h;
@@ -292,16 +343,160 @@ __device__ __forceinline__ void close_node(const Consts<f2> &K, const HalfPulled
     P.rb = H.own[1] + ab;
     // rest part of the density change on the axis links
     const f2 R1 = fmav(K.phr, P.rr - H.own[0], K.phb * (P.rb - H.own[1]));
-    const f2 up = (sr + sb) - R1, R4 = quarter * R1, up4 = quarter * up;
+    const f2 up = S.sum - R1;
     P.e1 = H.T1 - R1;
     P.e2 = H.T2 - R1;
     P.e3 = H.T3 - R1;
     P.e4 = T4 + up;
-    P.e5 = H.T5 - R4;
-    P.e6 = H.T6 - R4;
-    P.e7 = T7 + up4;
-    P.e8 = T8 + up4;
+    P.e5 = fmav(mquarter, R1, H.T5);
+    P.e6 = fmav(mquarter, R1, H.T6);
+    P.e7 = fmav(quarter, up, T7);
+    P.e8 = fmav(quarter, up, T8);
 }
+
+// Post-collision state of the nodes (x, y) and, with `both`, (x + 1, y) of a lattice of
+// descriptor d, and its copies in the ghost columns of a periodic lattice.  out_rho,
+// out_dev: where planes 0 of node (x, y) are.
+template <typename T, bool SPLIT>
+__device__ __forceinline__ void store_pair(const SimDesc &d, bool per_x, int x, bool both, char *out_rho, char *out_dev, f2 rr, f2 rb,
+                                           const Collided<f2> &o) {
+    constexpr int GMEM = 8;   // ghost columns (checked against the descriptor by the kernels)
+    const uint32_t ps_rho = (uint32_t)d.rho_plane * 4u, ps_dev = (uint32_t)d.dev_plane * (uint32_t)sizeof(T);
+    const long long nx = d.ph.nx;
+    auto store = [&](char *qr, char *qd) {
+        auto put = [&](char *q, f2 v) { pair_to(reinterpret_cast<float *>(q), v); };
+        put(qr, rr);
+        put(qr + ps_rho, rb);
+        if (SPLIT) {
+            put(qr + 2ull * ps_rho, o.m);
+            put(qr + 3ull * ps_rho, o.gx);
+            put(qr + 4ull * ps_rho, o.gy);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            pair_to(reinterpret_cast<T *>(qd + (unsigned long long)ps_dev * i), o.r[i]);
+            pair_to(reinterpret_cast<T *>(qd + (unsigned long long)ps_dev * (i + 8)), o.b[i]);
+        }
+    };
+    if (both) store(out_rho, out_dev);
+    if (per_x && (nx & 1) == 0) {
+        // the pair's copies in the ghost columns of the other side (both on lattices
+        // narrower than two ghosts)
+        if (x < GMEM) store(out_rho + nx * 4, out_dev + nx * (long long)sizeof(T));
+        if (x >= nx - GMEM) store(out_rho - nx * 4, out_dev - nx * (long long)sizeof(T));
+    } else if (!both || (per_x && (x < GMEM || x + 1 >= nx - GMEM))) {
+        // odd widths: single columns, in place (g = 0) or as ghost copies
+        auto single = [&](int h, auto pick) {
+            for (int g = both ? 1 : 0; g < 3; g++) {
+                if (g == 1 && !(per_x && x + h < GMEM)) continue;
+                if (g == 2 && !(per_x && x + h >= nx - GMEM)) continue;
+                const long long to = h + (g == 0 ? 0 : (g == 1 ? nx : -nx));
+                char *qr = out_rho + to * 4, *qd = out_dev + to * (long long)sizeof(T);
+                *reinterpret_cast<float *>(qr) = pick(rr);
+                *reinterpret_cast<float *>(qr + ps_rho) = pick(rb);
+                if (SPLIT) {
+                    *reinterpret_cast<float *>(qr + 2ull * ps_rho) = pick(o.m);
+                    *reinterpret_cast<float *>(qr + 3ull * ps_rho) = pick(o.gx);
+                    *reinterpret_cast<float *>(qr + 4ull * ps_rho) = pick(o.gy);
+                }
+#pragma unroll
+                for (int i = 0; i < 8; i++) {
+                    *reinterpret_cast<T *>(qd + (unsigned long long)ps_dev * i) = Codec<T>::enc(pick(o.r[i]));
+                    *reinterpret_cast<T *>(qd + (unsigned long long)ps_dev * (i + 8)) = Codec<T>::enc(pick(o.b[i]));
+                }
+            }
+        };
+        single(0, [](f2 v) { return v.x; });
+        if (both) single(1, [](f2 v) { return v.y; });
+    }
+}
+
+// Nodes beside a strip, link by link: the split form's shift of one link (gc: c_i . G) and the
+// colour field.  Every product that is added to something is an explicit fused operation, so
+// that such a node has the same bits wherever it is formed.
+__device__ __forceinline__ float edge_shift(const Phys &p, bool axis, float rr, float rb, float m, float gc) {
+    const float rest = __fmaf_rn(p.phi_r[1], rr, __fmul_rn(p.phi_b[1], rb)) * (axis ? 1.0f : 0.25f);
+    return __fmaf_rn(axis ? p.dphi[1] : p.dphi[2], m, __fmul_rn(__fmul_rn(axis ? 1.0f : 0.70710678118654752f, gc), rest));
+}
+__device__ __forceinline__ float edge_colour(const Phys &p, float rr, float rb) {
+    return __fmaf_rn(rr, p.inv_gamma, -rb) / __fmaf_rn(rr, p.inv_gamma, rb);
+}
+
+// One link of a node beside a strip, direction i of colour k, on one lane, from global memory:
+// lanes 8 k + (i - 1) of a half warp form the node's psi (and q u) by shuffles, with the
+// operations of the strip kernel's edge lanes.  `rp`, `dp`: the node's column in planes 0 of a
+// row, `rs`, `ds`: the distances of the planes.
+struct EdgeLink {
+    const Phys &p;
+    int i, k, cx, cy;
+    bool axis;
+    float phi;
+    __device__ __forceinline__ EdgeLink(const Phys &p_, int i_, int k_) : p(p_), i(i_), k(k_) {
+        cx = (i == 1 || i == 5 || i == 8) ? 1 : ((i == 3 || i == 6 || i == 7) ? -1 : 0);
+        cy = (i == 2 || i == 5 || i == 6) ? 1 : ((i == 4 || i == 7 || i == 8) ? -1 : 0);
+        axis = i <= 4;
+        phi = (k == 0 ? p.phi_r[1] : p.phi_b[1]) * (axis ? 1.0f : 0.25f);
+    }
+    // density and decoded deviation of direction (dx, dy), plane j, at the given column
+    template <typename T>
+    __device__ __forceinline__ void value(const float *rp, int rs, const T *dp, int ds, int j, int dx, int dy, float &s,
+                                          float &dv) const {
+        s = rp[k * rs];
+        dv = Codec<T>::dec(dp[(k * 8 + j - 1) * ds]);
+        if (SplitStore<T>::value) {
+            const float gc = (float)dx * rp[3 * rs] + (float)dy * rp[4 * rs];
+            const float h = edge_shift(p, axis, rp[0], rp[rs], rp[2 * rs], gc);
+            dv = __fadd_rn(dv, k == 0 ? h : -h);
+        }
+    }
+    // the link's source in its own row, the row of y - cy
+    template <typename T>
+    __device__ __forceinline__ void source(const float *rp, int rs, const T *dp, int ds, float &s, float &dv) const {
+        value<T>(rp - cx, rs, dp - cx, ds, i, cx, cy, s, dv);
+    }
+    // source across a wall next to the row: the node itself in the opposite direction, or (free
+    // slip) the row's neighbour in the mirrored one
+    template <typename T>
+    __device__ __forceinline__ void across(const float *rp, int rs, const T *dp, int ds, bool slip, float &s, float &dv) const {
+        const int opp = i <= 4 ? ((i + 1) & 3) + 1 : ((i - 3) & 3) + 5;
+        const int mir = i == 2 ? 4 : i == 4 ? 2 : i == 5 ? 8 : i == 8 ? 5 : i == 6 ? 7 : i == 7 ? 6 : i;
+        const int at = slip ? -cx : 0;
+        value<T>(rp + at, rs, dp + at, ds, slip ? mir : opp, slip ? cx : -cx, -cy, s, dv);
+    }
+    // the node's own density and deviation (its own shifts sum to 5 m dphi_1: an eighth per lane)
+    template <typename T>
+    __device__ __forceinline__ void own(const float *rp, int rs, const T *dp, int ds, float &s, float &dv) const {
+        s = rp[k * rs];
+        dv = Codec<T>::dec(dp[(k * 8 + i - 1) * ds]);
+        if (SplitStore<T>::value) dv = __fmaf_rn((k == 0 ? 0.625f : -0.625f) * p.dphi[1], rp[2 * rs], dv);
+    }
+    // psi and q u from the lanes' links (source density and deviation, own ones)
+    template <bool NEED_J>
+    __device__ __forceinline__ void node(unsigned lanes, float s, float dv, float own_s, float own_dv, float &psi, float &qx,
+                                         float &qy) const {
+        const float u = __fmaf_rn(phi, __fsub_rn(s, own_s), dv);
+        float v = __fsub_rn(u, own_dv);
+        v = __fadd_rn(v, __shfl_xor_sync(lanes, v, 1));
+        v = __fadd_rn(v, __shfl_xor_sync(lanes, v, 2));
+        v = __fadd_rn(v, __shfl_xor_sync(lanes, v, 4));
+        const float mine = __fadd_rn(own_s, v);                       // colour k's new density
+        const float other = __shfl_xor_sync(lanes, mine, 8);
+        const float rr = k == 0 ? mine : other, rb = k == 0 ? other : mine;
+        psi = edge_colour(p, rr, rb);
+        qx = qy = 0.0f;
+        if (NEED_J) {   // momentum: the shifts and rest parts cancel
+            float jx = (float)cx * u, jy = (float)cy * u;
+#pragma unroll
+            for (int o = 1; o < 16; o <<= 1) {
+                jx = __fadd_rn(jx, __shfl_xor_sync(lanes, jx, o));
+                jy = __fadd_rn(jy, __shfl_xor_sync(lanes, jy, o));
+            }
+            const float q = __fmaf_rn(p.q_r, rr, __fmul_rn(p.q_b, rb)), rho = __fadd_rn(rr, rb);
+            qx = __fmul_rn(q, __fadd_rn(jx / rho, 0.5f * p.gx));
+            qy = __fmul_rn(q, __fadd_rn(jy / rho, 0.5f * p.gy));
+        }
+    }
+};
 
 // Persistent fused step.  Block b processes the work items
 // items[item_off[b] .. item_off[b+1]) in order (strip segments, possibly of
@@ -457,25 +652,9 @@ __global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_st
         f2 sC = zero, cC = zero, sX = zero, cX = zero, qsC = zero, qcC = zero;
         float sW = 0.0f, sE = 0.0f, cW = 0.0f, cE = 0.0f, qsW = 0.0f, qsE = 0.0f, qcW = 0.0f, qcE = 0.0f;
 
-        // terms of a no-slip wall for the row next to it, from that row's own deviations:
-        // the opposite directions i, j, k of the links out of the wall (an axis, two
-        // diagonals); sgn: the wall's side in y
-        auto wall_terms = [&](const unsigned char *sp, int i, int j, int k, float sgn, f2 &sum_r, f2 &sum_b, f2 &Ti, f2 &Tj,
-                              f2 &Tk, f2 &h) {
-            const float *rp = reinterpret_cast<const float *>(sp) + tc + G;
-            const T *dp = reinterpret_cast<const T *>(sp + Cfg::RHO_BYTES) + tc + G;
-            auto at = [&](int plane) { return pair_at(dp + plane * BOXW); };
-            const f2 ri = at(i - 1), rj = at(j - 1), rk = at(k - 1), bi = at(i + 7), bj = at(j + 7), bk = at(k + 7);
-            sum_r = ri + (rj + rk);
-            sum_b = bi + (bj + bk);
-            Ti = ri + bi;
-            Tj = rj + bj;
-            Tk = rk + bk;
-            if (SPLIT) {
-                const f2 rest = fmav(K.phr, pair_at(rp), K.phb * pair_at(rp + BOXW));
-                h = fmav(bc<f2>(1.5f * p.dphi[1]), pair_at(rp + 2 * BOXW),
-                         bc<f2>(sgn * (1.0f + 0.5f * 0.70710678118654752f)) * (pair_at(rp + 4 * BOXW) * rest));
-            }
+        auto wall_terms = [&](const unsigned char *sp, int i, int j, int k, float sgn) {
+            return wall_row_terms<T>(reinterpret_cast<const float *>(sp) + tc + G, BOXW,
+                                     reinterpret_cast<const T *>(sp + Cfg::RHO_BYTES) + tc + G, BOXW, K, p.dphi[1], i, j, k, sgn);
         };
         int slot = 0;
         uint32_t phase = 0;
@@ -503,34 +682,36 @@ __global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_st
             }
             Pc = Pn;
             float *ring_psi = rings + (Y & 1) * RING + 2, *ring_qx = ring_psi + Cfg::QX_OFF, *ring_qy = ring_psi + Cfg::QY_OFF;
+            if (r < r_load && ok && !mbar_wait_bounded(&bars[slot], phase, WAIT_LIMIT_CYCLES)) ok = false;
             if (r < r_load) {
-                if (ok && !mbar_wait_bounded(&bars[slot], phase, WAIT_LIMIT_CYCLES)) ok = false;
                 const unsigned char *sp = slots + slot * Cfg::SLOT_BYTES;
                 if (active) {
-                    const RowTerms R = row_terms<T, BOXW, Cfg::RHO_BYTES>(sp, tc + G, K);
-                    f2 sr = K.phr * (R.own[0] - H.own[0]), sb = K.phb * (R.own[1] - H.own[1]);
-                    if (closes) close_node<SPLIT>(K, H, R.dn[0], R.dn[1], R.T4, R.T7, R.T8, R.h_dn, sr, sb, Pn);
+                    const RowTerms R = row_terms<T>(reinterpret_cast<const float *>(sp) + tc + G, BOXW,
+                                                    reinterpret_cast<const T *>(sp + Cfg::RHO_BYTES) + tc + G, BOXW, K);
+                    Step S = step_of(K, H.own, R.own);
+                    if (closes) close_node<SPLIT>(K, H, R.dn[0], R.dn[1], R.T4, R.T7, R.T8, R.h_dn, S, Pn);
                     if (wall_y && r == 0) {
                         // links from behind the lower wall: the node's own opposite
                         // populations (no slip), or those of its row travelling on
                         // mirrored (free slip)
-                        sr = sb = zero;
+                        S = no_step();
                         if (WET && d.wet.slip) {
                             lo0 = R.dn[0], lo1 = R.dn[1];
                             lo2 = R.T4, lo5 = R.T8, lo6 = R.T7, lo_h = R.h_dn;
                         } else {
-                            wall_terms(sp, 4, 7, 8, -1.0f, lo0, lo1, lo2, lo5, lo6, lo_h);
+                            const WallTerms L = wall_terms(sp, 4, 7, 8, -1.0f);
+                            lo0 = L.sum[0], lo1 = L.sum[1], lo2 = L.Ti, lo5 = L.Tj, lo6 = L.Tk, lo_h = L.h;
                         }
                     }
-                    const f2 z = sr + sb, z4 = z * lit<f2, LIT_QUARTER>(), c15 = lit<f2, LIT_3HALVES>();
+                    const f2 mquarter = lit<f2, LIT_MQUARTER>(), m15 = lit<f2, LIT_M3HALVES>();
                     H.own[0] = R.own[0], H.own[1] = R.own[1];
-                    H.acc[0] = (R.mid[0] + lo0) - c15 * sr;
-                    H.acc[1] = (R.mid[1] + lo1) - c15 * sb;
+                    H.acc[0] = fmav(m15, S.r, R.mid[0] + lo0);
+                    H.acc[1] = fmav(m15, S.b, R.mid[1] + lo1);
                     H.T1 = R.T1;
                     H.T3 = R.T3;
-                    H.T2 = lo2 - z;
-                    H.T5 = lo5 - z4;
-                    H.T6 = lo6 - z4;
+                    H.T2 = lo2 - S.sum;
+                    H.T5 = fmav(mquarter, S.sum, lo5);
+                    H.T6 = fmav(mquarter, S.sum, lo6);
                     if (SPLIT) H.h = lo_h + R.h_mid;
                     lo0 = R.up[0], lo1 = R.up[1];
                     lo2 = R.T2, lo5 = R.T5, lo6 = R.T6;
@@ -539,9 +720,11 @@ __global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_st
             } else if (active && !wall_row) {
                 // the row above is the upper wall (r == ny, row ny - 1 still in its slot)
                 f2 dn0 = lo0, dn1 = lo1, T4 = lo2, T7 = lo6, T8 = lo5, h_dn = lo_h;
-                if (!(WET && d.wet.slip))
-                    wall_terms(slots + ((p.ny - 1 - r0) % NSLOT) * Cfg::SLOT_BYTES, 2, 5, 6, 1.0f, dn0, dn1, T4, T7, T8, h_dn);
-                close_node<SPLIT>(K, H, dn0, dn1, T4, T7, T8, h_dn, zero, zero, Pn);
+                if (!(WET && d.wet.slip)) {
+                    const WallTerms L = wall_terms(slots + ((p.ny - 1 - r0) % NSLOT) * Cfg::SLOT_BYTES, 2, 5, 6, 1.0f);
+                    dn0 = L.sum[0], dn1 = L.sum[1], T4 = L.Ti, T7 = L.Tj, T8 = L.Tk, h_dn = L.h;
+                }
+                close_node<SPLIT>(K, H, dn0, dn1, T4, T7, T8, h_dn, no_step(), Pn);
             }
             // The columns beside the strip, x0 - 1 and x0 + w, need psi (and q u) only.  The last
             // warp computes them, 16 lanes per side, lane j = 8 k + (i - 1) for colour k's
@@ -565,10 +748,8 @@ __global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_st
                         s = rp[k * BOXW];
                         dv = Codec<T>::dec(reinterpret_cast<const T *>(row + Cfg::RHO_BYTES)[(k * 8 + j - 1) * BOXW + q]);
                         if (SPLIT) {
-                            const float rest = fmav(p.phi_r[1], rp[0], p.phi_b[1] * rp[BOXW]) * (axis ? 1.0f : 0.25f);
                             const float gc = (float)dx * rp[3 * BOXW] + (float)dy * rp[4 * BOXW];
-                            const float h = (axis ? p.dphi[1] : p.dphi[2]) * rp[2 * BOXW] +
-                                            (axis ? 1.0f : 0.70710678118654752f) * gc * rest;
+                            const float h = edge_shift(p, axis, rp[0], rp[BOXW], rp[2 * BOXW], gc);
                             dv += k == 0 ? h : -h;
                         }
                     };
@@ -589,7 +770,8 @@ __global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_st
                         now.w = Codec<T>::dec(reinterpret_cast<const T *>(row + Cfg::RHO_BYTES)[(k * 8 + i - 1) * BOXW + col]);
                         // (the node's own shifts sum to 5 m dphi_1: an eighth per lane)
                         if (SPLIT)
-                            now.w += (k == 0 ? 0.625f : -0.625f) * p.dphi[1] * reinterpret_cast<const float *>(row)[2 * BOXW + col];
+                            now.w = __fmaf_rn((k == 0 ? 0.625f : -0.625f) * p.dphi[1],
+                                              reinterpret_cast<const float *>(row)[2 * BOXW + col], now.w);
                         if (wall_y && r == 0) across(row, hist[3 * 32]);   // stands for row -1
                     } else {
                         across(slots + ((p.ny - 1 - r0) % NSLOT) * Cfg::SLOT_BYTES, now);   // stands for row ny
@@ -617,9 +799,9 @@ __global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_st
                         }
                         if ((lane & 15) == 0 &&
                             !(OPEN && (side == 0 ? open_l : open_r || open_next || (open_next2 && outer)))) {
-                            ring_psi[at] = colour_field(p, rr, rb);
+                            ring_psi[at] = edge_colour(p, rr, rb);
                             if (HERMITE_SRC && outer == 0) {
-                                const float q = p.q_r * rr + p.q_b * rb, rho = rr + rb;
+                                const float q = __fmaf_rn(p.q_r, rr, __fmul_rn(p.q_b, rb)), rho = rr + rb;
                                 ring_qx[at] = q * (jx / rho + 0.5f * p.gx);
                                 ring_qy[at] = q * (jy / rho + 0.5f * p.gy);
                             }
@@ -741,55 +923,7 @@ __global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_st
                 }
                 Collided<f2> o;
                 collide_of<CV, SPLIT, f2>(p, K, Pc, cC, Fx, Fy, dQx, dQy, o);
-                const uint32_t ps_rho = (uint32_t)d.rho_plane * 4u, ps_dev = (uint32_t)d.dev_plane * (uint32_t)sizeof(T);
-                auto store = [&](char *qr, char *qd) {
-                    auto put = [&](char *q, f2 v) { pair_to(reinterpret_cast<float *>(q), v); };
-                    put(qr, Pc.rr);
-                    put(qr + ps_rho, Pc.rb);
-                    if (SPLIT) {
-                        put(qr + 2ull * ps_rho, o.m);
-                        put(qr + 3ull * ps_rho, o.gx);
-                        put(qr + 4ull * ps_rho, o.gy);
-                    }
-#pragma unroll
-                    for (int i = 0; i < 8; i++) {
-                        pair_to(reinterpret_cast<T *>(qd + (unsigned long long)ps_dev * i), o.r[i]);
-                        pair_to(reinterpret_cast<T *>(qd + (unsigned long long)ps_dev * (i + 8)), o.b[i]);
-                    }
-                };
-                if (both) store(out_rho, out_dev);
-                const bool per_x = !OPEN && p.bc_x == BC_PERIODIC;
-                if (per_x && (p.nx & 1) == 0) {
-                    // the pair's copies in the ghost columns of the other side (both on lattices
-                    // narrower than two ghosts)
-                    const long long nx = p.nx;
-                    if (x < Cfg::GMEM) store(out_rho + nx * 4, out_dev + nx * (long long)sizeof(T));
-                    if (x >= nx - Cfg::GMEM) store(out_rho - nx * 4, out_dev - nx * (long long)sizeof(T));
-                } else if (!both || (per_x && (x < Cfg::GMEM || x + 1 >= p.nx - Cfg::GMEM))) {
-                    // odd widths: single columns, in place (g = 0) or as ghost copies
-                    auto single = [&](int h, auto pick) {
-                        for (int g = both ? 1 : 0; g < 3; g++) {
-                            if (g == 1 && !(per_x && x + h < Cfg::GMEM)) continue;
-                            if (g == 2 && !(per_x && x + h >= p.nx - Cfg::GMEM)) continue;
-                            const long long to = h + (g == 0 ? 0 : (g == 1 ? p.nx : -p.nx));
-                            char *qr = out_rho + to * 4, *qd = out_dev + to * (long long)sizeof(T);
-                            *reinterpret_cast<float *>(qr) = pick(Pc.rr);
-                            *reinterpret_cast<float *>(qr + ps_rho) = pick(Pc.rb);
-                            if (SPLIT) {
-                                *reinterpret_cast<float *>(qr + 2ull * ps_rho) = pick(o.m);
-                                *reinterpret_cast<float *>(qr + 3ull * ps_rho) = pick(o.gx);
-                                *reinterpret_cast<float *>(qr + 4ull * ps_rho) = pick(o.gy);
-                            }
-#pragma unroll
-                            for (int i = 0; i < 8; i++) {
-                                *reinterpret_cast<T *>(qd + (unsigned long long)ps_dev * i) = Codec<T>::enc(pick(o.r[i]));
-                                *reinterpret_cast<T *>(qd + (unsigned long long)ps_dev * (i + 8)) = Codec<T>::enc(pick(o.b[i]));
-                            }
-                        }
-                    };
-                    single(0, [](f2 v) { return v.x; });
-                    if (both) single(1, [](f2 v) { return v.y; });
-                }
+                store_pair<T, SPLIT>(d, !OPEN && p.bc_x == BC_PERIODIC, x, both, out_rho, out_dev, Pc.rr, Pc.rb, o);
                 out_rho += d.rho_row * 4;
                 out_dev += d.dev_row * (long long)sizeof(T);
             }
@@ -822,6 +956,246 @@ __global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_st
     // for this grid's completion before it reads anything); a block that
     // triggered at its start does not trigger again
     if (!(flags & FUSED_EARLY_NEXT)) asm volatile("griddepcontrol.launch_dependents;");
+}
+
+// ------------------------------------------------------------- tile kernel
+
+// Launch shape: columns per tile (two per thread), at most so many rows (one warp each),
+// blocks per SM the registers are sized for.
+constexpr int TILE_W = 64;
+constexpr int TILE_MAX_ROWS = 8;
+constexpr int TILE_THREADS = 32 * TILE_MAX_ROWS;
+constexpr int TILE_MINB = 2;
+
+// Pulled state of the nodes (x, Y), (x + 1, Y) from global memory by the strip kernel's
+// sequence of operations (bit-identical to it).  Y lies in the lattice.
+template <typename T, int CV>
+__device__ __forceinline__ void pull_pair(const SimDesc &d, const Consts<f2> &K, int b, int x, int Y, PulledOf<f2> &P) {
+    constexpr bool SPLIT = SplitStore<T>::value;
+    const Phys &p = d.ph;
+    const int ny = p.ny, rs = (int)d.rho_plane, ds = (int)d.dev_plane;
+    const bool wall_y = p.bc_y == BC_WALL, bottom = wall_y && Y == 0, top = wall_y && Y == ny - 1;
+    const bool slip = (CV & CV_WET) && d.wet.slip;
+    const float *r = d.rho + b * d.rho_buf + d.ghost + x;
+    const T *v = reinterpret_cast<const T *>(d.dev) + b * d.dev_buf + d.ghost + x;
+    const float *rp = r + Y * d.rho_row;
+    const T *dp = v + Y * d.dev_row;
+    const f2 zero{0.0f, 0.0f};
+    const RowTerms R = row_terms<T>(rp, rs, dp, ds, K);
+    HalfPulled H;
+    f2 lo0, lo1, lo2, lo5, lo6, lo_h;
+    Step S = no_step();
+    if (!bottom) {
+        const int Ym = Y > 0 ? Y - 1 : ny - 1;
+        const RowTerms A = row_terms<T>(r + Ym * d.rho_row, rs, v + Ym * d.dev_row, ds, K);
+        lo0 = A.up[0], lo1 = A.up[1], lo2 = A.T2, lo5 = A.T5, lo6 = A.T6, lo_h = A.h_up;
+        S = step_of(K, A.own, R.own);
+    } else if (slip) {
+        lo0 = R.dn[0], lo1 = R.dn[1], lo2 = R.T4, lo5 = R.T8, lo6 = R.T7, lo_h = R.h_dn;
+    } else {
+        const WallTerms L = wall_row_terms<T>(rp, rs, dp, ds, K, p.dphi[1], 4, 7, 8, -1.0f);
+        lo0 = L.sum[0], lo1 = L.sum[1], lo2 = L.Ti, lo5 = L.Tj, lo6 = L.Tk, lo_h = L.h;
+    }
+    const f2 mquarter = lit<f2, LIT_MQUARTER>(), m15 = lit<f2, LIT_M3HALVES>();
+    H.own[0] = R.own[0], H.own[1] = R.own[1];
+    H.acc[0] = fmav(m15, S.r, R.mid[0] + lo0);
+    H.acc[1] = fmav(m15, S.b, R.mid[1] + lo1);
+    H.T1 = R.T1;
+    H.T3 = R.T3;
+    H.T2 = lo2 - S.sum;
+    H.T5 = fmav(mquarter, S.sum, lo5);
+    H.T6 = fmav(mquarter, S.sum, lo6);
+    H.h = SPLIT ? lo_h + R.h_mid : zero;
+    f2 dn0, dn1, T4, T7, T8, h_dn;
+    S = no_step();
+    if (!top) {
+        const int Yp = Y + 1 < ny ? Y + 1 : 0;
+        const RowTerms B = row_terms<T>(r + Yp * d.rho_row, rs, v + Yp * d.dev_row, ds, K);
+        dn0 = B.dn[0], dn1 = B.dn[1], T4 = B.T4, T7 = B.T7, T8 = B.T8, h_dn = B.h_dn;
+        S = step_of(K, H.own, B.own);
+    } else if (slip) {
+        dn0 = R.up[0], dn1 = R.up[1], T4 = R.T2, T7 = R.T6, T8 = R.T5, h_dn = R.h_up;
+    } else {
+        const WallTerms L = wall_row_terms<T>(rp, rs, dp, ds, K, p.dphi[1], 2, 5, 6, 1.0f);
+        dn0 = L.sum[0], dn1 = L.sum[1], T4 = L.Ti, T7 = L.Tj, T8 = L.Tk, h_dn = L.h;
+    }
+    close_node<SPLIT>(K, H, dn0, dn1, T4, T7, T8, h_dn, S, P);
+}
+
+// One step of a lattice whose tiles all fit on the chip at once: block (bx, by) owns 64 columns
+// by `ty` rows, one thread per two neighbouring columns.  Every thread pulls its nodes straight
+// from global memory; the nodes around the tile (colour field and q u only) are pulled by
+// blockDim.x / 32 - ty more warps at the same time (by the tile's own warps if there are none);
+// after one barrier the tile is collided and stored.  Periodic in x; any walls.
+//
+// Such a lattice is in L2 and a step is bound by its chain of dependent latencies: a strip's
+// block waits for a row load, makes at least five row passes with a barrier each, and stores;
+// a tile's block makes one pull, one barrier and one collision.  It loads and pulls the nodes
+// around its tile again (1.6 times the nodes with 4 rows), so where the strips' blocks are
+// all busy they win.  Microseconds a step, strips and tiles (FP32): 64 x 64 5.8 / 4.6, 200 x
+// 200 8.8 / 5.8, 140 x 280 9.9 / 5.8, 256 x 256 9.5 / 6.9, 512 x 256 11.1 / 8.9, 512 x 512
+// 12.7 / 16.1.
+template <typename T, int CV>
+__global__ void __launch_bounds__(TILE_THREADS, TILE_MINB) k_step_tile(const SimDesc *__restrict__ gd, int step_offset, int ty,
+                                                                        int *__restrict__ err) {
+    constexpr bool SPLIT = SplitStore<T>::value, WET = (CV & CV_WET) != 0;
+    constexpr bool HERMITE_SRC = (CV & CV_MRT) && (CV & CV_HERMITE);
+    constexpr int PITCH = TILE_W + 4;   // columns x0 - 2 .. x0 + TILE_W + 1
+    __shared__ SimDesc d;
+    __shared__ Consts<f2> K;
+    __shared__ __align__(16) float s_psi[(TILE_MAX_ROWS + 2) * PITCH];
+    __shared__ __align__(16) float s_qx[HERMITE_SRC ? (TILE_MAX_ROWS + 2) * PITCH : 4], s_qy[HERMITE_SRC ? (TILE_MAX_ROWS + 2) * PITCH : 4];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = blockDim.x >> 5;
+    {   // read while the previous step still runs
+        const int4 *src = reinterpret_cast<const int4 *>(gd);
+        int4 *dst = reinterpret_cast<int4 *>(&d);
+        for (int j = tid; j < (int)(sizeof(SimDesc) / 16); j += blockDim.x) dst[j] = __ldcv(src + j);
+    }
+    __syncthreads();
+    if (tid == 0) fill_consts(K, d.ph);
+    __syncthreads();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    long long t0 = d.t0, t_end = d.t_end;
+    if (step_offset == 0) {   // written between chunks of steps
+        t0 = __ldcv(&gd->t0);
+        t_end = __ldcv(&gd->t_end);
+    }
+    const Phys &p = d.ph;
+    const long long t = t0 + step_offset;
+    if (t >= t_end) return;   // this simulation has stopped
+    if (d.variant != CV || d.ghost != 8 || p.bc_x != BC_PERIODIC || ty < 1 || ty > TILE_MAX_ROWS || ty > warps) {
+        if (tid == 0) atomicOr(err, ERR_BADITEM);
+        return;
+    }
+    const int bsrc = (int)(t & 1), bdst = bsrc ^ 1;
+    const int x0 = blockIdx.x * TILE_W, y0 = blockIdx.y * ty, nx = p.nx, ny = p.ny;
+    const int rows = min(ty, ny - y0);
+    if (x0 >= nx || rows <= 0) return;
+    const bool wall_y = p.bc_y == BC_WALL;
+
+    PulledOf<f2> P;
+    // Where the tile borders on another 128-column strip (or the lattice's end) the strip
+    // kernel forms the columns beyond link by link: so does this one, so that a lattice has the
+    // same states in tiles, in strips and in a batch.
+    const bool edge_l = x0 % FUSED_W == 0, edge_r = (x0 + TILE_W) % FUSED_W == 0 || x0 + TILE_W >= nx;
+    const int w = min(TILE_W, nx - x0);
+    // pull the nodes of pair `q` (columns x0 + 2 q, + 1), row `row` of the tile, and share
+    // their colour field
+    auto node = [&](int q, int row, PulledOf<f2> &N) {
+        int Y = y0 + row;
+        const int x = x0 + 2 * q;
+        if ((q < 0 && edge_l) || (edge_r && 2 * q >= w)) return;
+        if (Y < 0 || Y >= ny) {
+            if (wall_y) return;
+            Y = Y < 0 ? Y + ny : Y - ny;
+        }
+        pull_pair<T, CV>(d, K, bsrc, x, Y, N);
+        const int at = (row + 1) * PITCH + 2 * q + 2;
+        auto share = [&](float *to, f2 v) {   // (an odd lattice's last pair: the second column is beyond)
+            if (edge_r && 2 * q + 1 >= w) to[at] = v.x;
+            else pair_to(to + at, v);
+        };
+        share(s_psi, colour_field_of(K, N.rr, N.rb));
+        if (HERMITE_SRC) {
+            f2 jx, jy;
+            momentum_of(N, jx, jy);
+            const f2 rho = N.rr + N.rb;
+            const f2 u = fmav(K.q_r, N.rr, K.q_b * N.rb);
+            share(s_qx, u * (f2{jx.x / rho.x, jx.y / rho.y} + K.hgx));
+            share(s_qy, u * (f2{jy.x / rho.x, jy.y / rho.y} + K.hgy));
+        }
+    };
+    const int halo = 2 * (TILE_W / 2 + 2) + 2 * rows;
+    const int own_warps = warps > ty ? ty : 0;   // with extra warps, those pull the halo
+    if (warp >= own_warps) {
+        PulledOf<f2> N;
+        for (int h = tid - own_warps * 32; h < halo; h += blockDim.x - own_warps * 32) {
+            const int side = TILE_W / 2 + 2;
+            if (h < 2 * side) node(h < side ? h - 1 : h - side - 1, h < side ? -1 : rows, N);
+            else node((h & 1) ? TILE_W / 2 : -1, (h - 2 * side) >> 1, N);
+        }
+        // nodes beside strip borders, one per half warp: sides, rows, next column out (the wall
+        // rows' psi needs those)
+        const int rs = (int)d.rho_plane, ds = (int)d.dev_plane;
+        const unsigned lanes = 0xffffu << (tid & 16);
+        const EdgeLink E(p, (tid & 7) + 1, (tid >> 3) & 1);
+        for (int e = (tid - own_warps * 32) >> 4; e < 4 * (rows + 2); e += (blockDim.x - own_warps * 32) >> 4) {
+            const int side = e & 1, outer = e >= 2 * (rows + 2), row = (e >> 1) - (outer ? rows + 2 : 0) - 1;
+            int Y = y0 + row;
+            if (!(side == 0 ? edge_l : edge_r) || (wall_y && (Y < 0 || Y >= ny))) continue;
+            if (outer && !(wall_y && (Y == 0 || Y == ny - 1))) continue;
+            Y = Y < 0 ? Y + ny : (Y >= ny ? Y - ny : Y);
+            const int col = side == 0 ? -1 - outer : w + outer;
+            const float *rp = d.rho + bsrc * d.rho_buf + d.ghost + x0 + col;
+            const T *dp = reinterpret_cast<const T *>(d.dev) + bsrc * d.dev_buf + d.ghost + x0 + col;
+            float s, dv, own_s, own_dv, psi, qx, qy;
+            E.own<T>(rp + Y * d.rho_row, rs, dp + Y * d.dev_row, ds, own_s, own_dv);
+            const int from = Y - E.cy;
+            if (wall_y && (from < 0 || from >= ny)) {
+                E.across<T>(rp + Y * d.rho_row, rs, dp + Y * d.dev_row, ds, WET && d.wet.slip, s, dv);
+            } else {
+                const int ys = from < 0 ? from + ny : (from >= ny ? from - ny : from);
+                E.source<T>(rp + ys * d.rho_row, rs, dp + ys * d.dev_row, ds, s, dv);
+            }
+            __syncwarp(lanes);
+            E.node<HERMITE_SRC>(lanes, s, dv, own_s, own_dv, psi, qx, qy);
+            if ((tid & 15) == 0) {
+                const int at = (row + 1) * PITCH + col + 2;
+                s_psi[at] = psi;
+                if (HERMITE_SRC) s_qx[at] = qx, s_qy[at] = qy;
+            }
+        }
+    }
+    const int x = x0 + 2 * lane, y = y0 + warp;
+    const bool mine = warp < rows;
+    if (mine) node(lane, warp, P);
+    __syncthreads();
+    if (wall_y && (y0 == 0 || y0 + rows == ny)) {   // the walls' colour field; their q u is zero
+        for (int side = 0; side < 2; side++) {
+            if (side == 0 ? y0 != 0 : y0 + rows != ny) continue;
+            const float *f = s_psi + (side == 0 ? 1 : rows) * PITCH + 2;
+            float *to = s_psi + (side == 0 ? 0 : rows + 1) * PITCH + 2;
+            for (int c = tid - 1; c <= w; c += blockDim.x) {
+                to[c] = wall_psi(p, x0 + c, [&](int X) { return f[X - x0]; });
+                if (HERMITE_SRC) {
+                    s_qx[(to - s_psi) + c] = 0.0f;
+                    s_qy[(to - s_psi) + c] = 0.0f;
+                }
+            }
+        }
+        __syncthreads();
+    }
+    if (!mine || x >= nx) return;
+
+    // 12 times the S2I4 gradient, in the strip kernel's order
+    const f2 four = lit<f2, LIT_FOUR>();
+    auto row_diff = [](f2 m, float west, float east) { return f2{m.y - west, east - m.x}; };
+    const float *c = s_psi + (warp + 1) * PITCH + 2 * lane + 2, *s = c - PITCH, *n = c + PITCH;
+    const f2 cC = pair_at(c), sC = pair_at(s), nC = pair_at(n);
+    const float cW = c[-1], cE = c[2], sW = s[-1], sE = s[2], nW = n[-1], nE = n[2];
+    f2 Fx = fmav(four, row_diff(cC, cW, cE), row_diff(nC, nW, nE) + row_diff(sC, sW, sE));
+    const f2 dC = nC - sC;
+    f2 Fy = fmav(four, dC, f2{dC.y + (nW - sW), (nE - sE) + dC.x});
+    f2 dQx{0.0f, 0.0f}, dQy{0.0f, 0.0f};
+    if (WET) {
+        contact_angle_adjust(d.wet, p, y, Fx.x, Fy.x);
+        contact_angle_adjust(d.wet, p, y, Fx.y, Fy.y);
+    }
+    if (HERMITE_SRC) {
+        const float *qx = s_qx + (c - s_psi), *qy = s_qy + (c - s_psi);
+        auto diff = [&](const float *q) { return f2{q[1] - q[-1], q[2] - q[0]}; };
+        dQx = fmav(four, diff(qx), diff(qx + PITCH) + diff(qx - PITCH));
+        const f2 dq = pair_at(qy + PITCH) - pair_at(qy - PITCH);
+        dQy = fmav(four, dq, f2{dq.y + (qy[PITCH - 1] - qy[-PITCH - 1]), (qy[PITCH + 2] - qy[-PITCH + 2]) + dq.x});
+    }
+    Collided<f2> o;
+    collide_of<CV, SPLIT, f2>(p, K, P, cC, Fx, Fy, dQx, dQy, o);
+    store_pair<T, SPLIT>(d, true, x, x + 1 < nx,
+                         reinterpret_cast<char *>(d.rho + bdst * d.rho_buf + (long long)y * d.rho_row + d.ghost + x),
+                         reinterpret_cast<char *>(reinterpret_cast<T *>(d.dev) + bdst * d.dev_buf + (long long)y * d.dev_row +
+                                                  d.ghost + x),
+                         P.rr, P.rb, o);
 }
 
 // --------------------------------------------------------- two-pass kernels
