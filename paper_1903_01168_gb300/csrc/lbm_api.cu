@@ -554,8 +554,9 @@ cudaError_t launch_tile_any(lbm_sim *s, int off) {
 // thread: 3 blocks of 5 warps, 2 of 7 or 4 of 4 per SM); strips (tile_rows 0) beyond, with open
 // ends, and where the caller set a plan.  Warps of their own for the nodes around the tile
 // shorten the step while they fit.  Microseconds a step with 2 rows in 5 warps, 4 in 7, 4 in 4
-// and strips: 200 x 200 5.8, 6.9, 6.8, 8.8; 256 x 256 9.7, 6.9, 7.4, 9.5; 512 x 256 14.8, 12.5,
-// 8.9, 11.1; 512 x 512 24.5, 23.3, 16.1, 12.7.
+// and strips (the tiles' own times have since come down by 0.2 to 0.7): 200 x 200 5.8, 6.9,
+// 6.8, 8.8; 256 x 256 9.7, 6.9, 7.4, 9.5; 512 x 256 14.8, 12.5, 8.9, 11.1; 512 x 512 24.5,
+// 23.3, 16.1, 12.7.
 void tile_shape(lbm_sim *s) {
     if (s->p.bc_x != LBM_BC_PERIODIC || s->p.plan != LBM_PLAN_AUTO || s->p.plan_rows != 0) return;
     int sms = 0;

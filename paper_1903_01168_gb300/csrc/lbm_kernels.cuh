@@ -449,19 +449,17 @@ struct EdgeLink {
             dv = __fadd_rn(dv, k == 0 ? h : -h);
         }
     }
-    // the link's source in its own row, the row of y - cy
+    // the link's source: in the row of y - cy (rp, dp at the node's column there) or, `wall`, in
+    // the node's own row: the node itself in the opposite direction, or (free slip) the row's
+    // neighbour in the mirrored one
     template <typename T>
-    __device__ __forceinline__ void source(const float *rp, int rs, const T *dp, int ds, float &s, float &dv) const {
-        value<T>(rp - cx, rs, dp - cx, ds, i, cx, cy, s, dv);
-    }
-    // source across a wall next to the row: the node itself in the opposite direction, or (free
-    // slip) the row's neighbour in the mirrored one
-    template <typename T>
-    __device__ __forceinline__ void across(const float *rp, int rs, const T *dp, int ds, bool slip, float &s, float &dv) const {
+    __device__ __forceinline__ void source(const float *rp, int rs, const T *dp, int ds, bool wall, bool slip, float &s,
+                                           float &dv) const {
         const int opp = i <= 4 ? ((i + 1) & 3) + 1 : ((i - 3) & 3) + 5;
         const int mir = i == 2 ? 4 : i == 4 ? 2 : i == 5 ? 8 : i == 8 ? 5 : i == 6 ? 7 : i == 7 ? 6 : i;
-        const int at = slip ? -cx : 0;
-        value<T>(rp + at, rs, dp + at, ds, slip ? mir : opp, slip ? cx : -cx, -cy, s, dv);
+        const bool back = wall && !slip;
+        const int at = back ? 0 : -cx;
+        value<T>(rp + at, rs, dp + at, ds, !wall ? i : (slip ? mir : opp), back ? -cx : cx, wall ? -cy : cy, s, dv);
     }
     // the node's own density and deviation (its own shifts sum to 5 m dphi_1: an eighth per lane)
     template <typename T>
@@ -1032,8 +1030,8 @@ __device__ __forceinline__ void pull_pair(const SimDesc &d, const Consts<f2> &K,
 // block waits for a row load, makes at least five row passes with a barrier each, and stores;
 // a tile's block makes one pull, one barrier and one collision.  It loads and pulls the nodes
 // around its tile again (1.6 times the nodes with 4 rows), so where the strips' blocks are
-// all busy they win.  Microseconds a step, strips and tiles (FP32): 64 x 64 5.8 / 4.6, 200 x
-// 200 8.8 / 5.8, 140 x 280 9.9 / 5.8, 256 x 256 9.5 / 6.9, 512 x 256 11.1 / 8.9, 512 x 512
+// all busy they win.  Microseconds a step, strips and tiles (FP32): 64 x 64 5.8 / 4.3, 200 x
+// 200 8.8 / 5.3, 140 x 280 9.9 / 5.3, 256 x 256 9.5 / 6.3, 512 x 256 11.1 / 8.7, 512 x 512
 // 12.7 / 16.1.
 template <typename T, int CV>
 __global__ void __launch_bounds__(TILE_THREADS, TILE_MINB) k_step_tile(const SimDesc *__restrict__ gd, int step_offset, int ty,
@@ -1115,15 +1113,19 @@ __global__ void __launch_bounds__(TILE_THREADS, TILE_MINB) k_step_tile(const Sim
             if (h < 2 * side) node(h < side ? h - 1 : h - side - 1, h < side ? -1 : rows, N);
             else node((h & 1) ? TILE_W / 2 : -1, (h - 2 * side) >> 1, N);
         }
-        // nodes beside strip borders, one per half warp: sides, rows, next column out (the wall
-        // rows' psi needs those)
+        // nodes beside strip borders, one per half warp: rows, next column out (the wall rows'
+        // psi needs those), of the one or two sides that are borders.  All fit in one round of
+        // the extra warps away from walls (with every second half warp left to the side that
+        // mostly is none, two rounds: 200 x 200 6.0 us a step, now 5.3).
         const int rs = (int)d.rho_plane, ds = (int)d.dev_plane;
         const unsigned lanes = 0xffffu << (tid & 16);
         const EdgeLink E(p, (tid & 7) + 1, (tid >> 3) & 1);
-        for (int e = (tid - own_warps * 32) >> 4; e < 4 * (rows + 2); e += (blockDim.x - own_warps * 32) >> 4) {
-            const int side = e & 1, outer = e >= 2 * (rows + 2), row = (e >> 1) - (outer ? rows + 2 : 0) - 1;
+        const int sides = (edge_l ? 1 : 0) + (edge_r ? 1 : 0), edges = sides * (rows + 2) * (wall_y ? 2 : 1);
+        for (int e = (tid - own_warps * 32) >> 4; e < edges; e += (blockDim.x - own_warps * 32) >> 4) {
+            const int j = sides == 2 ? e >> 1 : e, side = sides == 2 ? e & 1 : (edge_l ? 0 : 1);
+            const int outer = j >= rows + 2, row = j - (outer ? rows + 2 : 0) - 1;
             int Y = y0 + row;
-            if (!(side == 0 ? edge_l : edge_r) || (wall_y && (Y < 0 || Y >= ny))) continue;
+            if (wall_y && (Y < 0 || Y >= ny)) continue;
             if (outer && !(wall_y && (Y == 0 || Y == ny - 1))) continue;
             Y = Y < 0 ? Y + ny : (Y >= ny ? Y - ny : Y);
             const int col = side == 0 ? -1 - outer : w + outer;
@@ -1131,13 +1133,10 @@ __global__ void __launch_bounds__(TILE_THREADS, TILE_MINB) k_step_tile(const Sim
             const T *dp = reinterpret_cast<const T *>(d.dev) + bsrc * d.dev_buf + d.ghost + x0 + col;
             float s, dv, own_s, own_dv, psi, qx, qy;
             E.own<T>(rp + Y * d.rho_row, rs, dp + Y * d.dev_row, ds, own_s, own_dv);
-            const int from = Y - E.cy;
-            if (wall_y && (from < 0 || from >= ny)) {
-                E.across<T>(rp + Y * d.rho_row, rs, dp + Y * d.dev_row, ds, WET && d.wet.slip, s, dv);
-            } else {
-                const int ys = from < 0 ? from + ny : (from >= ny ? from - ny : from);
-                E.source<T>(rp + ys * d.rho_row, rs, dp + ys * d.dev_row, ds, s, dv);
-            }
+            int from = Y - E.cy;
+            const bool wall = wall_y && (from < 0 || from >= ny);
+            from = wall ? Y : (from < 0 ? from + ny : (from >= ny ? from - ny : from));
+            E.source<T>(rp + from * d.rho_row, rs, dp + from * d.dev_row, ds, wall, WET && d.wet.slip, s, dv);
             __syncwarp(lanes);
             E.node<HERMITE_SRC>(lanes, s, dv, own_s, own_dv, psi, qx, qy);
             if ((tid & 15) == 0) {
