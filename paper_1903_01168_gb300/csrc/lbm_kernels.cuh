@@ -4,15 +4,15 @@
 //                  colour gradient, omega_eff, collision, perturbation,
 //                  recolouring, store) in a single pass.  Each thread block owns
 //                  a strip of W columns and marches up a range of rows; source
-//                  rows (all 18 planes, with a ghost margin in x) arrive in a
-//                  ring of shared-memory slots by 3D TMA loads, so every stored
-//                  population is read from HBM once per step.  The colour field
-//                  of the row above is computed one row ahead into a small
-//                  shared ring, which is what the gradient stencil reads.
+//                  rows (all planes, with a margin in x) arrive in shared-memory
+//                  slots by TMA loads, so every stored population is read from
+//                  HBM once per step.
+//   k_step_tile    the same step, bit-identical, of a small lattice: a block owns a
+//                  tile and pulls it and the nodes around it from global memory.
 //   k_tp_moments / k_tp_collide
 //                  the same step as two plain node-parallel kernels with a
 //                  global scratch field (psi, q u) in between: the reference
-//                  GPU path, bit-identical to the fused one.
+//                  GPU path (equal to the fused one but for rounding).
 //   k_init, k_fields, k_diag, k_slug_profile, k_advance, k_set_times   support kernels.
 #pragma once
 
