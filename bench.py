@@ -46,8 +46,8 @@ FALLBACK_HBM_GBS = 6800.0
 # DRAM traffic of one k_step_fused launch on this workload from an ncu capture of
 # `dram__bytes_read.sum + dram__bytes_write.sum`, valid only for the kernel
 # sources with this hash; reported as null otherwise.
-NCU_TRAFFIC = {"sources_sha": "60141a825c48cb2c",
-               "bytes_per_launch": {0: 229121536 + 154410496, 1: 170580992 + 96698624, 2: 170623488 + 96513792}}
+NCU_TRAFFIC = {"sources_sha": "332506fc9a68d153",
+               "bytes_per_launch": {0: 228982784 + 153013504, 1: 170608128 + 95448320}}
 
 
 def kernel_sources_sha() -> str:
