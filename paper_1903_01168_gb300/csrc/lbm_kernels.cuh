@@ -517,8 +517,8 @@ struct EdgeLink {
 // node and with warps in flight, and FP32 also with DRAM (5.5 TB/s of halo, state and ghost
 // traffic).  Instructions issued per node of the 40-lattice sweep, one column a thread with
 // scalar arithmetic and separate pulls of three rows (before): FP32 681, BF16 973; now FP32
-// 400, BF16 488.  Microseconds a step before and now: sweep BF16 107.6 and 65.6, FP32 78.9
-// and 79.4; eight open channels of mixed storage 293 and 174.
+// 389, BF16 476.  Microseconds a step before and now: sweep BF16 107.6 and 63.1, FP32 78.9
+// and 78.3; eight open channels of mixed storage 293 and 173.
 template <typename T, int CV, int W, int NSLOT>
 __global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_step_fused(
     const SimDesc *__restrict__ descs, const WorkItem *__restrict__ items, const int *__restrict__ item_off,
