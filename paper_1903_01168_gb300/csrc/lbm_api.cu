@@ -543,10 +543,14 @@ int plan_blocks(int storage, int variant, long long nodes) {
 }
 
 cudaError_t launch_tile_any(lbm_sim *s, int off) {
+    const bool walls = s->p.bc_y == LBM_BC_WALL;
     switch (s->p.storage) {
-    case ST_F32: return tile_launch<float>(s->h.variant, s->d_desc, s->nx, s->ny, s->tile_rows, s->tile_warps, off, s->d_err, s->stream);
-    case ST_F16DEV: return tile_launch<__half>(s->h.variant, s->d_desc, s->nx, s->ny, s->tile_rows, s->tile_warps, off, s->d_err, s->stream);
-    default: return tile_launch<__nv_bfloat16>(s->h.variant, s->d_desc, s->nx, s->ny, s->tile_rows, s->tile_warps, off, s->d_err, s->stream);
+    case ST_F32: return tile_launch<float>(s->h.variant, s->d_desc, s->nx, s->ny, walls, s->tile_rows, s->tile_warps, off,
+                                         s->d_err, s->stream);
+    case ST_F16DEV: return tile_launch<__half>(s->h.variant, s->d_desc, s->nx, s->ny, walls, s->tile_rows, s->tile_warps, off,
+                                         s->d_err, s->stream);
+    default: return tile_launch<__nv_bfloat16>(s->h.variant, s->d_desc, s->nx, s->ny, walls, s->tile_rows, s->tile_warps, off,
+                                         s->d_err, s->stream);
     }
 }
 

@@ -51,7 +51,7 @@ cudaError_t fused_launch_cv(const SimDesc *descs, const WorkItem *items, const i
 }
 
 template <typename T, int CV>
-cudaError_t tile_launch_cv(const SimDesc *desc, int nx, int ny, int rows, int warps, int off, int *err, cudaStream_t st) {
+cudaError_t tile_launch_cv(const SimDesc *desc, int nx, int ny, bool walls, int rows, int warps, int off, int *err, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((nx + TILE_W - 1) / TILE_W), (unsigned)((ny + rows - 1) / rows));
     cfg.blockDim = dim3((unsigned)(32 * warps));
@@ -61,7 +61,8 @@ cudaError_t tile_launch_cv(const SimDesc *desc, int nx, int ny, int rows, int wa
     attr[0].val.programmaticStreamSerializationAllowed = LBM_FUSED_PDL;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_step_tile<T, CV>, desc, off, rows, err);
+    if (walls && nx % FUSED_W == TILE_W + 1) return cudaLaunchKernelEx(&cfg, k_step_tile<T, CV, true>, desc, off, rows, err);
+    return cudaLaunchKernelEx(&cfg, k_step_tile<T, CV, false>, desc, off, rows, err);
 }
 
 template <typename T, int CV>
@@ -91,7 +92,7 @@ cudaError_t twopass_launch(int variant, const SimDesc *desc, int off, float *aux
     template int lbm::fused_smem_cv<T, CV>();
 
 #define LBM_INSTANTIATE_TILE(T, CV)                                                                                  \
-    template cudaError_t lbm::tile_launch_cv<T, CV>(const lbm::SimDesc *, int, int, int, int, int, int *, cudaStream_t);
+    template cudaError_t lbm::tile_launch_cv<T, CV>(const lbm::SimDesc *, int, int, bool, int, int, int, int *, cudaStream_t);
 
 #define LBM_INSTANTIATE_TWOPASS(T) \
     template cudaError_t lbm::twopass_launch<T>(int, const lbm::SimDesc *, int, float *, long long, cudaStream_t);

@@ -38,7 +38,8 @@ template <typename T, int CV>
 cudaError_t fused_launch_cv(const SimDesc *descs, const WorkItem *items, const int *item_off, int n_blocks, int off,
                             int flags, int *err, cudaStream_t st);
 template <typename T, int CV>
-cudaError_t tile_launch_cv(const SimDesc *desc, int nx, int ny, int rows, int warps, int off, int *err, cudaStream_t st);
+cudaError_t tile_launch_cv(const SimDesc *desc, int nx, int ny, bool walls, int rows, int warps, int off, int *err,
+                           cudaStream_t st);
 template <typename T, int CV>
 const void *fused_kernel_cv();
 template <typename T, int CV>
@@ -72,12 +73,13 @@ cudaError_t fused_launch(int variant, const SimDesc *descs, const WorkItem *item
     LBM_DISPATCH_CV(variant, LBM_CALL_)
 #undef LBM_CALL_
 }
-// One step of one lattice, periodic in x, in tiles of `rows` rows, `warps` >= rows warps a block.
+// One step of one lattice, periodic in x (with walls or not), in tiles of `rows` rows, `warps` >=
+// rows warps a block.
 template <typename T>
-cudaError_t tile_launch(int variant, const SimDesc *desc, int nx, int ny, int rows, int warps, int off, int *err,
+cudaError_t tile_launch(int variant, const SimDesc *desc, int nx, int ny, bool walls, int rows, int warps, int off, int *err,
                         cudaStream_t st) {
     if (variant & CV_OPEN) return cudaErrorInvalidValue;
-#define LBM_CALL_(cv) return tile_launch_cv<T, (cv) & ~CV_OPEN>(desc, nx, ny, rows, warps, off, err, st)
+#define LBM_CALL_(cv) return tile_launch_cv<T, (cv) & ~CV_OPEN>(desc, nx, ny, walls, rows, warps, off, err, st)
     LBM_DISPATCH_CV(variant, LBM_CALL_)
 #undef LBM_CALL_
 }

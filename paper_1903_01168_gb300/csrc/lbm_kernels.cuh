@@ -1033,7 +1033,12 @@ __device__ __forceinline__ void pull_pair(const SimDesc &d, const Consts<f2> &K,
 // all busy they win.  Microseconds a step, strips and tiles (FP32): 64 x 64 5.8 / 4.3, 200 x
 // 200 8.8 / 5.3, 140 x 280 9.9 / 5.3, 256 x 256 9.5 / 6.3, 512 x 256 11.1 / 8.7, 512 x 512
 // 12.7 / 16.1.
-template <typename T, int CV>
+//
+// LONE: between walls, with one column right of the last full tile (nx = 65 mod 128).  The strip
+// kernel forms the column beyond that one link by link, and a wall's psi at the last column, a
+// corner of the full tile's gradients, is made from both: so does the full tile.  A variant of
+// its own, because the test in every lattice's kernel cost 64 x 64 and 140 x 280 1.6 %.
+template <typename T, int CV, bool LONE>
 __global__ void __launch_bounds__(TILE_THREADS, TILE_MINB) k_step_tile(const SimDesc *__restrict__ gd, int step_offset, int ty,
                                                                         int *__restrict__ err) {
     constexpr bool SPLIT = SplitStore<T>::value, WET = (CV & CV_WET) != 0;
@@ -1078,6 +1083,7 @@ __global__ void __launch_bounds__(TILE_THREADS, TILE_MINB) k_step_tile(const Sim
     // same states in tiles, in strips and in a batch.
     const bool edge_l = x0 % FUSED_W == 0, edge_r = (x0 + TILE_W) % FUSED_W == 0 || x0 + TILE_W >= nx;
     const int w = min(TILE_W, nx - x0);
+    const bool link_r = edge_r || (LONE && x0 + TILE_W + 1 == nx);
     // pull the nodes of pair `q` (columns x0 + 2 q, + 1), row `row` of the tile, and share
     // their colour field
     auto node = [&](int q, int row, PulledOf<f2> &N) {
@@ -1091,7 +1097,7 @@ __global__ void __launch_bounds__(TILE_THREADS, TILE_MINB) k_step_tile(const Sim
         pull_pair<T, CV>(d, K, bsrc, x, Y, N);
         const int at = (row + 1) * PITCH + 2 * q + 2;
         auto share = [&](float *to, f2 v) {   // (an odd lattice's last pair: the second column is beyond)
-            if (edge_r && 2 * q + 1 >= w) to[at] = v.x;
+            if (link_r && 2 * q + 1 >= w) to[at] = v.x;
             else pair_to(to + at, v);
         };
         share(s_psi, colour_field_of(K, N.rr, N.rb));
@@ -1120,13 +1126,14 @@ __global__ void __launch_bounds__(TILE_THREADS, TILE_MINB) k_step_tile(const Sim
         const int rs = (int)d.rho_plane, ds = (int)d.dev_plane;
         const unsigned lanes = 0xffffu << (tid & 16);
         const EdgeLink E(p, (tid & 7) + 1, (tid >> 3) & 1);
-        const int sides = (edge_l ? 1 : 0) + (edge_r ? 1 : 0), edges = sides * (rows + 2) * (wall_y ? 2 : 1);
+        const int sides = (edge_l ? 1 : 0) + (link_r ? 1 : 0), edges = sides * (rows + 2) * (wall_y ? 2 : 1);
         for (int e = (tid - own_warps * 32) >> 4; e < edges; e += (blockDim.x - own_warps * 32) >> 4) {
             const int j = sides == 2 ? e >> 1 : e, side = sides == 2 ? e & 1 : (edge_l ? 0 : 1);
             const int outer = j >= rows + 2, row = j - (outer ? rows + 2 : 0) - 1;
             int Y = y0 + row;
             if (wall_y && (Y < 0 || Y >= ny)) continue;
             if (outer && !(wall_y && (Y == 0 || Y == ny - 1))) continue;
+            if (LONE && !outer && side == 1 && !edge_r) continue;   // the lone column itself: a pair's
             Y = Y < 0 ? Y + ny : (Y >= ny ? Y - ny : Y);
             const int col = side == 0 ? -1 - outer : w + outer;
             const float *rp = d.rho + bsrc * d.rho_buf + d.ghost + x0 + col;
