@@ -13,6 +13,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <vector>
 
@@ -78,13 +79,16 @@ struct lbm_sim {
     int n_items = 0, n_blocks = 0;
     int launch_flags = 0;   // fused-kernel flags of the plan (FUSED_EARLY_NEXT)
     int tile_rows = 0, tile_warps = 0;   // > 0: lbm_step runs the tile kernel in this shape
-    int *d_err = nullptr;
     float *d_aux = nullptr;      // two-pass scratch field
-    double *d_part = nullptr;    // diagnostic partials, the sums of both passes, block ticket
+    // Results on the device, one allocation: diagnostic partials, the sums of both passes, the
+    // error word (8 bytes), the slug profile (2 nx), the block ticket.  Either read-back is one
+    // copy of what lies on one side of the error word, and allocates nothing: a first read-back
+    // that got pinned memory of its own waited for the other streams of the device.
+    double *d_part = nullptr;
+    double *d_sums = nullptr, *d_prof = nullptr;   // into d_part: sums, profile
+    int *d_err = nullptr;                          // into d_part
+    unsigned *d_ticket = nullptr;                  // into d_part
     int diag_blocks = 0;
-    double *d_prof = nullptr;    // slug profile (2 nx), kept from the first call
-    double *h_read = nullptr;    // pinned host buffer of the diagnostics and the profile
-    size_t h_read_bytes = 0;
     cudaGraphExec_t graph = nullptr;
     int graph_steps = 0;
     bool has_center = false;
@@ -625,24 +629,24 @@ void launch_read_pops(lbm_sim *s, int g, double *out) {
 }
 
 template <typename T, bool H>
-void launch_diag_t(lbm_sim *s, double *fin, unsigned *ticket) {
+void launch_diag_t(lbm_sim *s) {
     k_diag<T, H, 0><<<s->diag_blocks, DIAG_THREADS, 0, s->stream>>>(s->d_desc, s->t, s->has_center, s->cx, s->cy, s->d_part,
-                                                                    fin, ticket);
+                                                                    s->d_sums, s->d_ticket);
     k_diag<T, H, 1><<<s->diag_blocks, DIAG_THREADS, 0, s->stream>>>(s->d_desc, s->t, s->has_center, s->cx, s->cy, s->d_part,
-                                                                    fin, ticket);
+                                                                    s->d_sums, s->d_ticket);
 }
 
 template <typename T>
-void launch_diag_s(lbm_sim *s, double *fin, unsigned *ticket) {
-    if (s->h.variant & CV_HERMITE) launch_diag_t<T, true>(s, fin, ticket);
-    else launch_diag_t<T, false>(s, fin, ticket);
+void launch_diag_s(lbm_sim *s) {
+    if (s->h.variant & CV_HERMITE) launch_diag_t<T, true>(s);
+    else launch_diag_t<T, false>(s);
 }
 
-void launch_diag(lbm_sim *s, double *fin, unsigned *ticket) {
+void launch_diag(lbm_sim *s) {
     switch (s->p.storage) {
-    case ST_F32: launch_diag_s<float>(s, fin, ticket); break;
-    case ST_F16DEV: launch_diag_s<__half>(s, fin, ticket); break;
-    default: launch_diag_s<__nv_bfloat16>(s, fin, ticket); break;
+    case ST_F32: launch_diag_s<float>(s); break;
+    case ST_F16DEV: launch_diag_s<__half>(s); break;
+    default: launch_diag_s<__nv_bfloat16>(s); break;
     }
 }
 
@@ -754,23 +758,6 @@ lbm_status check_err_word(lbm_sim *s, int *d_err) {
     return err_word_status(s, h);
 }
 
-// The simulation's pinned read-back buffer, at least `bytes` long (kept until lbm_destroy:
-// a pageable copy is staged by the driver and synchronises on its own).
-lbm_status read_buffer(lbm_sim *s, size_t bytes) {
-    if (s->h_read_bytes >= bytes) return LBM_OK;
-    if (s->h_read) cudaFreeHost(s->h_read);
-    s->h_read = nullptr;
-    s->h_read_bytes = 0;
-    if (cudaMallocHost(reinterpret_cast<void **>(&s->h_read), bytes) != cudaSuccess) {
-        cudaGetLastError();
-        s->h_read = nullptr;
-        set_err(s->err, "pinned read-back buffer of %zu bytes failed", bytes);
-        return LBM_ENOMEM;
-    }
-    s->h_read_bytes = bytes;
-    return LBM_OK;
-}
-
 // Launch `n` steps of a single simulation directly (no graph).
 lbm_status step_direct(lbm_sim *s, long n) {
     for (long j = 0; j < n; j++) {
@@ -869,7 +856,7 @@ lbm_status create_common(int nx, int ny, const lbm_params *p, void *buf, size_t 
     s->h.rho = reinterpret_cast<float *>(s->pop);
     s->h.dev = static_cast<char *>(s->pop) + rho_region_bytes(nx, ny, p->storage);
     if (encode_tmap(s) != LBM_OK) return fail(LBM_ECUDA);
-    if (cudaMalloc(&s->d_desc, sizeof(SimDesc)) != cudaSuccess || cudaMalloc(&s->d_err, sizeof(int)) != cudaSuccess) {
+    if (cudaMalloc(&s->d_desc, sizeof(SimDesc)) != cudaSuccess) {
         set_err(s->err, "cudaMalloc of descriptor failed");
         return fail(LBM_ENOMEM);
     }
@@ -899,14 +886,17 @@ lbm_status create_common(int nx, int ny, const lbm_params *p, void *buf, size_t 
         return fail(LBM_ENOMEM);
     }
     s->diag_blocks = std::min(grid_for((long long)nn, DIAG_THREADS), DIAG_BLOCKS);
-    if (cudaMalloc(&s->d_part, ((size_t)s->diag_blocks + 3) * DIAG_NQ * sizeof(double)) != cudaSuccess) {
+    const size_t parts = (size_t)s->diag_blocks * DIAG_NQ, after = 1 + 2 * (size_t)nx + 1;   // error word, profile, ticket
+    if (cudaMalloc(&s->d_part, (parts + DIAG_SUMS + after) * sizeof(double)) != cudaSuccess) {
         set_err(s->err, "cudaMalloc of diagnostic scratch failed");
         return fail(LBM_ENOMEM);
     }
+    s->d_sums = s->d_part + parts;
+    s->d_err = reinterpret_cast<int *>(s->d_sums + DIAG_SUMS);
+    s->d_prof = s->d_sums + DIAG_SUMS + 1;
+    s->d_ticket = reinterpret_cast<unsigned *>(s->d_prof + 2 * (size_t)nx);
     if (cudaMemcpyAsync(s->d_desc, &s->h, sizeof(SimDesc), cudaMemcpyHostToDevice, s->stream) != cudaSuccess ||
-        cudaMemsetAsync(s->d_err, 0, sizeof(int), s->stream) != cudaSuccess ||
-        cudaMemsetAsync(s->d_part + (size_t)(s->diag_blocks + 2) * DIAG_NQ, 0, DIAG_NQ * sizeof(double), s->stream) !=
-            cudaSuccess ||
+        cudaMemsetAsync(s->d_err, 0, after * sizeof(double), s->stream) != cudaSuccess ||
         cudaMemsetAsync(s->pop, 0, s->pop_bytes, s->stream) != cudaSuccess ||
         cudaStreamSynchronize(s->stream) != cudaSuccess) {
         set_err(s->err, "initial uploads failed: %s", cudaGetErrorString(cudaGetLastError()));
@@ -1119,16 +1109,12 @@ lbm_status lbm_diagnostics(lbm_sim *s, lbm_diag *out) {
     memset(out, 0, sizeof(*out));
     // both passes, one copy, one wait: the second pass takes the first one's sums from
     // device memory
-    constexpr size_t SUMS = 2 * DIAG_NQ;
-    lbm_status st = read_buffer(s, (SUMS + 1) * sizeof(double));
-    if (st != LBM_OK) return st;
-    double *fin = s->d_part + (size_t)s->diag_blocks * DIAG_NQ;
-    launch_diag(s, fin, reinterpret_cast<unsigned *>(fin + SUMS));
+    double h[DIAG_SUMS + 1];   // the error word last
+    launch_diag(s);
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(s->h_read, fin, SUMS * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
-    CK(cudaMemcpyAsync(s->h_read + SUMS, s->d_err, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+    CK(cudaMemcpyAsync(h, s->d_sums, sizeof(h), cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
-    const double *h = s->h_read, *h1 = h + DIAG_NQ;
+    const double *h1 = h + DIAG_NQ;
     out->t = s->t;
     out->mass_r = h[0];
     out->mass_b = h[1];
@@ -1146,8 +1132,8 @@ lbm_status lbm_diagnostics(lbm_sim *s, lbm_diag *out) {
     out->p_out = h1[3] > 0 ? h1[2] / h1[3] : 0.0;
     out->dp = out->p_in - out->p_out;
     int e = 0;
-    memcpy(&e, s->h_read + SUMS, sizeof(int));
-    st = err_word_status(s, e);
+    memcpy(&e, h + DIAG_SUMS, sizeof(int));
+    const lbm_status st = err_word_status(s, e);
     if (st != LBM_OK) return st;
     if (out->nonfinite > 0) {
         set_err(s->err, "%lld non-finite nodes at t = %lld", out->nonfinite, s->t);
@@ -1159,20 +1145,18 @@ lbm_status lbm_diagnostics(lbm_sim *s, lbm_diag *out) {
 lbm_status lbm_slug_geometry(lbm_sim *s, lbm_slug *out, double *gas) {
     if (!s || !out) return LBM_EINVAL;
     memset(out, 0, sizeof(*out));
-    const size_t nx = (size_t)s->nx, bytes = 2 * nx * sizeof(double);
-    lbm_status st = read_buffer(s, bytes + sizeof(double));
-    if (st != LBM_OK) return st;
-    if (!s->d_prof) CK(cudaMalloc(&s->d_prof, bytes));
+    const size_t nx = (size_t)s->nx;
+    const std::unique_ptr<double[]> h(new double[1 + 2 * nx]);   // the error word first; not cleared
     launch_slug_profile(s, s->d_prof);
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(s->h_read, s->d_prof, bytes, cudaMemcpyDeviceToHost, s->stream));
-    CK(cudaMemcpyAsync(s->h_read + 2 * nx, s->d_err, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+    CK(cudaMemcpyAsync(h.get(), s->d_err, (1 + 2 * nx) * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
     out->t = s->t;
-    slug_from_profile(s->h_read, s->h_read + nx, s->nx, s->ny, s->p.bc_x == LBM_BC_PERIODIC, out);
-    if (gas) memcpy(gas, s->h_read, nx * sizeof(double));
+    const double *g = h.get() + 1;
+    slug_from_profile(g, g + nx, s->nx, s->ny, s->p.bc_x == LBM_BC_PERIODIC, out);
+    if (gas) memcpy(gas, g, nx * sizeof(double));
     int e = 0;
-    memcpy(&e, s->h_read + 2 * nx, sizeof(int));
+    memcpy(&e, h.get(), sizeof(int));
     return err_word_status(s, e);
 }
 
@@ -1213,11 +1197,8 @@ void lbm_destroy(lbm_sim *s) {
     cudaFree(s->d_desc);
     cudaFree(s->d_items);
     cudaFree(s->d_off);
-    cudaFree(s->d_err);
     cudaFree(s->d_aux);
     cudaFree(s->d_part);
-    cudaFree(s->d_prof);
-    if (s->h_read) cudaFreeHost(s->h_read);
     if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
     delete s;
 }

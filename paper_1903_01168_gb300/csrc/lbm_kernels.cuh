@@ -1462,6 +1462,7 @@ __global__ void k_read_pops(const SimDesc *__restrict__ dp, long long t, double 
 
 // ---------------------------------------------------------------- diagnostics
 constexpr int DIAG_NQ = 16;        // slots of a block's partial sums
+constexpr int DIAG_SUMS = 2 * DIAG_NQ;   // of both passes
 constexpr int DIAG_THREADS = 256;
 constexpr int DIAG_BLOCKS = 152 * 2;   // at most: all resident at 128 registers a thread, one reduction each
 
