@@ -532,7 +532,7 @@ def main():
                    "autotune": (None if tuned is None else
                                 {"seconds": round(tune_s, 2), "row_overhead": tuned["row_overhead"],
                                  "plan": {0: "auto", 1: "balanced", 2: "split"}[tuned["plan"]],
-                                 "plan_rows": {k: v for k, v in tuned["classes"].items() if v != 8}}),
+                                 "plan_rows": {k: v for k, v in tuned["classes"].items() if v != 0}}),
                    "l2": f"inputs larger than L2: {STORED_BYTES[storage] * nodes / 1e6:.0f} MB of state "
                          f"touched per step",
                    "parallelism":

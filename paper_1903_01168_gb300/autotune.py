@@ -8,7 +8,8 @@ lattices may even run faster on the node-parallel two-pass kernel.  The shortest
 segment a lattice may be cut into (`plan_rows`) and the kernel are therefore
 chosen per size class by timing, not by rule: every candidate runs a few steps on
 the device, timed with CUDA events on the stream it runs on, and the fastest
-wins.
+wins.  The library's own choice (plan_rows 0: tiles for a small lattice alone, short
+segments where 8-row ones would leave blocks idle) is always one of them.
 
 A size class is (storage type, collision, equilibrium, nx and ny rounded up to
 powers of two).  Tuning a single lattice times it alone; tuning for a batch
@@ -30,10 +31,10 @@ import os
 
 from . import lbm as L
 
-PLAN_CANDIDATES = (8, 16, 32, 64)
-ROW_OVERHEAD_CANDIDATES = (0.0, 0.5, 1.0, 2.0, 4.0)
-# (plan kind, row overhead) pairs timed on a whole batch
-PLAN_OPTION_CANDIDATES = tuple((L.LBM_PLAN_SPLIT, o) for o in (0.0, 1.0, 4.0)) + \
+PLAN_CANDIDATES = (0, 8, 16, 32, 64)      # 0: the library's default
+ROW_OVERHEAD_CANDIDATES = (0.0, 0.5, 1.0, 2.0, 4.0, 8.0)
+# (plan kind, row overhead) pairs timed on a whole batch, the library's default first
+PLAN_OPTION_CANDIDATES = ((L.LBM_PLAN_AUTO, -1.0),) + tuple((L.LBM_PLAN_SPLIT, o) for o in (0.0, 1.0, 4.0, 8.0)) + \
     tuple((L.LBM_PLAN_BALANCED, o) for o in ROW_OVERHEAD_CANDIDATES)
 
 
@@ -129,7 +130,8 @@ class Autotuner:
         Coordinate descent: start from the default plan for every member; for
         each size class (largest share of nodes first) try every candidate
         plan_rows for that class's members with the others fixed, and keep one
-        that is at least `gain` faster.  Then time the plan kinds and row costs
+        that is at least `gain` faster than the plan so far, timed again beside it (one
+        slow timing of the default must not decide).  Then time the plan kinds and row costs
         (`tune_plan`) with the chosen plan_rows.  The members' states advance:
         re-initialise them afterwards.  Returns {"classes": {class: plan_rows},
         "member_plan_rows": [...], "plan": kind, "row_overhead": r, "ms": t}; the
@@ -153,14 +155,15 @@ class Autotuner:
         for k in sorted(weight, key=weight.get, reverse=True):
             pick = 0
             for r in self.candidates:
-                if r == 8:
-                    continue   # the default (0 = 8) is the incumbent
-                trial = [r if kk == k else v for kk, v in zip(keys, rows)]
-                t = timed(trial)
+                if r == 0:
+                    continue   # the default is the first incumbent
+                t = timed([r if kk == k else v for kk, v in zip(keys, rows)])
+                if t < best * (1.0 - gain):
+                    best = min(best, timed(rows))
                 if t < best * (1.0 - gain):
                     best, pick = t, r
-            rows = [pick if kk == k else v for kk, v in zip(keys, rows)]
-            chosen[k] = pick if pick else 8
+                    rows = [r if kk == k else v for kk, v in zip(keys, rows)]
+            chosen[k] = pick
             self.table["batch-" + k] = {"kernel": L.LBM_KERNEL_FUSED, "plan_rows": chosen[k]}
         (kind, ovh), timings = tune_plan(sims, steps=steps, member_plan_rows=rows)
         return {"classes": chosen, "member_plan_rows": rows, "plan": kind, "row_overhead": ovh,
