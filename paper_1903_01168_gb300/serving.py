@@ -169,13 +169,15 @@ class Server:
 
     def __init__(self, budget_bytes: float = 150e9, chunk: int = 500, max_chunk: int = 4000,
                  graph_steps: int = 32, max_active_nodes: int | None = 8_000_000, priority: str = "arrival",
-                 plan: int = L.LBM_PLAN_BALANCED, row_overhead: float | None = 4.0,
+                 plan: int = L.LBM_PLAN_AUTO, row_overhead: float | None = None,
                  clock=time.perf_counter, sleep=time.sleep):
         """plan / row_overhead: the batch work plan (LBM_PLAN_*) and the planner's
-        fixed cost of a strip row in busy warps.  The active sets are uneven (lattices
-        of 64 to 256 rows whose last strips are often narrow): the balanced plan with a
-        row cost of 4 busy warps ran 10-20 lattice batches 19 % (FP32) to 44 % (FP16)
-        faster than the split plan."""
+        fixed cost of a strip row in quarters of a full strip's width (None: the
+        library's).  The active sets are uneven (lattices of 64 to 256 rows whose last
+        strips are often narrow).  On open-channel sets the library's plan ran faster
+        than the balanced one with a row cost of 4: 10 FP32 lattices 304 us a step
+        against 369, 10 FP16 ones 155 against 182, 8 of mixed storage 186 against
+        197, 4 of mixed storage 93 against 104."""
         if priority not in self.PRIORITIES:
             raise ValueError(f"priority must be one of {self.PRIORITIES}")
         self.priority = priority
