@@ -118,8 +118,8 @@ typedef struct {
     int kernel;          /* lbm_kernel */
     int plan_rows;       /* fused kernel work plan: fewest rows of this lattice a thread
                             block marches over in one segment (0 = 8, or 1 to 2
-                            where that would leave resident blocks idle); larger values trade parallelism for less halo
-                            re-reading.  Never changes results, only speed (the
+                            where that would leave resident blocks idle); larger
+                            values trade parallelism for less halo re-reading.  Never changes results, only speed (the
                             Python autotuner picks it per lattice size class). */
     int plan;            /* lbm_plan_kind of this lattice's own launches (0 = AUTO) */
     int wall_slip;       /* walls (bc_y = WALL): 0 no slip (halfway bounce-back), 1 free
@@ -337,9 +337,10 @@ lbm_status lbm_batch_create_ex(lbm_sim *const *sims, int n, const lbm_batch_opts
 /* Host only (no device call): the work plan a batch of n lattices of sizes
  * nx[i] x ny[i] would get with these options and max_blocks resident thread
  * blocks (the library queries that number from the device; pass any positive
- * value here).  plan_rows: NULL or the members' plan_rows (opts->member_plan_rows
- * takes precedence); 0 stands for 8 rows here, also where a batch would take fewer.  Sets *n_items and *n_blocks and writes the first
- * `capacity` items as 6 ints each: member, first column, width (<= 128), first
+ * value here; large FP32 batches are planned for 5/6 of them).  plan_rows: the members'
+ * plan_rows (opts->member_plan_rows takes precedence), 0 as in lbm_params; NULL for both:
+ * 8 rows for every member.  Sets *n_items and *n_blocks and writes the first `capacity`
+ * items as 6 ints each: member, first column, width (<= 128), first
  * row, end row, thread block.  Items of one block are listed in the order the
  * block runs them.  LBM_EINVAL for invalid sizes or options. */
 lbm_status lbm_plan_preview(const int *nx, const int *ny, const int *plan_rows, int n, const lbm_batch_opts *opts,

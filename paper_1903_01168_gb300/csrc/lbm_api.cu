@@ -1229,7 +1229,7 @@ lbm_status lbm_plan_preview(const int *nx, const int *ny, const int *plan_rows, 
         strips_of(strips, i, nx[i], ny[i], pr);
     }
     const double ovh = opts->row_overhead < 0.0f ? DEFAULT_ROW_OVERHEAD : (double)opts->row_overhead;
-    default_pieces(strips, max_blocks, false);
+    default_pieces(strips, max_blocks, plan_rows || opts->member_plan_rows);
     const Plan P = make_plan(strips, opts->plan, opts->rows_per_item, max_blocks, ovh);
     *n_items = (int)P.items.size();
     *n_blocks = P.blocks;

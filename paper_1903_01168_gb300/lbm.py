@@ -331,7 +331,8 @@ def lbm_batch_create(sims, rows_per_item: int = 0, row_overhead: float | None = 
 def lbm_plan_preview(sizes, max_blocks: int, plan: int = LBM_PLAN_AUTO, row_overhead: float | None = None,
                      rows_per_item: int = 0, plan_rows=None) -> tuple[int, np.ndarray]:
     """Host-only preview of a batch's work plan: (blocks, items) with items an
-    (n_items, 6) int array of member, x0, width, first row, end row, block."""
+    (n_items, 6) int array of member, x0, width, first row, end row, block.
+    plan_rows: the members' plan_rows, 0 the library's choice (None: 8 for every member)."""
     n = len(sizes)
     nx = (ctypes.c_int * n)(*[int(a) for a, _ in sizes])
     ny = (ctypes.c_int * n)(*[int(b) for _, b in sizes])
