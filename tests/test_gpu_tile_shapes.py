@@ -50,3 +50,27 @@ def test_lone_column_beside_the_last_tile(flow, nx, ny, storage):
     for model in MODELS.values():
         kw = dict(FLOWS[flow], **model, storage=storage)
         assert states(nx, ny, L.LBM_PLAN_AUTO, (1, 1, 3), **kw) == states(nx, ny, L.LBM_PLAN_SPLIT, (1, 1, 3), **kw)
+
+
+def launch_shape(nx, ny):
+    """Rows and warps of a tile's block by the library's rule: the first shape whose tiles are all
+    resident (None: strips)."""
+    torch = pytest.importorskip("torch")
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for rows, warps, per_sm in ((2, 5, 3), (4, 7, 2), (4, 4, 4)):
+        if -(-nx // 64) * -(-ny // rows) <= per_sm * sms:
+            return rows, warps
+    return None
+
+
+@pytest.mark.parametrize("storage", [L.LBM_F32, L.LBM_F16DEV, L.LBM_BF16DEV])
+@pytest.mark.parametrize("nx,ny,shape", [(201, 139, (2, 5)), (300, 203, (4, 7)), (193, 301, (4, 7)), (509, 254, (4, 4)),
+                                         (449, 301, (4, 4)), (1025, 131, (4, 4)), (450, 313, None)])
+def test_every_launch_shape(nx, ny, shape, storage):
+    """Ragged sizes of every shape: last columns odd, a last row of tiles of one to three rows; five
+    direct launches and a graph of 32 with one more."""
+    assert launch_shape(nx, ny) == shape
+    for flow in FLOWS.values():
+        for model in MODELS.values():
+            kw = dict(flow, **model, storage=storage)
+            assert states(nx, ny, L.LBM_PLAN_AUTO, (5, 33), **kw) == states(nx, ny, L.LBM_PLAN_SPLIT, (5, 33), **kw)
