@@ -1263,13 +1263,11 @@ lbm_status lbm_batch_create_ex(lbm_sim *const *sims, int n, const lbm_batch_opts
                 return LBM_EINVAL;
             }
     *out = nullptr;
-    long long strip_rows = 0;
     for (int i = 0; i < n; i++) {
         if (!sims[i] || sims[i]->dev != sims[0]->dev) {
             set_err(g_create_err, "batch members must exist and share a device");
             return LBM_EINVAL;
         }
-        strip_rows += (long long)((sims[i]->nx + FUSED_W - 1) / FUSED_W) * sims[i]->ny;
     }
     lbm_batch *b = new lbm_batch();
     b->sims.assign(sims, sims + n);

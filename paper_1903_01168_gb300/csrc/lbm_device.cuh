@@ -55,8 +55,8 @@ enum : int { ERR_TIMEOUT = 1, ERR_BADITEM = 2, ERR_ALIGN = 4 };
 // streams markedly slower).  Rows keep `ghost` columns on each side (periodic
 // copies in x).  The tensor
 // maps come first so that they keep the 64-byte alignment TMA requires.
-// Per-simulation constants the node operators read; kernels copy this struct
-// into registers once.
+// Per-simulation constants the node operators read (the step kernels keep them in
+// shared memory, the node-parallel ones in registers).
 struct Phys {
     int nx, ny, bc_x, bc_y;
     int inlet_mode, inlet_period_r, inlet_period_b, inlet_layer;
@@ -74,8 +74,8 @@ struct Phys {
     float u_in_r, u_in_b, p_out;
 };
 
-// Wetting-wall parameters (free slip, static contact angle).  Kept out of Phys:
-// the fused kernel, which holds Phys in registers, never runs such lattices.
+// Wetting-wall parameters (free slip, static contact angle), read by the CV_WET
+// variants of the step kernels and by the node-parallel kernels.
 struct Wetting {
     int slip;                  // walls: 0 no slip, 1 free slip
     int on;                    // 1: contact-angle adjustment of F next to the walls
@@ -129,7 +129,7 @@ constexpr int AUX_FIELDS = 5;
 // Compile-time variants of the step kernels: bit 0 = MRT (else BGK), bit 1 =
 // Hermite equilibrium (with the U^k source when combined with MRT), bit 2 =
 // wetting walls (free-slip links and the contact-angle adjustment of F; without
-// it walls are no-slip and the fused kernel keeps fewer registers), bit 3 =
+// it walls are no-slip), bit 3 =
 // inlet / outlet columns in x (else periodic in x).  The fused kernel of a
 // periodic lattice carries no open-column code: its mere presence in the loop
 // cost the periodic sweep 2 %.
@@ -156,9 +156,6 @@ __host__ __device__ constexpr int CY(int i) { return (i == 2 || i == 5 || i == 6
 __host__ __device__ constexpr int OPP(int i) { return i == 0 ? 0 : (i <= 4 ? ((i + 1) & 3) + 1 : ((i - 3) & 3) + 5); }
 __host__ __device__ constexpr int C2(int i) { return CX(i) * CX(i) + CY(i) * CY(i); }
 __host__ __device__ constexpr float WT(int i) { return C2(i) == 0 ? 4.0f / 9.0f : (C2(i) == 1 ? 1.0f / 9.0f : 1.0f / 36.0f); }
-__host__ __device__ constexpr float BP(int i) { return C2(i) == 0 ? -4.0f / 27.0f : (C2(i) == 1 ? 2.0f / 27.0f : 5.0f / 108.0f); }
-// S2I4 weights xi_i, Eq. (eq:colorGradient)
-__host__ __device__ constexpr float XI(int i) { return C2(i) == 0 ? 0.0f : (C2(i) == 1 ? 1.0f / 3.0f : 1.0f / 12.0f); }
 
 static_assert(OPP(1) == 3 && OPP(2) == 4 && OPP(3) == 1 && OPP(4) == 2, "opposites");
 static_assert(OPP(5) == 7 && OPP(6) == 8 && OPP(7) == 5 && OPP(8) == 6, "opposites");
@@ -342,30 +339,14 @@ struct Link {
 
 __host__ __device__ constexpr int MIRY(int i) { return i == 2 ? 4 : i == 4 ? 2 : i == 5 ? 8 : i == 8 ? 5 : i == 6 ? 7 : i == 7 ? 6 : i; }
 
-// Link sets a pull is compiled for: no-slip walls only (the fused kernel, which
-// never runs lattices with wetting walls: their extra logic would cost the hot
-// loop registers on every row), or no-slip and free-slip walls (all others).
-constexpr int LINKS_NOSLIP = 1, LINKS_ALL = 2;
-
-template <int LINKS>
 __device__ __forceinline__ Link link_of(const Phys &p, int slip, int i, int x, int y, bool bottom, bool top) {
     const bool wall = (CY(i) > 0 && bottom) || (CY(i) < 0 && top);
     if (!wall) return Link{x - CX(i), y - CY(i), i, false};
-    if (LINKS == LINKS_NOSLIP) return Link{x, y, OPP(i), true};
     const int xs = x - CX(i);
     if (slip && (p.bc_x == BC_PERIODIC || (xs >= 0 && xs < p.nx))) return Link{xs, y, MIRY(i), CX(i) == 0};
     return Link{x, y, OPP(i), true};
 }
 
-// Pull the pre-collision populations of node (x, y) at time t (Eq. (eq:subop4)):
-// N^k_i(x) = phi^k_i rho_k(x - c_i) + d^k_i(x - c_i), with halfway bounce-back
-// across walls (the node's own opposite population) and two-phase Zou-He on
-// the inlet / outlet columns (Sec. 2.5).  The loader provides
-//   ld.rho(k, xs, ys), ld.dev(k, i, xs, ys)   (i = 1..8)
-// of a source node; xs may be -1 or nx (ghost column); ys is one of y-1, y, y+1
-// NOT wrapped (the loader wraps periodic rows); y itself may lie one row
-// outside [0, ny) on a periodic lattice.  With have_rho the node's new colour
-// densities are already known (rr_new, rb_new) and are not recomputed.
 // pull_node for the split form (16-bit storage), away from open columns.  The
 // loader gives the stored residual r^k_i and the shift h_i of the split form
 // (d^r_i = r^r_i + h_i, d^b_i = r^b_i - h_i).  The shifts cancel in the colour-blind
@@ -373,7 +354,7 @@ __device__ __forceinline__ Link link_of(const Phys &p, int slip, int i, int x, i
 //   sum_i h_i(source of i) - sum_i h_i(x),
 // where the node's own sum is 4 m (dphi_1 + dphi_2) (the flux parts cancel in
 // opposite pairs).
-template <int LINKS, class Loader>
+template <class Loader>
 __device__ __forceinline__ void pull_node_split(const Phys &p, const Loader &ld, int x, int y, bool have_rho,
                                                 float rr_new, float rb_new, Pulled &P) {
     const bool wall_y = p.bc_y == BC_WALL;
@@ -387,7 +368,7 @@ __device__ __forceinline__ void pull_node_split(const Phys &p, const Loader &ld,
     float T[9], acc[2] = {0.0f, 0.0f}, hsum = 0.0f;
 #pragma unroll
     for (int i = 1; i < 9; i++) {
-        const Link lk = link_of<LINKS>(p, ld.slip, i, x, y, bottom, top);
+        const Link lk = link_of(p, ld.slip, i, x, y, bottom, top);
         const int xs = lk.xs, ys = lk.ys, ii = lk.ii;
         float ti = 0.0f;
 #pragma unroll
@@ -422,14 +403,23 @@ __device__ __forceinline__ void pull_node_split(const Phys &p, const Loader &ld,
     P.e[0] = -e0;
 }
 
-template <bool HERMITE, int LINKS, class Loader>
-__device__ __forceinline__ void pull_node_rows(const Phys &p, const Loader &ld, int x, int y, long long t,
-                                               bool have_rho, float rr_new, float rb_new, Pulled &P) {
+// Pull the pre-collision populations of node (x, y) at time t (Eq. (eq:subop4)):
+// N^k_i(x) = phi^k_i rho_k(x - c_i) + d^k_i(x - c_i), with halfway bounce-back
+// across walls (the node's own opposite population) and two-phase Zou-He on
+// the inlet / outlet columns (Sec. 2.5).  The loader provides
+//   ld.rho(k, xs, ys), ld.dev(k, i, xs, ys)   (i = 1..8)
+// of a source node; xs may be -1 or nx (ghost column); ys is one of y-1, y, y+1
+// NOT wrapped (the loader wraps periodic rows); y itself may lie one row
+// outside [0, ny) on a periodic lattice.  With have_rho the node's new colour
+// densities are already known (rr_new, rb_new) and are not recomputed.
+template <bool HERMITE, class Loader>
+__device__ __forceinline__ void pull_node(const Phys &p, const Loader &ld, int x, int y, long long t,
+                                          bool have_rho, float rr_new, float rb_new, Pulled &P) {
     const bool wall_y = p.bc_y == BC_WALL;
     const bool open_col = p.bc_x == BC_INOUT && (x == 0 || x == p.nx - 1);
     const bool bottom = wall_y && y == 0, top = wall_y && y == p.ny - 1;
     if (Loader::SPLIT && !open_col) {
-        pull_node_split<LINKS>(p, ld, x, y, have_rho, rr_new, rb_new, P);
+        pull_node_split(p, ld, x, y, have_rho, rr_new, rb_new, P);
         return;
     }
     float s[2][9], dl[2][9], own_rho[2];
@@ -438,21 +428,9 @@ __device__ __forceinline__ void pull_node_rows(const Phys &p, const Loader &ld, 
         own_rho[k] = ld.rho(k, x, y);
 #pragma unroll
         for (int i = 1; i < 9; i++) {
-            if (LINKS == LINKS_NOSLIP) {
-                // constant plane offsets in both branches (no run-time direction index)
-                const bool bounce = (CY(i) > 0 && bottom) || (CY(i) < 0 && top);
-                if (bounce) {
-                    s[k][i] = own_rho[k];
-                    dl[k][i] = ld.dev(k, OPP(i), x, y);
-                } else {
-                    s[k][i] = ld.rho(k, x - CX(i), y - CY(i));
-                    dl[k][i] = ld.dev(k, i, x - CX(i), y - CY(i));
-                }
-            } else {
-                const Link lk = link_of<LINKS>(p, ld.slip, i, x, y, bottom, top);
-                s[k][i] = lk.self ? own_rho[k] : ld.rho(k, lk.xs, lk.ys);
-                dl[k][i] = ld.dev(k, lk.ii, lk.xs, lk.ys);
-            }
+            const Link lk = link_of(p, ld.slip, i, x, y, bottom, top);
+            s[k][i] = lk.self ? own_rho[k] : ld.rho(k, lk.xs, lk.ys);
+            dl[k][i] = ld.dev(k, lk.ii, lk.xs, lk.ys);
         }
     }
     if (!open_col) {
@@ -507,120 +485,6 @@ __device__ __forceinline__ void pull_node_rows(const Phys &p, const Loader &ld, 
     for (int i = 0; i < 9; i++) P.e[i] = (nr[i] + nb[i]) - (rr * p.phi_r[C2(i)] + rb * p.phi_b[C2(i)]);
 }
 
-// Pull with every kind of wall link.
-template <bool HERMITE, class Loader>
-__device__ __forceinline__ void pull_node(const Phys &p, const Loader &ld, int x, int y, long long t,
-                                          bool have_rho, float rr_new, float rb_new, Pulled &P) {
-    pull_node_rows<HERMITE, LINKS_ALL>(p, ld, x, y, t, have_rho, rr_new, rb_new, P);
-}
-
-// Moments of the pulled node (x, y) without forming its populations: the new
-// colour densities
-//   rho_k' = rho_k(x) + sum_{i>=1} [phi^k_i (s^k_i - rho_k(x)) + delta^k_i - d^k_i(x)]
-// (s, delta: density and deviation of the source of direction i) and, with
-// NEED_J, the momentum sum_i c_i N_i summed over opposite pairs.  Open columns
-// take the full pull.
-template <bool HERMITE, bool NEED_J, int LINKS, class Loader>
-__device__ __forceinline__ void pull_moments_rows(const Phys &p, const Loader &ld, int x, int y, long long t,
-                                                  float &rr, float &rb, float &jx, float &jy) {
-    if (p.bc_x == BC_INOUT && (x == 0 || x == p.nx - 1)) {
-        Pulled P;
-        pull_node<HERMITE>(p, ld, x, y, t, false, 0.0f, 0.0f, P);
-        rr = P.rr;
-        rb = P.rb;
-        jx = (P.e[1] - P.e[3]) + (P.e[5] - P.e[7]) + (P.e[8] - P.e[6]);
-        jy = (P.e[2] - P.e[4]) + (P.e[5] - P.e[7]) + (P.e[6] - P.e[8]);
-        return;
-    }
-    const bool wall_y = p.bc_y == BC_WALL;
-    const bool bottom = wall_y && y == 0, top = wall_y && y == p.ny - 1;
-    if (Loader::SPLIT) {
-        // split form: residual differences per colour, one shift sum for both
-        // (as in pull_node_split)
-        float n[2][9], acc[2], own[2];
-        float hsum = 0.0f;
-        own[0] = ld.rho(0, x, y);
-        own[1] = ld.rho(1, x, y);
-#pragma unroll
-        for (int i = 1; i < 9; i++) {
-            const Link lk = link_of<LINKS>(p, ld.slip, i, x, y, bottom, top);
-            const int xs = lk.xs, ys = lk.ys, ii = lk.ii;
-#pragma unroll
-            for (int k = 0; k < 2; k++) {
-                const float sv = lk.self ? own[k] : ld.rho(k, xs, ys);
-                n[k][i] = phi_k(p, k, C2(i)) * (sv - own[k]) + ld.res(k, ii, xs, ys);
-            }
-            hsum += ld.shift(ii, xs, ys);
-        }
-        const float dh = hsum - ld.own_shift_sum(x, y);
-#pragma unroll
-        for (int k = 0; k < 2; k++) {
-            float a = 0.0f;
-#pragma unroll
-            for (int i = 1; i < 9; i++) a += n[k][i] - ld.res(k, i, x, y);
-            acc[k] = own[k] + (k == 0 ? a + dh : a - dh);
-        }
-        rr = acc[0];
-        rb = acc[1];
-        if (NEED_J) {
-            // colour-blind momentum: the shifts cancel between the colours
-            float m[9];
-#pragma unroll
-            for (int i = 1; i < 9; i++) m[i] = n[0][i] + n[1][i];
-            jx = (m[1] - m[3]) + (m[5] - m[7]) + (m[8] - m[6]);
-            jy = (m[2] - m[4]) + (m[5] - m[7]) + (m[6] - m[8]);
-        } else {
-            jx = jy = 0.0f;
-        }
-        return;
-    }
-    float n[2][9];   // n[k][i] = N^k_i - phi^k_i rho_k(x) for i >= 1 (small)
-    float acc[2];
-#pragma unroll
-    for (int k = 0; k < 2; k++) {
-        const float own = ld.rho(k, x, y);
-        float a = 0.0f;
-#pragma unroll
-        for (int i = 1; i < 9; i++) {
-            float sv, dv;
-            if (LINKS == LINKS_NOSLIP) {
-                const bool bounce = (CY(i) > 0 && bottom) || (CY(i) < 0 && top);
-                if (bounce) {
-                    sv = own;
-                    dv = ld.dev(k, OPP(i), x, y);
-                } else {
-                    sv = ld.rho(k, x - CX(i), y - CY(i));
-                    dv = ld.dev(k, i, x - CX(i), y - CY(i));
-                }
-            } else {
-                const Link lk = link_of<LINKS>(p, ld.slip, i, x, y, bottom, top);
-                sv = lk.self ? own : ld.rho(k, lk.xs, lk.ys);
-                dv = ld.dev(k, lk.ii, lk.xs, lk.ys);
-            }
-            n[k][i] = phi_k(p, k, C2(i)) * (sv - own) + dv;
-            a += n[k][i] - ld.dev(k, i, x, y);
-        }
-        acc[k] = own + a;
-    }
-    rr = acc[0];
-    rb = acc[1];
-    if (NEED_J) {
-        float m[9];
-#pragma unroll
-        for (int i = 1; i < 9; i++) m[i] = n[0][i] + n[1][i];
-        jx = (m[1] - m[3]) + (m[5] - m[7]) + (m[8] - m[6]);
-        jy = (m[2] - m[4]) + (m[5] - m[7]) + (m[6] - m[8]);
-    } else {
-        jx = jy = 0.0f;
-    }
-}
-
-template <bool HERMITE, bool NEED_J, class Loader>
-__device__ __forceinline__ void pull_moments(const Phys &p, const Loader &ld, int x, int y, long long t,
-                                             float &rr, float &rb, float &jx, float &jy) {
-    pull_moments_rows<HERMITE, NEED_J, LINKS_ALL>(p, ld, x, y, t, rr, rb, jx, jy);
-}
-
 // Pre-collision populations of both colours of node (x, y) at time t in FP64
 // (boundary conditions included), for state export.
 template <bool HERMITE, class Loader>
@@ -631,7 +495,7 @@ __device__ __forceinline__ void pull_populations(const Phys &p, const Loader &ld
     double sr = 0.0, sb = 0.0;
 #pragma unroll
     for (int i = 1; i < 9; i++) {
-        const Link lk = link_of<LINKS_ALL>(p, ld.slip, i, x, y, bottom, top);
+        const Link lk = link_of(p, ld.slip, i, x, y, bottom, top);
         const int xs = lk.xs, ys = lk.ys, ii = lk.ii;
         nr[i] = (double)p.phi_r[C2(i)] * ld.rho(0, xs, ys) + ld.dev(0, ii, xs, ys);
         nb[i] = (double)p.phi_b[C2(i)] * ld.rho(1, xs, ys) + ld.dev(1, ii, xs, ys);
@@ -1041,11 +905,6 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t by
 
 __device__ __forceinline__ void mbar_inval(uint64_t *bar) {
     asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-// Plain arrival (no transaction bytes): completes the phase of a count-1 barrier.
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-    asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
