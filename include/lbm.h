@@ -337,7 +337,7 @@ lbm_status lbm_batch_create_ex(lbm_sim *const *sims, int n, const lbm_batch_opts
 /* Host only (no device call): the work plan a batch of n lattices of sizes
  * nx[i] x ny[i] would get with these options and max_blocks resident thread
  * blocks (the library queries that number from the device; pass any positive
- * value here; large FP32 batches are planned for 5/6 of them).  plan_rows: the members'
+ * value here; large FP32 batches are planned for 5/6 or 4/6 of them).  plan_rows: the members'
  * plan_rows (opts->member_plan_rows takes precedence), 0 as in lbm_params; NULL for both:
  * 8 rows for every member.  Sets *n_items and *n_blocks and writes the first `capacity`
  * items as 6 ints each: member, first column, width (<= 128), first

@@ -314,20 +314,23 @@ struct Plan {
     int blocks = 0;
 };
 
-// Launch flags for a plan run as the only launch of each step: a plan of one piece per
-// block, all within an eighth of the same height, lets the next step launch early (its
-// blocks then land on whichever SMs free first, which only matters where the pieces
-// differ): 1000 x 301 MRT, whose last strip is narrower, 19.8 us a step without and 16.5
-// with.  So does a plan that leaves half the resident blocks' slots free.
-int plan_flags(const Plan &P, int resident) {
-    if (P.blocks * 2 <= resident) return FUSED_EARLY_NEXT;
-    if (P.items.empty() || (int)P.items.size() != P.blocks) return 0;
+// One piece per block, all within an eighth of the same height.
+bool even_pieces(const Plan &P) {
+    if (P.items.empty() || (int)P.items.size() != P.blocks) return false;
     int lo = 1 << 30, hi = 0;
     for (const WorkItem &it : P.items) {
         lo = std::min(lo, it.yb - it.ya);
         hi = std::max(hi, it.yb - it.ya);
     }
-    return hi - lo <= std::max(1, hi / 8) ? FUSED_EARLY_NEXT : 0;
+    return hi - lo <= std::max(1, hi / 8);
+}
+
+// Launch flags for a plan run as the only launch of each step: a plan of even pieces lets
+// the next step launch early (its blocks then land on whichever SMs free first, which only
+// matters where the pieces differ): 1000 x 301 MRT, whose last strip is narrower, 19.8 us a
+// step without and 16.5 with.  So does a plan that leaves half the resident blocks' slots free.
+int plan_flags(const Plan &P, int resident) {
+    return P.blocks * 2 <= resident || even_pieces(P) ? FUSED_EARLY_NEXT : 0;
 }
 
 constexpr int MIN_PIECE = 8;   // default shortest row range worth a 4-row halo
@@ -535,15 +538,48 @@ int resident_blocks(int storage, int variant) {
     return cache[storage][variant];
 }
 
-// Thread blocks a plan over `nodes` nodes is made for: all resident ones (6 per SM), which
-// hides the latency of the row passes best, except on FP32 lattices far beyond L2.  Those
-// are held by DRAM, and 5 per SM load fewer halo rows: 4096 x 512 FP32 62.3 -> 57.9 us a
-// step, 8192 x 256 open 71.5 -> 66.8, 2048 x 2048 120.6 -> 113; at 1024 x 1024 (151 MB of
-// state, mostly in L2) 6 per SM are faster (29.2 against 30.1), and FP16 storage is at every
-// size (2048 x 1280: 61.8 with 6 per SM, 69 with 5).
+// Thread blocks a plan over `nodes` nodes is made for: all resident ones (6 per SM: every
+// variant compiles to 165 to 168 registers), which hides the latency of the row passes best,
+// except on FP32 lattices far beyond L2.  Those are held by DRAM, and 5 per SM load fewer halo
+// rows: 4096 x 512 FP32 62.3 -> 57.9 us a step, 8192 x 256 open 71.5 -> 66.8; at 1024 x 1024
+// (151 MB of state, mostly in L2) 6 per SM are faster (29.2 against 30.1), and FP16 storage is
+// at every size (2048 x 1280: 61.8 with 6 per SM, 69 with 5).
 int plan_blocks(int storage, int variant, long long nodes) {
     const int all = resident_blocks(storage, variant);
     return storage == ST_F32 && nodes >= 1500000 ? std::max(1, all * 5 / 6) : all;
+}
+
+struct PlanFor {
+    Plan plan;
+    int flags;   // launch flags
+};
+
+// The plan of one launch per step over strips of `nodes` nodes; `periodic`: all of them in both
+// directions.
+//
+// Even pieces of a BGK lattice in FP32 without wetting or open columns go to 4 blocks per SM,
+// each step launched after the one before it, where that leaves less than a twentieth of those
+// blocks without a piece.  The taller pieces load fewer halo rows again; with early launches
+// the waiting blocks take the free slots, so that SMs get unequal shares, which costs more.
+// us a step with 5 per SM and early launches, 4 with and 4 without them: 2000 x 2000 111.6,
+// 118.5, 107.2; 2048 x 2048 115.5, 117, 102.8; 256 x 8192 64.3, 63.4, 57.7; 4096 x 2048 222, 226,
+// 195.  Below two million nodes it gains nothing (4096 x 384 44.6, 48.3, 44.1); between walls
+// 5 per SM are as good up to 4 million (2000 x 2000 109.6 and 111.3, 4096 x 2048 214 and 201).
+// MRT, wetting and open lattices are bound by more instructions: MRT 2000 x 2000 109.4 and
+// 110.9, with the Hermite source 155.5 and 186 (with early launches), wet 4096 x 512 58.5 and 60.1.
+PlanFor plan_for(std::vector<StripRef> &strips, int kind, int rows_per_item, int storage, int variant, long long nodes,
+                 bool periodic, double row_overhead) {
+    const int all = resident_blocks(storage, variant), blocks = plan_blocks(storage, variant, nodes);
+    default_pieces(strips, blocks, true);
+    PlanFor r{make_plan(strips, kind, rows_per_item, blocks, row_overhead), 0};
+    r.flags = plan_flags(r.plan, all);
+    const bool plain = !(variant & (CV_WET | CV_OPEN | CV_MRT));
+    if (storage == ST_F32 && plain && rows_per_item == 0 && nodes >= (periodic ? 2000000 : 5000000) && even_pieces(r.plan)) {
+        const int fewer = std::max(1, all * 4 / 6);
+        Plan P = make_plan(strips, kind, 0, fewer, row_overhead);
+        if (even_pieces(P) && (long long)P.blocks * 20 >= (long long)fewer * 19) r = {std::move(P), 0};
+    }
+    return r;
 }
 
 cudaError_t launch_tile_any(lbm_sim *s, int off) {
@@ -863,12 +899,12 @@ lbm_status create_common(int nx, int ny, const lbm_params *p, void *buf, size_t 
     {
         std::vector<StripRef> strips;
         strips_of(strips, 0, nx, ny, p->plan_rows);
-        const int blocks = plan_blocks(p->storage, variant_of(p), (long long)nx * ny);
-        default_pieces(strips, blocks, true);
-        Plan P = make_plan(strips, p->plan, 0, blocks, DEFAULT_ROW_OVERHEAD);
+        const PlanFor r = plan_for(strips, p->plan, 0, p->storage, variant_of(p), (long long)nx * ny,
+                                   p->bc_x == LBM_BC_PERIODIC && p->bc_y == LBM_BC_PERIODIC, DEFAULT_ROW_OVERHEAD);
+        const Plan &P = r.plan;
         s->n_items = (int)P.items.size();
         s->n_blocks = P.blocks;
-        s->launch_flags = plan_flags(P, resident_blocks(p->storage, variant_of(p)));
+        s->launch_flags = r.flags;
         if (cudaMalloc(&s->d_items, P.items.size() * sizeof(WorkItem)) != cudaSuccess ||
             cudaMalloc(&s->d_off, P.off.size() * sizeof(int)) != cudaSuccess ||
             cudaMemcpy(s->d_items, P.items.data(), P.items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice) !=
@@ -1288,17 +1324,18 @@ lbm_status lbm_batch_create_ex(lbm_sim *const *sims, int n, const lbm_batch_opts
         for (int cv = 0; cv < N_VARIANTS; cv++) {
             std::vector<StripRef> strips;
             long long nodes = 0;
+            bool periodic = true;
             for (int i = 0; i < n; i++)
                 if (sims[i]->p.storage == st && sims[i]->h.variant == cv) {
                     nodes += (long long)sims[i]->nx * sims[i]->ny;
+                    periodic = periodic && sims[i]->p.bc_x == LBM_BC_PERIODIC && sims[i]->p.bc_y == LBM_BC_PERIODIC;
                     strips_of(strips, i, sims[i]->nx, sims[i]->ny,
                               opts->member_plan_rows ? opts->member_plan_rows[i] : sims[i]->p.plan_rows);
                 }
             if (strips.empty()) continue;
-            const int blocks = plan_blocks(st, cv, nodes);
-            default_pieces(strips, blocks, true);
-            Plan P = make_plan(strips, opts->plan, rows_per_item, blocks, row_overhead);
-            lbm_batch::Group g{st, cv, (int)items.size(), (int)offs.size(), P.blocks, plan_flags(P, resident_blocks(st, cv))};
+            PlanFor r = plan_for(strips, opts->plan, rows_per_item, st, cv, nodes, periodic, row_overhead);
+            Plan &P = r.plan;
+            lbm_batch::Group g{st, cv, (int)items.size(), (int)offs.size(), P.blocks, r.flags};
             for (int &o : P.off) o += g.item0;
             items.insert(items.end(), P.items.begin(), P.items.end());
             offs.insert(offs.end(), P.off.begin(), P.off.end());
