@@ -1541,7 +1541,7 @@ __global__ void __launch_bounds__(DIAG_THREADS, 2) k_diag(const SimDesc *__restr
             const float f2 = fx * fx + fy * fy;
             bool inside = f2 < in2, outside = f2 > out2;
             // FP32 rounding of the coordinates and of the squares: 1e-5 of the lattice and of r^2
-            const float slack = 1e-5f * f2 + 4e-6f * (float)(nx + ny) * (fx + fy + 1.0f);
+            const float slack = 1e-5f * f2 + 4e-6f * (float)(nx + ny) * (fabsf(fx) + fabsf(fy) + 1.0f);
             if (!(fabsf(f2 - in2) > slack && fabsf(f2 - out2) > slack)) {
                 double dx = fabs(x - cx), dy = fabs(y - cy);
                 if (p.bc_x == BC_PERIODIC) dx = fmin(dx, nx - dx);
