@@ -15,6 +15,7 @@
 #include <cstring>
 #include <memory>
 #include <mutex>
+#include <new>
 #include <vector>
 
 #include "lbm.h"
@@ -1182,7 +1183,8 @@ lbm_status lbm_slug_geometry(lbm_sim *s, lbm_slug *out, double *gas) {
     if (!s || !out) return LBM_EINVAL;
     memset(out, 0, sizeof(*out));
     const size_t nx = (size_t)s->nx;
-    const std::unique_ptr<double[]> h(new double[1 + 2 * nx]);   // the error word first; not cleared
+    const std::unique_ptr<double[]> h(new (std::nothrow) double[1 + 2 * nx]);   // the error word first; not cleared
+    if (!h) { set_err(s->err, "out of host memory for the profile of %zu columns", nx); return LBM_ENOMEM; }
     launch_slug_profile(s, s->d_prof);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(h.get(), s->d_err, (1 + 2 * nx) * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
