@@ -564,18 +564,26 @@ struct PlanFor {
 // the waiting blocks take the free slots, so that SMs get unequal shares, which costs more.
 // us a step with 5 per SM and early launches, 4 with and 4 without them: 2000 x 2000 111.6,
 // 118.5, 107.2; 2048 x 2048 115.5, 117, 102.8; 256 x 8192 64.3, 63.4, 57.7; 4096 x 2048 222, 226,
-// 195.  Below two million nodes it gains nothing (4096 x 384 44.6, 48.3, 44.1); between walls
-// 5 per SM are as good up to 4 million (2000 x 2000 109.6 and 111.3, 4096 x 2048 214 and 201).
-// MRT, wetting and open lattices are bound by more instructions: MRT 2000 x 2000 109.4 and
-// 110.9, with the Hermite source 155.5 and 186 (with early launches), wet 4096 x 512 58.5 and 60.1.
+// 195.  Below two million nodes it gains nothing (4096 x 384 44.6, 48.3, 44.1), with a narrower
+// last strip below three (2500 x 820 59.0 and 59.8); between walls 5 per SM are as good up to
+// four (2000 x 2000 109.6 and 111.3, 4096 x 2048 214 and 201).  Odd widths, whose nodes are stored
+// one by one, and MRT, wetting and open lattices are bound by more instructions: 3681 x 570 67.8
+// and 74.9, MRT 2000 x 2000 109.4 and 110.9, with the Hermite source 155.5 and 186 (with early
+// launches), wet 4096 x 512 58.5 and 60.1.
 PlanFor plan_for(std::vector<StripRef> &strips, int kind, int rows_per_item, int storage, int variant, long long nodes,
                  bool periodic, double row_overhead) {
     const int all = resident_blocks(storage, variant), blocks = plan_blocks(storage, variant, nodes);
     default_pieces(strips, blocks, true);
     PlanFor r{make_plan(strips, kind, rows_per_item, blocks, row_overhead), 0};
     r.flags = plan_flags(r.plan, all);
-    const bool plain = !(variant & (CV_WET | CV_OPEN | CV_MRT));
-    if (storage == ST_F32 && plain && rows_per_item == 0 && nodes >= (periodic ? 2000000 : 5000000) && even_pieces(r.plan)) {
+    bool full = true, pairs = true;   // strips of 128 columns, of whole pairs of columns
+    for (const auto &s : strips) {
+        full = full && s.w == FUSED_W;
+        pairs = pairs && s.w % 2 == 0;
+    }
+    const bool plain = !(variant & (CV_WET | CV_OPEN | CV_MRT)) && pairs;
+    const long long least = !periodic ? 5000000 : (full ? 2000000 : 3000000);
+    if (storage == ST_F32 && plain && rows_per_item == 0 && nodes >= least && even_pieces(r.plan)) {
         const int fewer = std::max(1, all * 4 / 6);
         Plan P = make_plan(strips, kind, 0, fewer, row_overhead);
         if (even_pieces(P) && (long long)P.blocks * 20 >= (long long)fewer * 19) r = {std::move(P), 0};

@@ -16,14 +16,13 @@ MRT_HERMITE = dict(collision=L.LBM_MRT, equilibrium=L.LBM_EQ_HERMITE)
 @pytest.mark.parametrize("nx,ny,per_sm,kw", [
     (256, 8192, 4, dict()), (2048, 2048, 4, dict()), (2048, 2048, 4, dict(equilibrium=L.LBM_EQ_HERMITE)),
     (4096, 2048, 4, WALLS), (2048, 1280, 5, WALLS), (2048, 2048, 5, MRT_HERMITE), (2048, 2048, 5, dict(collision=L.LBM_MRT)), (4096, 2048, 5, SLIP),
-    (8192, 256, 5, dict()), (1024, 1792, 5, dict()), (2048, 2048, 6, dict(storage=L.LBM_F16DEV))])
+    (2000, 2000, 4, dict()), (2047, 2048, 5, dict()), (2496, 820, 5, dict()), (8192, 256, 5, dict()), (1024, 1792, 5, dict()), (2048, 2048, 6, dict(storage=L.LBM_F16DEV))])
 def test_blocks_of_a_large_lattice(nx, ny, per_sm, kw):
     torch = pytest.importorskip("torch")
-    strips = nx // 128
-    blocks = per_sm * torch.cuda.get_device_properties(0).multi_processor_count
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
     with L.Simulation(nx, ny, gamma=2.0, **kw) as s:
         b = L.Batch([s])
-        assert b.items == strips * (blocks // strips)
+        assert -(-b.items // sms) == per_sm       # one piece per block
         b.close()
 
 
