@@ -78,7 +78,7 @@ struct lbm_sim {
     WorkItem *d_items = nullptr;
     int *d_off = nullptr;        // per-block item ranges of the plan
     int n_items = 0, n_blocks = 0;
-    int launch_flags = 0;   // fused-kernel flags of the plan (FUSED_EARLY_NEXT)
+    int launch_flags = 0;   // fused-kernel flags (FUSED_EARLY_NEXT of the plan, FUSED_ODD)
     int tile_rows = 0, tile_warps = 0;   // > 0: lbm_step runs the tile kernel in this shape
     float *d_aux = nullptr;      // two-pass scratch field
     // Results on the device, one allocation: diagnostic partials, the sums of both passes, the
@@ -332,6 +332,20 @@ bool even_pieces(const Plan &P) {
 // step without and 16.5 with.  So does a plan that leaves half the resident blocks' slots free.
 int plan_flags(const Plan &P, int resident) {
     return P.blocks * 2 <= resident || even_pieces(P) ? FUSED_EARLY_NEXT : 0;
+}
+
+// Whether an odd width takes the kernel that stages its side columns (FUSED_ODD).  That one costs a
+// few instructions more a pass and saves the blocks at the sides most of their single stores.
+// It loses where the lone last column has a warp (nearly) of its own, whose few stores are no
+// burden: last strips of 1 and 65 columns, FP32 us a step without and with it, 1025 x 1025 34.0 and
+// 38.9, 577 x 500 13.4 and 14.3; of 3, 1283 x 1000 44.0 and 47.6; but of 5, 645 x 500 18.9 and 18.0;
+// of 67, 451 x 900 23.3 and 22.0; of 127, 255 x 2000 20.3 and 19.3.  MRT with the Hermite source needs
+// a wide one: 15, 1551 x 300 28.4 and 28.9; 77, 333 x 777 20.7 and 20.4.
+bool stage_sides(int variant, int nx) {
+    if (nx % 2 == 0 || (variant & CV_OPEN)) return false;
+    const int w = (nx - 1) % FUSED_W + 1;
+    const bool hermite_source = (variant & (CV_MRT | CV_HERMITE)) == (CV_MRT | CV_HERMITE);
+    return w > FUSED_W / 2 ? w >= FUSED_W / 2 + 3 : w >= 5 && !hermite_source;
 }
 
 constexpr int MIN_PIECE = 8;   // default shortest row range worth a 4-row halo
@@ -913,7 +927,7 @@ lbm_status create_common(int nx, int ny, const lbm_params *p, void *buf, size_t 
         const Plan &P = r.plan;
         s->n_items = (int)P.items.size();
         s->n_blocks = P.blocks;
-        s->launch_flags = r.flags;
+        s->launch_flags = r.flags | (stage_sides(s->h.variant, nx) ? FUSED_ODD : 0);
         if (cudaMalloc(&s->d_items, P.items.size() * sizeof(WorkItem)) != cudaSuccess ||
             cudaMalloc(&s->d_off, P.off.size() * sizeof(int)) != cudaSuccess ||
             cudaMemcpy(s->d_items, P.items.data(), P.items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice) !=
@@ -1333,11 +1347,13 @@ lbm_status lbm_batch_create_ex(lbm_sim *const *sims, int n, const lbm_batch_opts
     for (int st = 0; st < 3; st++)
         for (int cv = 0; cv < N_VARIANTS; cv++) {
             std::vector<StripRef> strips;
-            long long nodes = 0;
-            bool periodic = true;
+            long long nodes = 0, staged = 0;
+            bool periodic = true, unstaged = false;
             for (int i = 0; i < n; i++)
                 if (sims[i]->p.storage == st && sims[i]->h.variant == cv) {
                     nodes += (long long)sims[i]->nx * sims[i]->ny;
+                    if (stage_sides(cv, sims[i]->nx)) staged += (long long)sims[i]->nx * sims[i]->ny;
+                    else unstaged = unstaged || sims[i]->nx % 2;
                     periodic = periodic && sims[i]->p.bc_x == LBM_BC_PERIODIC && sims[i]->p.bc_y == LBM_BC_PERIODIC;
                     strips_of(strips, i, sims[i]->nx, sims[i]->ny,
                               opts->member_plan_rows ? opts->member_plan_rows[i] : sims[i]->p.plan_rows);
@@ -1345,14 +1361,15 @@ lbm_status lbm_batch_create_ex(lbm_sim *const *sims, int n, const lbm_batch_opts
             if (strips.empty()) continue;
             PlanFor r = plan_for(strips, opts->plan, rows_per_item, st, cv, nodes, periodic, row_overhead);
             Plan &P = r.plan;
-            lbm_batch::Group g{st, cv, (int)items.size(), (int)offs.size(), P.blocks, r.flags};
+            lbm_batch::Group g{st, cv, (int)items.size(), (int)offs.size(), P.blocks,
+                               r.flags | (!unstaged && staged * 2 > nodes ? FUSED_ODD : 0)};
             for (int &o : P.off) o += g.item0;
             items.insert(items.end(), P.items.begin(), P.items.end());
             offs.insert(offs.end(), P.off.begin(), P.off.end());
             b->groups.push_back(g);
         }
     if (b->groups.size() > 1)   // concurrent launch groups: no early launch of the next step
-        for (auto &g : b->groups) g.flags = 0;
+        for (auto &g : b->groups) g.flags &= ~FUSED_EARLY_NEXT;
     b->n_items = (int)items.size();
     if (cudaMalloc(&b->d_descs, n * sizeof(SimDesc)) != cudaSuccess ||
         cudaMalloc(&b->d_items, items.size() * sizeof(WorkItem)) != cudaSuccess ||

@@ -138,6 +138,7 @@ constexpr int N_VARIANTS = 16;
 // Launch flag of the fused kernel: the next step may launch as soon as this one
 // starts (plans of equal pieces, one launch per step).
 constexpr int FUSED_EARLY_NEXT = 1;
+constexpr int FUSED_ODD = 2;   // (host) the kernel that stages the side columns of odd widths
 
 // One unit of work of a step launch: a strip of w <= W columns starting at x0,
 // marching over rows [ya, yb) of simulation `sim`.

@@ -14,22 +14,22 @@ namespace lbm {
 
 template <typename T, int CV>
 const void *fused_kernel_cv() {
-    return reinterpret_cast<const void *>(&k_step_fused<T, CV, FUSED_W, FUSED_NSLOT>);
+    return reinterpret_cast<const void *>(&k_step_fused<T, CV, FUSED_W, FUSED_NSLOT, !(CV & CV_OPEN)>);
 }
 
 template <typename T, int CV>
 int fused_smem_cv() {
-    return FusedCfg<T, CV, FUSED_W, FUSED_NSLOT>::SMEM;
+    return FusedCfg<T, CV, FUSED_W, FUSED_NSLOT, !(CV & CV_OPEN)>::SMEM;
 }
 
-template <typename T, int CV>
-cudaError_t fused_launch_cv(const SimDesc *descs, const WorkItem *items, const int *item_off, int n_blocks, int off,
-                            int flags, int *err, cudaStream_t st) {
-    constexpr int SMEM = FusedCfg<T, CV, FUSED_W, FUSED_NSLOT>::SMEM;
+template <typename T, int CV, bool ODD>
+cudaError_t fused_launch_odd(const SimDesc *descs, const WorkItem *items, const int *item_off, int n_blocks, int off,
+                             int flags, int *err, cudaStream_t st) {
+    constexpr int SMEM = FusedCfg<T, CV, FUSED_W, FUSED_NSLOT, ODD>::SMEM;
     static bool attr_done[64] = {false};
     int dev = 0;
     cudaGetDevice(&dev);
-    auto kernel = k_step_fused<T, CV, FUSED_W, FUSED_NSLOT>;
+    auto kernel = k_step_fused<T, CV, FUSED_W, FUSED_NSLOT, ODD>;
     if (dev < 64 && !attr_done[dev]) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
         if (e != cudaSuccess) return e;
@@ -48,6 +48,15 @@ cudaError_t fused_launch_cv(const SimDesc *descs, const WorkItem *items, const i
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, descs, items, item_off, n_blocks, off, flags, err);
+}
+
+template <typename T, int CV>
+cudaError_t fused_launch_cv(const SimDesc *descs, const WorkItem *items, const int *item_off, int n_blocks, int off,
+                            int flags, int *err, cudaStream_t st) {
+    constexpr bool PERIODIC = !(CV & CV_OPEN);
+    if (PERIODIC && (flags & FUSED_ODD))
+        return fused_launch_odd<T, CV, PERIODIC>(descs, items, item_off, n_blocks, off, flags, err, st);
+    return fused_launch_odd<T, CV, false>(descs, items, item_off, n_blocks, off, flags, err, st);
 }
 
 template <typename T, int CV>

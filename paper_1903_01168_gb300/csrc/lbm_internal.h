@@ -33,7 +33,8 @@ constexpr int FUSED_NSLOT = LBM_FUSED_NSLOT;
 // fused kernel is instantiated explicitly in its own translation unit group
 // (lbm_fused_*.cu: variants without and with wetting walls), and the two-pass
 // kernels of each T in lbm_twopass_*.cu, so that the units compile in parallel.
-// `flags`: FUSED_EARLY_NEXT lets the next step launch as soon as this one starts.
+// `flags`: FUSED_EARLY_NEXT lets the next step launch as soon as this one starts; FUSED_ODD
+// takes the kernel that stages the side columns of odd widths (periodic lattices of any width).
 template <typename T, int CV>
 cudaError_t fused_launch_cv(const SimDesc *descs, const WorkItem *items, const int *item_off, int n_blocks, int off,
                             int flags, int *err, cudaStream_t st);

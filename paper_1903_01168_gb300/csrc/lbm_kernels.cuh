@@ -119,7 +119,18 @@ __device__ __forceinline__ void s2i4(const V &v, float &gx, float &gy) {
 constexpr int OPEN_ROWS = 32;
 constexpr int OPEN_VALUES = 10;
 
-template <typename T, int CV, int W, int NSLOT>
+// Side columns of a row of an odd lattice, in shared memory between the pass that collides it
+// and the next one, which stores them: columns 0 .. 7 and, from the second place on,
+// nx - 8 .. nx - 1 (nx - 9 is even: pairs of columns start at even places), per plane.
+template <typename T>
+struct SideCols {
+    static constexpr int NS = ScalarPlanes<T>::value, PITCH = 10;
+    static constexpr int DEV_AT = NS * PITCH * 4;                             // bytes, of a side
+    static constexpr int BYTES = (DEV_AT + 16 * PITCH * (int)sizeof(T) + 15) / 16 * 16;
+    static constexpr int FLOATS = 2 * BYTES / 4;                              // of a row
+};
+
+template <typename T, int CV, int W, int NSLOT, bool ODD>
 struct FusedCfg {
     static constexpr int GMEM = 8;                           // ghost columns kept in memory
     static constexpr int G = 16 / (int)sizeof(T);            // halo columns loaded each side
@@ -140,7 +151,8 @@ struct FusedCfg {
     static constexpr int HIST_OFF = ((QY_OFF + (QRING ? 2 * RING : 0)) + 3) / 4 * 4;
     static constexpr int CONST_OFF = HIST_OFF + 2 * 4 * 32 * 4;
     static constexpr int OPEN_OFF = CONST_OFF + (int)sizeof(Consts<f2>) / 4;
-    static constexpr int RING_FLOATS = OPEN_OFF + ((CV & CV_OPEN) ? 4 * OPEN_ROWS * OPEN_VALUES : 0);
+    static constexpr int SIDE_OFF = ((CV & CV_OPEN) ? OPEN_OFF + 4 * OPEN_ROWS * OPEN_VALUES + 3 : OPEN_OFF + 3) / 4 * 4;
+    static constexpr int RING_FLOATS = SIDE_OFF + (ODD ? 2 * SideCols<T>::FLOATS : 0);
     static constexpr int DESC_BYTES = ((int)sizeof(SimDesc) + 127) / 128 * 128;
     static constexpr int RING_BYTES = ((RING_FLOATS * 4 + 15) / 16) * 16;
     static constexpr int SMEM = DESC_BYTES + NSLOT * SLOT_BYTES + RING_BYTES + NSLOT * 8 + 16;
@@ -356,10 +368,11 @@ __device__ __forceinline__ void close_node(const Consts<f2> &K, const HalfPulled
 
 // Post-collision state of the nodes (x, y) and, with `both`, (x + 1, y) of a lattice of
 // descriptor d, and its copies in the ghost columns of a periodic lattice.  out_rho,
-// out_dev: where planes 0 of node (x, y) are.
-template <typename T, bool SPLIT>
+// out_dev: where planes 0 of node (x, y) are.  STAGED: of an odd lattice the copies and a lone
+// last column go to `side` instead (SideCols).
+template <typename T, bool SPLIT, bool STAGED = false>
 __device__ __forceinline__ void store_pair(const SimDesc &d, bool per_x, int x, bool both, char *out_rho, char *out_dev, f2 rr, f2 rb,
-                                           const Collided<f2> &o) {
+                                           const Collided<f2> &o, unsigned char *side = nullptr) {
     constexpr int GMEM = 8;   // ghost columns (checked against the descriptor by the kernels)
     const uint32_t ps_rho = (uint32_t)d.rho_plane * 4u, ps_dev = (uint32_t)d.dev_plane * (uint32_t)sizeof(T);
     const long long nx = d.ph.nx;
@@ -384,6 +397,28 @@ __device__ __forceinline__ void store_pair(const SimDesc &d, bool per_x, int x, 
         // narrower than two ghosts)
         if (x < GMEM) store(out_rho + nx * 4, out_dev + nx * (long long)sizeof(T));
         if (x >= nx - GMEM) store(out_rho - nx * 4, out_dev - nx * (long long)sizeof(T));
+    } else if constexpr (STAGED) {
+        using Side = SideCols<T>;
+        if (x >= GMEM && x + 1 < nx - GMEM) return;
+#pragma unroll 1
+        for (int right = x < GMEM ? 0 : 1; right < 2; right++) {
+            if (right && x + 1 < nx - GMEM) break;
+            const int at = right ? x - ((int)nx - GMEM - 1) : x;
+            float *q = reinterpret_cast<float *>(side + right * Side::BYTES) + at;
+            T *v = reinterpret_cast<T *>(side + right * Side::BYTES + Side::DEV_AT) + at;
+            pair_to(q, rr);
+            pair_to(q + Side::PITCH, rb);
+            if (SPLIT) {
+                pair_to(q + 2 * Side::PITCH, o.m);
+                pair_to(q + 3 * Side::PITCH, o.gx);
+                pair_to(q + 4 * Side::PITCH, o.gy);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+                pair_to(v + i * Side::PITCH, o.r[i]);
+                pair_to(v + (i + 8) * Side::PITCH, o.b[i]);
+            }
+        }
     } else if (!both || (per_x && (x < GMEM || x + 1 >= nx - GMEM))) {
         // odd widths: single columns, in place (g = 0) or as ghost copies
         auto single = [&](int h, auto pick) {
@@ -519,17 +554,26 @@ struct EdgeLink {
 // scalar arithmetic and separate pulls of three rows (before): FP32 681, BF16 973; now FP32
 // 389, BF16 476.  Microseconds a step before and now: sweep BF16 107.6 and 63.1, FP32 78.9
 // and 78.3; eight open channels of mixed storage 293 and 173.
-template <typename T, int CV, int W, int NSLOT>
-__global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_step_fused(
+//
+// ODD: stages the side columns of odd widths.  The ghost copies of an odd lattice start at odd
+// columns, so that no pair is aligned; stored by the thread that has the values, 36 single ones
+// more a row, they make the blocks at the sides the last ones.  Here they go through shared
+// memory, and in the next pass all threads store a few values each, eight columns of a plane by
+// eight threads.  us a step without and with it: FP32 2001 x 2001 130 and 119, 40 of 255 x 256 92
+// and 80, FP16 2271 x 911 67.9 and 61.1.  A variant of its own (stage_sides says where), because
+// the test in every lattice's kernel cost even widths 1 to 2 % (1280 x 640 23.0 and 23.3).
+template <typename T, int CV, int W, int NSLOT, bool ODD>
+__global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT, ODD>::MINB)) k_step_fused(
     const SimDesc *__restrict__ descs, const WorkItem *__restrict__ items, const int *__restrict__ item_off,
     int n_blocks, int step_offset, int flags, int *__restrict__ err) {
-    using Cfg = FusedCfg<T, CV, W, NSLOT>;
+    using Cfg = FusedCfg<T, CV, W, NSLOT, ODD>;
     constexpr int G = Cfg::G, BOXW = Cfg::BOXW, RING = Cfg::RING, NT = W / 2;
     constexpr bool HERMITE = (CV & CV_HERMITE) != 0;
     constexpr bool HERMITE_SRC = Cfg::QRING;
     constexpr bool WET = Cfg::WET;
     constexpr bool OPEN = (CV & CV_OPEN) != 0;
     constexpr bool SPLIT = SplitStore<T>::value;
+    static_assert(!(ODD && OPEN), "open lattices have no ghost copies");
     extern __shared__ __align__(128) unsigned char smem[];
 
     const int tid = threadIdx.x;
@@ -539,6 +583,7 @@ __global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_st
     float *rings = reinterpret_cast<float *>(slots + NSLOT * Cfg::SLOT_BYTES);
     Consts<f2> &K = *reinterpret_cast<Consts<f2> *>(rings + Cfg::CONST_OFF);
     float *opens = rings + Cfg::OPEN_OFF;
+    unsigned char *sides = reinterpret_cast<unsigned char *>(rings + Cfg::SIDE_OFF);
     uint64_t *bars = reinterpret_cast<uint64_t *>(reinterpret_cast<unsigned char *>(rings) + Cfg::RING_BYTES);
 
     if (smem_u32(slots) & 127) {   // TMA destinations must be 128-byte aligned
@@ -653,6 +698,30 @@ __global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_st
         auto wall_terms = [&](const unsigned char *sp, int i, int j, int k, float sgn) {
             return wall_row_terms<T>(reinterpret_cast<const float *>(sp) + tc + G, BOXW,
                                      reinterpret_cast<const T *>(sp + Cfg::RHO_BYTES) + tc + G, BOXW, K, p.dphi[1], i, j, k, sgn);
+        };
+        // side columns of an odd lattice, collided in the pass before
+        const bool odd_sides = ODD && (p.nx & 1) && (x0 == 0 || x0 + w > p.nx - 8);
+        auto store_sides = [&](int y) {
+            using Side = SideCols<T>;
+            constexpr int PLANES = Side::NS + 16;
+            float *orho = d.rho + bdst * d.rho_buf + (long long)y * d.rho_row + d.ghost;
+            T *odev = reinterpret_cast<T *>(d.dev) + bdst * d.dev_buf + (long long)y * d.dev_row + d.ghost;
+            const unsigned char *row = sides + (y & 1) * Side::FLOATS * 4;
+            auto put = [&](int plane, int right, int from, int col) {
+                const unsigned char *s = row + right * Side::BYTES;
+                if (plane < Side::NS)
+                    orho[plane * d.rho_plane + col] = reinterpret_cast<const float *>(s)[plane * Side::PITCH + from];
+                else
+                    odev[(plane - Side::NS) * d.dev_plane + col] =
+                        reinterpret_cast<const T *>(s + Side::DEV_AT)[(plane - Side::NS) * Side::PITCH + from];
+            };
+            const int c = tid & 7;
+            if (x0 == 0)
+                for (int k = tid >> 3; k < PLANES; k += NT / 8) put(k, 0, c, p.nx + c);
+            const int col = p.nx - 8 + c;   // (a narrow last strip leaves some to the one before it)
+            if (col >= x0 && col < x0 + w)
+                for (int k = tid >> 3; k < PLANES; k += NT / 8) put(k, 1, c + 1, c - 8);
+            if (x0 + w == p.nx && tid < PLANES) put(tid, 1, 8, p.nx - 1);   // the lone last column itself
         };
         int slot = 0;
         uint32_t phase = 0;
@@ -875,6 +944,7 @@ __global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_st
                     phase ^= 1u;
                 }
             }
+            if (ODD && odd_sides && r - 3 >= ya) store_sides(r - 3);
             if (!closes) continue;
             if (wall_y && Y == 0 && ya == 0) {   // the wall below row 0
                 float *wall = rings + 2 * RING + 2;
@@ -921,7 +991,8 @@ __global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_st
                 }
                 Collided<f2> o;
                 collide_of<CV, SPLIT, f2>(p, K, Pc, cC, Fx, Fy, dQx, dQy, o);
-                store_pair<T, SPLIT>(d, !OPEN && p.bc_x == BC_PERIODIC, x, both, out_rho, out_dev, Pc.rr, Pc.rb, o);
+                store_pair<T, SPLIT, ODD>(d, !OPEN && p.bc_x == BC_PERIODIC, x, both, out_rho, out_dev, Pc.rr, Pc.rb, o,
+                                          sides + (r & 1) * SideCols<T>::FLOATS * 4);
                 out_rho += d.rho_row * 4;
                 out_dev += d.dev_row * (long long)sizeof(T);
             }
@@ -949,6 +1020,7 @@ __global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT>::MINB)) k_st
             __syncthreads();
             return;
         }
+        if (ODD && odd_sides) store_sides(yb - 1);
     }
     // this block's stores are issued: the next step may launch (it still waits
     // for this grid's completion before it reads anything); a block that
