@@ -329,8 +329,13 @@ bool even_pieces(const Plan &P) {
 // Launch flags for a plan run as the only launch of each step: a plan of even pieces lets
 // the next step launch early (its blocks then land on whichever SMs free first, which only
 // matters where the pieces differ): 1000 x 301 MRT, whose last strip is narrower, 19.8 us a
-// step without and 16.5 with.  So does a plan that leaves half the resident blocks' slots free.
+// step without and 16.5 with.  So does a plan that leaves half the resident blocks' slots free:
+// the waiting blocks fit there.  Between a half and two thirds of them they do not, and with
+// free slots on every SM some SMs start the next step with more blocks than others: 300 lattices
+// of 255 x 255 (600 blocks of 912) 609 us early and 523 without, 550 of 64 x 64 131 and 105, FP16
+// 143 and 113, open 512 x 256 13.9 and 12.7.
 int plan_flags(const Plan &P, int resident) {
+    if (P.blocks * 2 > resident && P.blocks * 3 <= resident * 2) return 0;
     return P.blocks * 2 <= resident || even_pieces(P) ? FUSED_EARLY_NEXT : 0;
 }
 
