@@ -563,10 +563,13 @@ int resident_blocks(int storage, int variant) {
 // except on FP32 lattices far beyond L2.  Those are held by DRAM, and 5 per SM load fewer halo
 // rows: 4096 x 512 FP32 62.3 -> 57.9 us a step, 8192 x 256 open 71.5 -> 66.8; at 1024 x 1024
 // (151 MB of state, mostly in L2) 6 per SM are faster (29.2 against 30.1), and FP16 storage is
-// at every size (2048 x 1280: 61.8 with 6 per SM, 69 with 5).
+// at every size (2048 x 1280: 61.8 with 6 per SM, 69 with 5).  So is MRT with the Hermite source,
+// whose passes have half as many instructions again: 2048 x 2048 148 with 5 and 125 with 6, 8192 x
+// 256 82.8 and 69.3, 2001 x 2001 177 and 152, 40 of 256 x 256 104 and 89.
 int plan_blocks(int storage, int variant, long long nodes) {
     const int all = resident_blocks(storage, variant);
-    return storage == ST_F32 && nodes >= 1500000 ? std::max(1, all * 5 / 6) : all;
+    const bool hermite_source = (variant & (CV_MRT | CV_HERMITE)) == (CV_MRT | CV_HERMITE);
+    return storage == ST_F32 && !hermite_source && nodes >= 1500000 ? std::max(1, all * 5 / 6) : all;
 }
 
 struct PlanFor {
