@@ -345,12 +345,20 @@ int plan_flags(const Plan &P, int resident) {
 // burden: last strips of 1 and 65 columns, FP32 us a step without and with it, 1025 x 1025 34.0 and
 // 38.9, 577 x 500 13.4 and 14.3; of 3, 1283 x 1000 44.0 and 47.6; but of 5, 645 x 500 18.9 and 18.0;
 // of 67, 451 x 900 23.3 and 22.0; of 127, 255 x 2000 20.3 and 19.3.  MRT with the Hermite source needs
-// a wide one: 15, 1551 x 300 28.4 and 28.9; 77, 333 x 777 20.7 and 20.4.
+// a wide one: 15, 1551 x 300 28.4 and 28.9; 77, 333 x 777 20.7 and 20.4.  Pieces of less than three
+// rows lose (tall_pieces): a row's side columns are stored a pass later, and there are few passes:
+// 1727 x 144 (2.2 rows) 13.5 and 14.3, 535 x 287 11.6 and 12.3; 3001 x 130 (3.4 rows) 19.6 and 19.0.
 bool stage_sides(int variant, int nx) {
     if (nx % 2 == 0 || (variant & CV_OPEN)) return false;
     const int w = (nx - 1) % FUSED_W + 1;
     const bool hermite_source = (variant & (CV_MRT | CV_HERMITE)) == (CV_MRT | CV_HERMITE);
     return w > FUSED_W / 2 ? w >= FUSED_W / 2 + 3 : w >= 5 && !hermite_source;
+}
+
+bool tall_pieces(const Plan &P) {
+    long long rows = 0;
+    for (const WorkItem &it : P.items) rows += it.yb - it.ya;
+    return rows >= 3 * (long long)P.items.size();
 }
 
 constexpr int MIN_PIECE = 8;   // default shortest row range worth a 4-row halo
@@ -935,7 +943,7 @@ lbm_status create_common(int nx, int ny, const lbm_params *p, void *buf, size_t 
         const Plan &P = r.plan;
         s->n_items = (int)P.items.size();
         s->n_blocks = P.blocks;
-        s->launch_flags = r.flags | (stage_sides(s->h.variant, nx) ? FUSED_ODD : 0);
+        s->launch_flags = r.flags | (stage_sides(s->h.variant, nx) && tall_pieces(P) ? FUSED_ODD : 0);
         if (cudaMalloc(&s->d_items, P.items.size() * sizeof(WorkItem)) != cudaSuccess ||
             cudaMalloc(&s->d_off, P.off.size() * sizeof(int)) != cudaSuccess ||
             cudaMemcpy(s->d_items, P.items.data(), P.items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice) !=
@@ -1370,7 +1378,7 @@ lbm_status lbm_batch_create_ex(lbm_sim *const *sims, int n, const lbm_batch_opts
             PlanFor r = plan_for(strips, opts->plan, rows_per_item, st, cv, nodes, periodic, row_overhead);
             Plan &P = r.plan;
             lbm_batch::Group g{st, cv, (int)items.size(), (int)offs.size(), P.blocks,
-                               r.flags | (!unstaged && staged * 2 > nodes ? FUSED_ODD : 0)};
+                               r.flags | (!unstaged && staged * 2 > nodes && tall_pieces(P) ? FUSED_ODD : 0)};
             for (int &o : P.off) o += g.item0;
             items.insert(items.end(), P.items.begin(), P.items.end());
             offs.insert(offs.end(), P.off.begin(), P.off.end());
