@@ -1198,14 +1198,19 @@ __global__ void __launch_bounds__(TILE_THREADS, TILE_MINB) k_step_tile(const Sim
         const int rs = (int)d.rho_plane, ds = (int)d.dev_plane;
         const unsigned lanes = 0xffffu << (tid & 16);
         const EdgeLink E(p, (tid & 7) + 1, (tid >> 3) & 1);
-        const int sides = (edge_l ? 1 : 0) + (link_r ? 1 : 0), edges = sides * (rows + 2) * (wall_y ? 2 : 1);
-        for (int e = (tid - own_warps * 32) >> 4; e < edges; e += (blockDim.x - own_warps * 32) >> 4) {
-            const int j = sides == 2 ? e >> 1 : e, side = sides == 2 ? e & 1 : (edge_l ? 0 : 1);
-            const int outer = j >= rows + 2, row = j - (outer ? rows + 2 : 0) - 1;
+        // (beside a lone column, two more: the column beyond it in the rows next to the walls)
+        const bool lone = LONE && link_r && !edge_r;
+        const int sides = (edge_l ? 1 : 0) + (edge_r ? 1 : 0), edges = sides * (rows + 2) * (wall_y ? 2 : 1);
+        for (int e = (tid - own_warps * 32) >> 4; e < edges + (lone ? 2 : 0); e += (blockDim.x - own_warps * 32) >> 4) {
+            const int j = sides == 2 ? e >> 1 : e;
+            int side = sides == 2 ? e & 1 : (edge_l ? 0 : 1), outer = j >= rows + 2, row = j - (outer ? rows + 2 : 0) - 1;
+            if (lone && e >= edges) {
+                side = 1, outer = 1, row = e == edges ? -y0 : ny - 1 - y0;
+                if (row < 0 || row >= rows) continue;
+            }
             int Y = y0 + row;
             if (wall_y && (Y < 0 || Y >= ny)) continue;
             if (outer && !(wall_y && (Y == 0 || Y == ny - 1))) continue;
-            if (LONE && !outer && side == 1 && !edge_r) continue;   // the lone column itself: a pair's
             Y = Y < 0 ? Y + ny : (Y >= ny ? Y - ny : Y);
             const int col = side == 0 ? -1 - outer : w + outer;
             const float *rp = d.rho + bsrc * d.rho_buf + d.ghost + x0 + col;
