@@ -46,8 +46,8 @@ FALLBACK_HBM_GBS = 6800.0
 # DRAM traffic of one k_step_fused launch on this workload from an ncu capture of
 # `dram__bytes_read.sum + dram__bytes_write.sum`, valid only for the kernel
 # sources with this hash; reported as null otherwise.
-NCU_TRAFFIC = {"sources_sha": "1b1a048e50d62a0e",
-               "bytes_per_launch": {0: 228982784 + 153013504, 1: 170608128 + 95448320}}
+NCU_TRAFFIC = {"sources_sha": "e9231c0fd8d18aa3",
+               "bytes_per_launch": {0: 228960512 + 153112064, 1: 170644992 + 96049152, 2: 170683648 + 96100864}}
 
 
 def kernel_sources_sha() -> str:

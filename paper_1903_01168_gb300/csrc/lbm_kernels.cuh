@@ -158,11 +158,13 @@ struct FusedCfg {
     static constexpr int SMEM = DESC_BYTES + NSLOT * SLOT_BYTES + RING_BYTES + NSLOT * 8 + 16;
     static constexpr uint32_t TX_BYTES = (uint32_t)(NS * BOXW * 4 + DEV_BYTES);
     // Blocks per SM the registers are sized for: 6 blocks of 2 warps are 3 warps on each
-    // scheduler, 168 registers a thread, which holds both columns' state without spills in
-    // the loop (spilled variants were 1.5-2x slower: their local memory misses the small L1
-    // that the shared-memory carve-out leaves).  Measured on the 40-lattice sweep with 4 and 6
-    // blocks: BF16 76.9 and 63.8 us a step, FP32 74.3 and 81.4 (the plans of large FP32
-    // lattices use 5, see plan_blocks).
+    // scheduler, 168 registers a thread (so are 5 blocks).  That holds both columns' state of
+    // periodic BGK and MRT lattices; other variants spill some (FP16 open BGK 84 bytes stored and
+    // 48 loaded, MRT with the Hermite source 28 to 220 stored) and are still faster than
+    // without spills at 4 blocks and up to 255 registers.  us a step of 2048 x 512 with 6 and with
+    // 4: FP32 BGK 27.6 and 30.7, FP16 27.9 and 31.6, open 39.8 and 41.7, MRT + Hermite 45.2 and 47.8,
+    // wet 47.1 and 50.9; only 16-bit open MRT + Hermite is a little slower (59.8 and 59.5).  How
+    // many of them a plan uses: plan_blocks, plan_for.
     static constexpr int MINB = LBM_FUSED_MIN_BLOCKS > 0 ? LBM_FUSED_MIN_BLOCKS : 6;
     static_assert(BOXW <= 256, "TMA box dimension limit");
     static_assert((BOXW * sizeof(T)) % 16 == 0 && (BOXW * 4) % 16 == 0, "TMA inner box bytes");
@@ -553,7 +555,7 @@ struct EdgeLink {
 // traffic).  Instructions issued per node of the 40-lattice sweep, one column a thread with
 // scalar arithmetic and separate pulls of three rows (before): FP32 681, BF16 973; now FP32
 // 389, BF16 476.  Microseconds a step before and now: sweep BF16 107.6 and 63.1, FP32 78.9
-// and 78.3; eight open channels of mixed storage 293 and 173.
+// and 76.5; eight open channels of mixed storage 293 and 173.
 //
 // ODD: stages the side columns of odd widths.  The ghost copies of an odd lattice start at odd
 // columns, so that no pair is aligned; stored by the thread that has the values, 36 single ones
@@ -615,8 +617,8 @@ __global__ void __launch_bounds__(W / 2, (FusedCfg<T, CV, W, NSLOT, ODD>::MINB))
     // writes are visible.  The descriptors' times are written between chunks of steps: the
     // first step of a chunk reads them again after the wait; a later one is launched by
     // blocks that have all waited for that write themselves.
-    // With FUSED_EARLY_NEXT (plans of equal pieces or with most of the chip idle, one launch
-    // per step) the next step may launch at once, its blocks waiting in free slots;
+    // With FUSED_EARLY_NEXT (plan_flags: plans of even pieces or with half the chip idle, one
+    // launch per step) the next step may launch at once, its blocks waiting in free slots;
     // otherwise only once this block's work is done (below): on uneven batches
     // and concurrent launch groups the early trigger placed waiting blocks on SMs
     // in the order slots freed and cost 5-16 %.
@@ -1477,7 +1479,7 @@ __global__ void k_fields(const SimDesc *__restrict__ dp, long long t, double *__
 // A block takes 32 columns, each warp every SLUG_WARPS-th row of them (neighbouring columns
 // in a warp); the warps' sums are added in a fixed order.  Bound by the latency of the
 // pulls, which a thread walking a whole column made one after another: diagnostics and
-// profile of a 2048 x 128 lattice together took 842 us, now 118 (profile 50).
+// profile of a 2048 x 128 lattice together took 842 us, now 119 (profile 50).
 constexpr int SLUG_WARPS = 16;
 template <typename T, bool HERMITE>
 __global__ void __launch_bounds__(32 * SLUG_WARPS) k_slug_profile(const SimDesc *__restrict__ dp, long long t,
